@@ -634,9 +634,8 @@ template <typename T>
 static int smooth_from_zero(mg_handle *H, int l, const LevelDev<T> &D, const T *b, T *out,
                             T *scratch, int sweeps, double omega, cudaStream_t s)
 {
-    if (coarse_solve_fits(D.nlon, D.nlat, sizeof(T))) {  // all sweeps in one launch
-        KRUN(K_SMOOTH0, l, prec_of<T>(),
-             launch_coarse_solve<T>(D, b, out, scratch, omega, sweeps, s));
+    if (coarse_solve_fits(D.nlon, D.nlat, D.nz, sizeof(T))) {  // all sweeps in one launch
+        KRUN(K_SMOOTH0, l, prec_of<T>(), launch_coarse_solve<T>(D, b, out, omega, sweeps, s));
         return MG_OK;
     }
     T *cur = (sweeps % 2 == 1) ? out : scratch;
@@ -875,6 +874,20 @@ static int bicg_precond(mg_handle *H, int slot, const T *in, T *out, cudaStream_
 {
     if (H->p.method == MG_METHOD_BICGSTAB) return vcycle_graph<T>(H, slot, in, out, s, nullptr);
     LevelHost &f = H->lev[0];
+    if constexpr (sizeof(T) == 8) {
+        // FP64 runs to the rounding floor of a line-relaxed Krylov method, whose
+        // attainable accuracy hangs on the preconditioner's roundings: the
+        // column walk, with the same roundings at every size
+        const LevelDev<T> D = dev<T>(f);
+        const int sweeps = H->p.line_sweeps;
+        T *cur = (sweeps % 2 == 1) ? out : Vec<T>::w(f), *oth = (cur == out) ? Vec<T>::w(f) : out;
+        for (int it = 0; it < sweeps; ++it) {
+            if (it > 0) std::swap(cur, oth);
+            KRUN(it ? K_SMOOTH : K_SMOOTH0, 0, 0,
+                 launch_smooth_walk<T>(D, in, it ? oth : nullptr, cur, H->p.omega, s));
+        }
+        return MG_OK;
+    }
     return smooth_from_zero<T>(H, 0, dev<T>(f), in, out, Vec<T>::w(f), H->p.line_sweeps,
                                H->p.omega, s);
 }

@@ -315,7 +315,9 @@ void build_items(StepHost<T> &st, int block, int nsys)
     int next = (int)st.items.size();
     for (int i : st.big) {
         const BOp<T> &op = st.ops[i];
-        const int grid = cdiv((long long)op.L.nlon * op.L.nlat, kBlock);
+        const int grid = st.kind == BK_SMOOTH_DOT
+                             ? smooth_dot_partials<T>(op.L, op.a, op.x, op.y)
+                             : cdiv((long long)op.L.nlon * op.L.nlat, kBlock);
         st.base.push_back(next);
         st.off[op.sys] = next;
         st.off[nsys + op.sys] = next + grid;

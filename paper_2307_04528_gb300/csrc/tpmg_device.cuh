@@ -648,51 +648,6 @@ __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], 
     }
 }
 
-template <typename T, bool ZERO, int CM = kWarpLayers>
-__device__ __forceinline__ void smooth_warp_column(const LevelDev<T> &L, const T *__restrict__ b,
-                                                   const T *uin, T *uout, T omega, int col,
-                                                   int lane)
-{
-    const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
-    const int j = col / nlon, i = col - j * nlon;
-    const int ie = (i + 1 == nlon) ? col - i : col + 1;
-    const int iw = (i == 0) ? col + nlon - 1 : col - 1;
-    const bool hasN = j + 1 < nlat, hasS = j > 0;
-    const size_t plane = (size_t)nlon * nlat;
-    const int C = (nz + 31) / 32;
-    const int k0 = lane * C;
-    T v[CM], tz[CM], m[CM], dq[CM], u0[CM];
-#pragma unroll
-    for (int c = 0; c < CM; ++c) {
-        const int k = k0 + c;
-        v[c] = tz[c] = m[c] = dq[c] = u0[c] = T(0);
-        if (c < C && k < nz) {
-            const size_t o = (size_t)k * plane;
-            T vv = __ldg(b + o + col);
-            if (!ZERO) {
-                vv = fma(__ldg(L.tx + o + col), uin[o + ie], vv);
-                vv = fma(__ldg(L.tx + o + iw), uin[o + iw], vv);
-                if (hasN) vv = fma(__ldg(L.ty + o + col), uin[o + col + nlon], vv);
-                if (hasS) vv = fma(__ldg(L.ty + o + col - nlon), uin[o + col - nlon], vv);
-                u0[c] = uin[o + col];
-            }
-            v[c] = vv;
-            tz[c] = __ldg(L.tz + o + col);
-            m[c] = __ldg(L.m + o + col);
-            dq[c] = __ldg(L.dq + o + col);
-        }
-    }
-    const T tprev = (k0 >= 1 && k0 - 1 < nz) ? __ldg(L.tz + (size_t)(k0 - 1) * plane + col) : T(0);
-    warp_column_scan<T, CM>(v, tz, m, dq, tprev, C, k0, nz, lane);
-    const T om1 = T(1) - omega;
-#pragma unroll
-    for (int c = 0; c < CM; ++c) {
-        const int k = k0 + c;
-        if (c < C && k < nz)
-            uout[(size_t)k * plane + col] = ZERO ? omega * v[c] : fma(om1, u0[c], omega * v[c]);
-    }
-}
-
 // The coarsest-level solve (sweeps of Eq. (1) from zero) by one block with
 // the whole level in shared memory: b, t_z, 1/p, q/p,
 // t_x, t_y and the two sweep vectors, each stored as [column][layer], so a

@@ -79,13 +79,30 @@ template <typename T>
 cudaError_t launch_smooth(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
                           double omega, cudaStream_t s, const int *flag = nullptr);
 
-// The coarsest-level solve: `sweeps` sweeps from a zero guess in one
-// one-block launch (result in out; scratch: a second level vector), for
-// coarsest levels where coarse_solve_fits(nlon, nlat, sizeof value).
-bool coarse_solve_fits(int nlon, int nlat, size_t value_bytes);
+// The same sweep as a column walk, whatever the level's size.
 template <typename T>
-cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, T *scratch, double omega,
-                                int sweeps, cudaStream_t s);
+cudaError_t launch_smooth_walk(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
+                               double omega, cudaStream_t s, const int *flag = nullptr);
+
+// The sweep with the column solve split over segments of layers
+// (tpmg_sweep.cu; u_in == nullptr: zero guess; partial != nullptr: the block
+// sums of <b, u_out>): the number of blocks, or -1 where the column walk of
+// launch_smooth is the faster form.
+template <typename T>
+int launch_sweep(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out, double omega,
+                 double *partial, cudaStream_t s, const int *flag);
+// Partial sums launch_smooth_dot writes for these arguments.
+template <typename T>
+int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out);
+// Shared-memory limits of the segmented sweeps (before any stream capture).
+cudaError_t sweep_prepare();
+
+// The coarsest-level solve: `sweeps` sweeps from a zero guess in one
+// one-block launch, for the coarsest levels that coarse_solve_fits.
+bool coarse_solve_fits(int nlon, int nlat, int nz, size_t value_bytes);
+template <typename T>
+cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
+                                cudaStream_t s);
 
 // The same sweep (non-zero guess) writing the block sums of <b, u_out> to
 // partial[block]; returns the number of blocks.

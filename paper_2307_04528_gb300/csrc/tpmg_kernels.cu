@@ -232,77 +232,13 @@ template <typename T>
 int launch_smooth_dot(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out, double omega,
                       double *partial, cudaStream_t s, const int *flag)
 {
+    const int blocks = launch_sweep<T>(L, b, u_in, u_out, omega, partial, s, flag);
+    if (blocks >= 0) return blocks;
     const size_t smem = kYOut<T> ? 0 : (size_t)L.nz * kBlock * sizeof(T);
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
     k_smooth_dot<T><<<grid, kBlock, smem, s>>>(L, b, u_in, u_out, (T)omega, partial, flag);
     return grid;
-}
-
-// One warp per column (smooth_warp_column), for levels small enough that
-// the serial column recurrences would dominate.
-template <typename T, bool ZERO, int CM>
-__global__ void __launch_bounds__(kBlock)
-k_smooth_warp(LevelDev<T> L, const T *__restrict__ b, const T *uin, T *uout, T omega,
-              const int *__restrict__ flag)
-{
-    if (flag && !*flag) return;
-    const int col = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    if (col >= L.nlon * L.nlat) return;  // whole warps
-    smooth_warp_column<T, ZERO, CM>(L, b, uin, uout, omega, col, threadIdx.x & 31);
-}
-
-// Layers per lane the warp sweeps are unrolled for (smooth_warp_column):
-// the smallest of 2, 3 and kWarpLayers that holds nz layers in 32 lanes.
-static inline int warp_layers_for(int nz) { return nz <= 64 ? 2 : nz <= 96 ? 3 : kWarpLayers; }
-
-// f.template operator()<CM>() for the CM of nz.
-template <typename F>
-static inline auto with_warp_layers(int nz, F &&f)
-{
-    switch (warp_layers_for(nz)) {
-    case 2: return f(std::integral_constant<int, 2>{});
-    case 3: return f(std::integral_constant<int, 3>{});
-    default: return f(std::integral_constant<int, kWarpLayers>{});
-    }
-}
-
-// The coarsest-level solve (Section 2.3's simple iteration: `sweeps`
-// block-Jacobi sweeps from a zero guess) as one block: the warps share the
-// columns, a block barrier separates the sweeps, and the sweeps alternate
-// between out and scratch so that the last one lands in out.
-
-template <typename T, int CM>
-__global__ void __launch_bounds__(kCoarseSolveThreads)
-k_coarse_solve(LevelDev<T> L, const T *__restrict__ b, T *out, T *scratch, T omega, int sweeps,
-               const int *__restrict__ flag)
-{
-    if (flag && !*flag) return;
-    const int ncol = L.nlon * L.nlat;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T *cur = (sweeps % 2 == 1) ? out : scratch;
-    T *oth = (cur == out) ? scratch : out;
-    for (int c = warp; c < ncol; c += nw)
-        smooth_warp_column<T, true, CM>(L, b, nullptr, cur, omega, c, lane);
-    for (int it = 1; it < sweeps; ++it) {
-        __syncthreads();  // the previous sweep is visible to the whole block
-        for (int c = warp; c < ncol; c += nw)
-            smooth_warp_column<T, false, CM>(L, b, cur, oth, omega, c, lane);
-        T *t = cur;
-        cur = oth;
-        oth = t;
-    }
-}
-
-// The same solve with the whole level in shared memory (coarse_solve_sh).
-template <typename T, int CM>
-__global__ void __launch_bounds__(kCoarseSolveThreads)
-k_coarse_solve_sh(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
-                  const int *__restrict__ flag)
-{
-    if (flag && !*flag) return;
-    extern __shared__ __align__(16) unsigned char sh_raw[];
-    coarse_solve_sh<T, CM>(L, b, out, omega, sweeps, reinterpret_cast<T *>(sh_raw));
 }
 
 // Opt-in shared memory per block (set by smooth_prepare).
@@ -318,60 +254,20 @@ bool coarse_sh_fits(int ncol, int nz, size_t value_bytes)
     return coarse_sh_bytes(ncol, nz, value_bytes) <= (size_t)g_smem_optin;
 }
 
-// FP32 levels with at most this many cells take the warp sweep (larger
-// ones do not fit L2, where the warp's strided column loads cost sectors).
-constexpr size_t kWarpSweepCells = (size_t)1 << 17;
-// Coarsest levels with at most this many columns take the one-block solve.
-constexpr int kCoarseSolveColumns = 2048;
-
-// FP32 only: the scans cost about twice the FP64 operations of the serial
-// sweep, and the FP64 sweeps are bound by FP64 arithmetic.
-bool coarse_solve_fits(int nlon, int nlat, size_t value_bytes)
-{
-    return value_bytes == 4 && nlon * nlat <= kCoarseSolveColumns;
-}
-
-template <typename T>
-cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, T *scratch, double omega,
-                                int sweeps, cudaStream_t s)
-{
-    const size_t sh = coarse_sh_bytes(L.nlon * L.nlat, L.nz, sizeof(T));
-    const bool in_sh = sweeps >= 1 && coarse_sh_fits(L.nlon * L.nlat, L.nz, sizeof(T));
-    with_warp_layers(L.nz, [&](auto cm) {
-        constexpr int CM = decltype(cm)::value;
-        if (in_sh)
-            k_coarse_solve_sh<T, CM><<<1, kCoarseSolveThreads, sh, s>>>(L, b, out, (T)omega,
-                                                                        sweeps, nullptr);
-        else
-            k_coarse_solve<T, CM><<<1, kCoarseSolveThreads, 0, s>>>(L, b, out, scratch,
-                                                                    (T)omega, sweeps, nullptr);
-        return 0;
-    });
-    return cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t launch_smooth(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out, double omega,
                           cudaStream_t s, const int *flag)
 {
+    if (launch_sweep<T>(L, b, u_in, u_out, omega, nullptr, s, flag) >= 0) return cudaGetLastError();
+    return launch_smooth_walk<T>(L, b, u_in, u_out, omega, s, flag);
+}
+
+template <typename T>
+cudaError_t launch_smooth_walk(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
+                               double omega, cudaStream_t s, const int *flag)
+{
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
-    if constexpr (sizeof(T) == 4) {
-        if ((size_t)ncol * L.nz <= kWarpSweepCells) {
-            const int wgrid = (int)(((size_t)ncol * 32 + kBlock - 1) / kBlock);
-            with_warp_layers(L.nz, [&](auto cm) {
-                constexpr int CM = decltype(cm)::value;
-                if (u_in == nullptr)
-                    k_smooth_warp<T, true, CM><<<wgrid, kBlock, 0, s>>>(L, b, nullptr, u_out,
-                                                                        (T)omega, flag);
-                else
-                    k_smooth_warp<T, false, CM><<<wgrid, kBlock, 0, s>>>(L, b, u_in, u_out,
-                                                                         (T)omega, flag);
-                return 0;
-            });
-            return cudaGetLastError();
-        }
-    }
     if (u_in == nullptr) {
         const size_t smem = ring_smem_bytes<T, true>(L.nz, kBlock);
         k_smooth0<T><<<grid, kBlock, smem, s>>>(L, b, u_out, (T)omega, flag);
@@ -409,16 +305,10 @@ cudaError_t smooth_prepare()
     if (lim > 0) g_smem_optin = lim;
     const void *kernels[] = {(const void *)k_smooth<double>,     (const void *)k_smooth<float>,
                              (const void *)k_smooth0<double>,    (const void *)k_smooth0<float>,
-                             (const void *)k_smooth_dot<double>, (const void *)k_smooth_dot<float>,
-                             (const void *)k_coarse_solve_sh<double, 2>,
-                             (const void *)k_coarse_solve_sh<double, 3>,
-                             (const void *)k_coarse_solve_sh<double, kWarpLayers>,
-                             (const void *)k_coarse_solve_sh<float, 2>,
-                             (const void *)k_coarse_solve_sh<float, 3>,
-                             (const void *)k_coarse_solve_sh<float, kWarpLayers>};
+                             (const void *)k_smooth_dot<double>, (const void *)k_smooth_dot<float>};
     for (const void *k : kernels)
         if ((e = set_dynamic_smem_limit(k, lim)) != cudaSuccess) return e;
-    return cudaSuccess;
+    return sweep_prepare();
 }
 
 // Largest dynamic shared memory one smoother block of kBlock columns needs
@@ -1068,6 +958,8 @@ cudaError_t launch_coeff_grad(int nlon, int nlat, int nz, const double *lam, con
                                    cudaStream_t, const int *);                                    \
     template cudaError_t launch_smooth<T>(const LevelDev<T> &, const T *, const T *, T *, double,  \
                                           cudaStream_t, const int *);                             \
+    template cudaError_t launch_smooth_walk<T>(const LevelDev<T> &, const T *, const T *, T *,     \
+                                               double, cudaStream_t, const int *);                \
     template int launch_smooth_dot<T>(const LevelDev<T> &, const T *, const T *, T *, double,      \
                                       double *, cudaStream_t, const int *);                       \
     template cudaError_t launch_resid_restrict<T>(const LevelDev<T> &, const LinkDev &, const T *, \
@@ -1085,8 +977,6 @@ cudaError_t launch_coeff_grad(int nlon, int nlat, int nz, const double *lam, con
     template cudaError_t launch_cg_direction<T>(const T *, const T *, T *, size_t,                \
                                                 const CgScalars *, bool, cudaStream_t);           \
     template cudaError_t launch_add<T>(T *, const T *, size_t, cudaStream_t);                    \
-    template cudaError_t launch_coarse_solve<T>(const LevelDev<T> &, const T *, T *, T *, double, \
-                                                int, cudaStream_t);                               \
     template int launch_dir_apply<T>(const LevelDev<T> &, const T *, const T *, const CgScalars *, \
                                      T *, T *, double *, cudaStream_t, const int *);            \
     template int dir_apply_partials<T>(const LevelDev<T> &, const T *, const T *, const T *,      \

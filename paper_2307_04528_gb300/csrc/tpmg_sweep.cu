@@ -1,0 +1,269 @@
+// Launchers of the segmented sweeps (tpmg_sweep.cuh) and of the one-block
+// coarsest-level solve, and the rules that pick a shape for a level.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+#include <type_traits>
+
+#include "tpmg_internal.h"
+#include "tpmg_sweep.cuh"
+
+namespace tpmg {
+namespace {
+
+// A block takes the tiles blockIdx, + gridDim, ...: one, unless a level has
+// more tiles than there are slots for partial sums.  (The loop also has the
+// compiler issue a tile's loads in one run: 0.534 ms against 0.698 without it
+// at 1536 x 1152 x 70, the same instructions otherwise.)
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+k_sweep(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
+        T omega, double *__restrict__ partial, const int *__restrict__ flag)
+{
+    if (flag && !*flag) return;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int tiles = (L.nlon * L.nlat + QL * CV - 1) / (QL * CV);
+    T acc = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        if (tile != (int)blockIdx.x) __syncthreads();  // the last tile's maps have been read
+        acc += sweep_tile<T, CV, LZ, QL, GUESS, DOT>(L, b, uin, uout, omega, tile,
+                                                     reinterpret_cast<T *>(smraw));
+    }
+    if (DOT) block_store<0>((double)acc, partial);
+}
+
+// A shape of the sweep: CV columns per thread, LZ layers per segment, QL
+// lanes along longitude, MAXT threads at most, MINB blocks per SM.
+template <int CV_, int LZ_, int QL_, int MAXT_, int MINB_, bool GUESS_ = true>
+struct Shape {
+    static constexpr int CV = CV_, LZ = LZ_, QL = QL_, MAXT = MAXT_, MINB = MINB_;
+    static constexpr bool GUESS = GUESS_;  // false: sweeps from zero only
+};
+
+// FP32 levels that fill the GPU.  From zero the sweep reads b, 1/p and q/p and
+// is bound by HBM: pairs of columns in 256-byte rows (1536 x 1152 x 70: 0.480
+// -> 0.274 ms, 7.2 TB/s; quads 0.290, single columns 0.316).  On a guess a
+// thread also reads five arrays around it, and instructions bind beside HBM:
+// quads of columns (16-byte loads), 64 columns to a block of 128 threads so
+// that two blocks share an SM (0.777 -> 0.534 ms, 6.5 TB/s; with <b, u_out>
+// 0.817 -> 0.627; one block of 256 threads 0.584 / 0.659, pairs 0.77 / 1.04).
+using Large0 = Shape<2, 9, 32, 256, 3, false>;
+using Large = Shape<4, 9, 16, 128, 2>;
+// the same with segments of 5 layers, for layer counts that leave fewer of
+// their slots empty (256 x 192 x 50: 10.7 -> 9.3 us; 352 x 226 x 37: 17.1 -> 12.2)
+using Large5 = Shape<4, 5, 16, 256, 2>;
+// rows that are no multiple of 2 columns (only from zero: 0.316 ms as above)
+using Odd0 = Shape<1, 9, 32, 256, 4, false>;
+// Levels of 2048 to 8192 columns in FP32: latency; 32 columns to a block
+// (48 x 82 x 70 on a guess: 13.5 -> 3.3 us, Large 3.6)
+using Mid = Shape<2, 5, 16, 256, 2>;
+// Small levels: 8 columns to a block, short segments (24 x 46 x 70 on a guess:
+// FP32 4.7 -> 3.0 us, Mid 3.2; 8 x 18 x 70 in FP64: 43 -> 6.2 us)
+using Small = Shape<1, 3, 8, 192, 1>;
+using SmallTall = Shape<1, 3, 8, 512, 1>;  // more than 72 layers
+// FP64 levels from 2^16 cells to 8192 columns, where the extra FP64 operations
+// of the exchanged maps begin to count: long segments (64 x 98 x 70 on a guess:
+// 43.8 -> 20.3 us, Small 26.2; 64 x 32 x 16: 9.6 -> 7.6, Small 4.1)
+using Mid64 = Shape<1, 9, 8, 192, 1>;
+
+template <typename T, typename S, bool GUESS, bool DOT>
+constexpr auto kernel_of()
+{
+    return k_sweep<T, S::CV, S::LZ, S::QL, GUESS, DOT, S::MAXT, S::MINB>;
+}
+
+template <typename S>
+int threads_of(int nz)  // whole warps: a segment past the last owns no layer
+{
+    return ((nz + S::LZ - 1) / S::LZ * S::QL + 31) / 32 * 32;
+}
+
+template <typename T, typename S, bool DOT>
+size_t smem_of(int threads)
+{
+    return (size_t)(3 + (DOT ? S::LZ : 0)) * threads * S::CV * sizeof(T);
+}
+
+template <typename T, typename S>
+bool suits(const LevelDev<T> &L, uintptr_t ptrs)
+{
+    return L.nlon % S::CV == 0 && threads_of<S>(L.nz) <= S::MAXT && ptrs % (S::CV * sizeof(T)) == 0;
+}
+
+// The arguments of one sweep; count: only its number of blocks is wanted.
+template <typename T>
+struct Sweep {
+    const T *b, *uin;
+    T *uout;
+    double omega;
+    double *partial;
+    cudaStream_t s;
+    const int *flag;
+    bool dot, count;
+};
+
+template <typename T, typename S>
+int go(const LevelDev<T> &L, const Sweep<T> &a)
+{
+    const long long per = S::QL * S::CV;
+    const long long tiles = ((long long)L.nlon * L.nlat + per - 1) / per;
+    const int grid = (int)std::min<long long>(tiles, kReduceSlots), threads = threads_of<S>(L.nz);
+    if (a.count) return grid;
+    const T *b = a.b, *uin = a.uin;
+    T *uout = a.uout;
+    double *partial = a.partial;
+    const double omega = a.omega;
+    const cudaStream_t s = a.s;
+    const int *flag = a.flag;
+    if (!uin)
+        kernel_of<T, S, false, false>()<<<grid, threads, smem_of<T, S, false>(threads), s>>>(
+            L, b, uin, uout, (T)omega, partial, flag);
+    if constexpr (S::GUESS) {
+        if (uin && partial)
+            kernel_of<T, S, true, true>()<<<grid, threads, smem_of<T, S, true>(threads), s>>>(
+                L, b, uin, uout, (T)omega, partial, flag);
+        else if (uin)
+            kernel_of<T, S, true, false>()<<<grid, threads, smem_of<T, S, false>(threads), s>>>(
+                L, b, uin, uout, (T)omega, partial, flag);
+    }
+    return grid;
+}
+
+// Slots left empty by segments of lz layers, in percent of the layers.
+int waste(int nz, int lz) { return ((nz + lz - 1) / lz * lz - nz) * 100 / nz; }
+
+constexpr int kSmallColumns = 2048, kMidColumns = 8192;
+
+template <typename T, typename S, bool DOT>
+cudaError_t allow_smem()
+{
+    const int need = (int)smem_of<T, S, DOT>(S::MAXT);
+    if (need <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute((const void *)kernel_of<T, S, true, DOT>(),
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, need);
+}
+
+template <typename T, int LZ>
+__global__ void __launch_bounds__(kCoarseSolveThreads, 1)
+k_coarse_sweeps(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    coarse_sweeps<T, LZ>(L, b, out, omega, sweeps, reinterpret_cast<T *>(smraw));
+}
+
+// The shape for a level and its buffers, or -1 where the column walk is the
+// faster form: FP64 levels beyond 8192 columns (the maps cost 16 FP64
+// operations per cell against 10, and the walk is bound by the FP64 pipe),
+// FP32 levels that fill the GPU with rows of no whole quad, and layer counts
+// beyond the shapes' registers.
+template <typename T>
+int pick(const LevelDev<T> &L, const Sweep<T> &a)
+{
+    const long long ncol = (long long)L.nlon * L.nlat;
+    if ((unsigned long long)ncol * L.nz * sizeof(T) >= 1ull << 32) return -1;  // 32-bit offsets
+    const uintptr_t ptrs = (uintptr_t)a.b | (uintptr_t)a.uin | (uintptr_t)a.uout |
+                           (uintptr_t)L.tx | (uintptr_t)L.ty | (uintptr_t)L.m | (uintptr_t)L.dq;
+    if constexpr (sizeof(T) == 8) {
+        if (ncol > kMidColumns) return -1;
+        if (ncol * L.nz >= 1 << 16 && suits<T, Mid64>(L, ptrs)) return go<T, Mid64>(L, a);
+    } else if (ncol < kMidColumns) {
+        if (ncol >= kSmallColumns && suits<T, Mid>(L, ptrs)) return go<T, Mid>(L, a);
+    } else {
+        if (waste(L.nz, 9) >= waste(L.nz, 5) + 8 && suits<T, Large5>(L, ptrs))
+            return go<T, Large5>(L, a);
+        if (a.uin || a.dot) return suits<T, Large>(L, ptrs) ? go<T, Large>(L, a) : -1;
+        if (suits<T, Large0>(L, ptrs)) return go<T, Large0>(L, a);
+        return suits<T, Odd0>(L, ptrs) ? go<T, Odd0>(L, a) : -1;
+    }
+    return suits<T, Small>(L, ptrs) ? go<T, Small>(L, a) : go<T, SmallTall>(L, a);
+}
+
+}  // namespace
+
+template <typename T>
+int launch_sweep(const LevelDev<T> &L, const T *b, const T *uin, T *uout, double omega,
+                 double *partial, cudaStream_t s, const int *flag)
+{
+    return pick<T>(L, {b, uin, uout, omega, partial, s, flag, partial != nullptr, false});
+}
+
+template <typename T>
+int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *uin, T *uout)
+{
+    const int n = pick<T>(L, {b, uin, uout, 0.0, nullptr, nullptr, nullptr, true, true});
+    return n >= 0 ? n : (L.nlon * L.nlat + kBlock - 1) / kBlock;
+}
+
+// The one-block coarsest-level solve: FP32 levels of at most 8192 cells and
+// 1024 columns (a sweep costs ~1.5 us where a launch per sweep costs ~3), FP64
+// levels of at most 512 cells (one SM retires 2 FP64 operations a clock, 17
+// per cell and sweep).
+bool coarse_solve_fits(int nlon, int nlat, int nz, size_t value_bytes)
+{
+    const long long ncol = (long long)nlon * nlat;
+    return ncol <= 1024 && ncol * nz <= (value_bytes == 4 ? 8192 : 512);
+}
+
+template <typename T>
+cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
+                                cudaStream_t s)
+{
+    const int ncol = L.nlon * L.nlat, n = ncol * L.nz;
+    auto run = [&](auto lz) {
+        constexpr int LZ = decltype(lz)::value;
+        const int threads = (ncol * ((L.nz + LZ - 1) / LZ) + 31) / 32 * 32;
+        const size_t smem = (4 * (size_t)n + 3 * (size_t)threads) * sizeof(T);
+        k_coarse_sweeps<T, LZ><<<1, threads, smem, s>>>(L, b, out, (T)omega, sweeps);
+        return cudaGetLastError();
+    };
+    auto holds = [&](int lz) { return ncol * ((L.nz + lz - 1) / lz) <= kCoarseSolveThreads; };
+    // the shortest segments whose threads one block holds (ncol nz <= 8192
+    // and ncol <= 1024 leave at most 16 layers per thread)
+    if constexpr (sizeof(T) == 8) {  // at most 512 cells
+        return run(std::integral_constant<int, 2>{});
+    } else {
+        if (holds(2)) return run(std::integral_constant<int, 2>{});
+        if (holds(4)) return run(std::integral_constant<int, 4>{});
+        if (holds(6)) return run(std::integral_constant<int, 6>{});
+        if (holds(8)) return run(std::integral_constant<int, 8>{});
+        if (holds(12)) return run(std::integral_constant<int, 12>{});
+        return run(std::integral_constant<int, 16>{});
+    }
+}
+
+cudaError_t sweep_prepare()
+{
+    cudaError_t e;
+    int dev = 0, lim = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
+        cudaSuccess)
+        return e;
+    for (cudaError_t q : {allow_smem<float, Large, true>(), allow_smem<float, Large5, true>(),
+                          allow_smem<float, Mid, true>(), allow_smem<float, SmallTall, true>(),
+                          allow_smem<double, Mid64, true>(), allow_smem<double, SmallTall, true>()})
+        if (q != cudaSuccess) return q;
+    const void *coarse[] = {
+        (const void *)k_coarse_sweeps<float, 2>, (const void *)k_coarse_sweeps<float, 4>,
+        (const void *)k_coarse_sweeps<float, 6>, (const void *)k_coarse_sweeps<float, 8>,
+        (const void *)k_coarse_sweeps<float, 12>,
+        (const void *)k_coarse_sweeps<float, 16>};
+    for (const void *k : coarse)
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      std::min(lim, 4 * 8192 * 4 + 3 * 1024 * 4))) != cudaSuccess)
+            return e;
+    return cudaSuccess;
+}
+
+#define TPMG_SWEEP_INST(T)                                                                       \
+    template int launch_sweep<T>(const LevelDev<T> &, const T *, const T *, T *, double, double *, \
+                                 cudaStream_t, const int *);                                     \
+    template int smooth_dot_partials<T>(const LevelDev<T> &, const T *, const T *, T *);           \
+    template cudaError_t launch_coarse_solve<T>(const LevelDev<T> &, const T *, T *, double, int, \
+                                                cudaStream_t);
+TPMG_SWEEP_INST(double)
+TPMG_SWEEP_INST(float)
+#undef TPMG_SWEEP_INST
+
+}  // namespace tpmg

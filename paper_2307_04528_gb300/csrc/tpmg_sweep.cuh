@@ -1,0 +1,416 @@
+// Block-Jacobi sweeps of Eq. (1) with the column solve split over segments
+// of layers.
+//
+// Both recurrences of the column solve are first-order and linear, so a
+// segment of layers acts on the value entering it as an affine map.  With
+// the setup factors m = 1/p and dq = q/p, p = q + t, the forward elimination
+//   y_k = (v_k + t_{k-1} y_{k-1}) m_k
+// is carried as h_k = t_k y_k = t_k m_k w_k = (1 - dq_k) w_k, w_k = v_k +
+// h_{k-1}, y_k = m_k w_k: t_z is not read at all (20 -> 16 bytes per cell
+// from a zero guess in FP32, 32 -> 28 on a guess), and w - dq w keeps the row
+// sums that the rounded factor t m would lose.  The backward substitution x_k
+// = x_{k+1} + (y_k - dq_k x_{k+1}) is as in the serial sweep (smooth_column);
+// the maps of both directions share the factor A = prod (1 - dq).
+//
+// A thread owns CV adjacent columns and LZ consecutive layers; QL lanes sit
+// side by side along longitude, so a warp covers QL CV columns of 32 / QL
+// segments and a block all segments of those columns.  Every load of the sweep
+// is independent of the recurrences: a thread issues them all at once, where
+// a thread walking a column keeps a few layers in flight, and the segments'
+// maps are then exchanged through shared memory, each thread combining the
+// maps below (above) its own to the value entering its segment before it
+// re-runs its layers with the serial formulas.  Each array is read once.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "tpmg_device.cuh"
+#include "tpmg_internal.h"
+
+namespace tpmg {
+
+// CV adjacent values of T, loaded and stored together.
+template <typename T, int CV>
+struct Vals {
+    T a[CV];
+};
+
+template <typename T, int CV>
+struct VecOf;
+template <>
+struct VecOf<float, 2> {
+    using type = float2;
+};
+template <>
+struct VecOf<float, 4> {
+    using type = float4;
+};
+template <>
+struct VecOf<double, 2> {
+    using type = double2;
+};
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> ldv(const T *__restrict__ p, unsigned byte)
+{
+    Vals<T, CV> r;
+    const char *q = reinterpret_cast<const char *>(p) + byte;
+    if constexpr (CV == 1) {
+        r.a[0] = __ldg(reinterpret_cast<const T *>(q));
+    } else {
+        using V = typename VecOf<T, CV>::type;
+        const V v = __ldg(reinterpret_cast<const V *>(q));
+        r.a[0] = v.x;
+        r.a[1] = v.y;
+        if constexpr (CV == 4) {
+            r.a[2] = v.z;
+            r.a[3] = v.w;
+        }
+    }
+    return r;
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ void stv(T *__restrict__ p, unsigned byte, const Vals<T, CV> &x)
+{
+    char *q = reinterpret_cast<char *>(p) + byte;
+    if constexpr (CV == 1) {
+        *reinterpret_cast<T *>(q) = x.a[0];
+    } else {
+        using V = typename VecOf<T, CV>::type;
+        V v;
+        v.x = x.a[0];
+        v.y = x.a[1];
+        if constexpr (CV == 4) {
+            v.z = x.a[2];
+            v.w = x.a[3];
+        }
+        *reinterpret_cast<V *>(q) = v;
+    }
+}
+
+// Element-wise arithmetic; two FP32 values per instruction (f32x2).
+__device__ __forceinline__ unsigned long long pk(float x, float y)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void upk(unsigned long long r, float &x, float &y)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r));
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> vfma(const Vals<T, CV> &x, const Vals<T, CV> &y,
+                                            const Vals<T, CV> &z)
+{
+    Vals<T, CV> r;
+    if constexpr (sizeof(T) == 4 && CV % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < CV; i += 2) {
+            unsigned long long d;
+            asm("fma.rn.f32x2 %0, %1, %2, %3;"
+                : "=l"(d)
+                : "l"(pk(x.a[i], x.a[i + 1])), "l"(pk(y.a[i], y.a[i + 1])),
+                  "l"(pk(z.a[i], z.a[i + 1])));
+            upk(d, r.a[i], r.a[i + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = fma(x.a[i], y.a[i], z.a[i]);
+    }
+    return r;
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> vadd(const Vals<T, CV> &x, const Vals<T, CV> &y)
+{
+    Vals<T, CV> r;
+    if constexpr (sizeof(T) == 4 && CV % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < CV; i += 2) {
+            unsigned long long d;
+            asm("add.rn.f32x2 %0, %1, %2;"
+                : "=l"(d)
+                : "l"(pk(x.a[i], x.a[i + 1])), "l"(pk(y.a[i], y.a[i + 1])));
+            upk(d, r.a[i], r.a[i + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = x.a[i] + y.a[i];
+    }
+    return r;
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> vmul(const Vals<T, CV> &x, const Vals<T, CV> &y)
+{
+    Vals<T, CV> r;
+    if constexpr (sizeof(T) == 4 && CV % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < CV; i += 2) {
+            unsigned long long d;
+            asm("mul.rn.f32x2 %0, %1, %2;"
+                : "=l"(d)
+                : "l"(pk(x.a[i], x.a[i + 1])), "l"(pk(y.a[i], y.a[i + 1])));
+            upk(d, r.a[i], r.a[i + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = x.a[i] * y.a[i];
+    }
+    return r;
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> splat(T x)
+{
+    Vals<T, CV> r;
+#pragma unroll
+    for (int i = 0; i < CV; ++i) r.a[i] = x;
+    return r;
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> vneg(const Vals<T, CV> &x)
+{
+    if constexpr (sizeof(T) == 4 && CV % 2 == 0) {  // two per instruction
+        return vmul<T, CV>(x, splat<T, CV>(T(-1)));
+    } else {
+        Vals<T, CV> r;
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = -x.a[i];
+        return r;
+    }
+}
+
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> lds_v(const T *p)
+{
+    Vals<T, CV> r;
+    if constexpr (CV == 1) {
+        r.a[0] = *p;
+    } else {
+        using V = typename VecOf<T, CV>::type;
+        const V v = *reinterpret_cast<const V *>(p);
+        r.a[0] = v.x;
+        r.a[1] = v.y;
+        if constexpr (CV == 4) {
+            r.a[2] = v.z;
+            r.a[3] = v.w;
+        }
+    }
+    return r;
+}
+
+// One tile of QL CV columns.  DOT: returns the thread's part of <b, u_out>,
+// b waiting for the last pass in the thread's own slots of shared memory.
+// Byte offsets are 32-bit (sweep_fits).  sh: 3 blockDim CV values, and LZ
+// blockDim CV more for DOT.
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT>
+__device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restrict__ b,
+                                        const T *__restrict__ uin, T *__restrict__ uout, T omega,
+                                        int tile, T *sh)
+{
+    using X = Vals<T, CV>;
+    constexpr unsigned SZ = sizeof(T);
+    const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
+    const int ncol = nlon * nlat;
+    const int q = threadIdx.x % QL, seg = threadIdx.x / QL, nseg = blockDim.x / QL;
+    const int own = (tile * QL + q) * CV;
+    const int col = own < ncol ? own : ncol - CV;  // past the end: read, not stored
+    const int k0 = seg * LZ;
+    const unsigned plane = (unsigned)ncol * SZ;
+    const unsigned first = (unsigned)col * SZ + (unsigned)min(k0, nz - 1) * plane;
+    const int row = blockDim.x * CV;  // values per slot row of shared memory
+    T *sb = sh + 3 * row + threadIdx.x * CV;
+
+    X v[LZ], m[LZ], dq[LZ], uc[GUESS ? LZ : 1];
+    // No load sits behind a branch: layers past the top re-read the last one.
+    unsigned off = first;
+#pragma unroll
+    for (int c = 0; c < LZ; ++c) {
+        m[c] = ldv<T, CV>(L.m, off);
+        dq[c] = ldv<T, CV>(L.dq, off);
+        v[c] = ldv<T, CV>(b, off);
+        if (GUESS) uc[c] = ldv<T, CV>(uin, off);
+        off += k0 + c + 1 < nz ? plane : 0u;
+    }
+    if (GUESS) {
+        const int j = col / nlon, i = col - j * nlon;
+        const bool hasN = j + 1 < nlat, hasS = j > 0;
+        // rows past a pole read the cell itself
+        const T *ue = uin + (i + CV == nlon ? -i : CV), *uw = uin + (i == 0 ? nlon - 1 : -1);
+        const T *un = uin + (hasN ? nlon : 0), *us = uin - (hasS ? nlon : 0);
+        const T *tw = L.tx + (i == 0 ? nlon - 1 : -1), *ts = L.ty - (hasS ? nlon : 0);
+        off = first;
+#pragma unroll
+        for (int c = 0; c < LZ; ++c) {
+            const X t = ldv<T, CV>(L.tx, off);
+            const X N = ldv<T, CV>(un, off), S = ldv<T, CV>(us, off);
+            const X tn = ldv<T, CV>(L.ty, off), tS = ldv<T, CV>(ts, off);
+            const T E = ldv<T, 1>(ue, off).a[0], W = ldv<T, 1>(uw, off).a[0];
+            const T tW = ldv<T, 1>(tw, off).a[0];
+            if (DOT) stv<T, CV>(sb + c * row, 0u, v[c]);
+#pragma unroll
+            for (int e = 0; e < CV; ++e) {
+                v[c].a[e] = fma(t.a[e], e + 1 < CV ? uc[c].a[e + 1 < CV ? e + 1 : e] : E, v[c].a[e]);
+                v[c].a[e] = fma(e > 0 ? t.a[e > 0 ? e - 1 : 0] : tW,
+                                e > 0 ? uc[c].a[e > 0 ? e - 1 : 0] : W, v[c].a[e]);
+            }
+            const X vn = vfma<T, CV>(tn, N, v[c]);
+            v[c] = hasN ? vn : v[c];
+            const X vs = vfma<T, CV>(tS, S, v[c]);
+            v[c] = hasS ? vs : v[c];
+            off += k0 + c + 1 < nz ? plane : 0u;
+        }
+    }
+    // layers past the top: 1/p = 0 makes their y and x zero; the sign of
+    // every use of q/p is taken here
+    const X zero = splat<T, CV>(T(0));
+#pragma unroll
+    for (int c = 0; c < LZ; ++c) {
+        m[c] = k0 + c < nz ? m[c] : zero;
+        dq[c] = vneg<T, CV>(dq[c]);
+    }
+
+    // forward: the segment's map h_out = A h_in + C
+    X A = splat<T, CV>(T(1)), C = zero;
+#pragma unroll
+    for (int c = 0; c < LZ; ++c) {
+        const X t = vadd<T, CV>(v[c], C);
+        C = vfma<T, CV>(dq[c], t, t);
+        A = vfma<T, CV>(dq[c], A, A);
+    }
+    T *sA = sh + q * CV, *sC = sA + row, *sF = sC + row;
+    stv<T, CV>(sA + seg * QL * CV, 0u, A);
+    stv<T, CV>(sC + seg * QL * CV, 0u, C);
+    __syncthreads();
+    X h = zero;
+    for (int s = 0; s < seg; ++s)
+        h = vfma<T, CV>(lds_v<T, CV>(sA + s * QL * CV), h, lds_v<T, CV>(sC + s * QL * CV));
+    // the segment's layers with the value entering it; v now holds y.  F:
+    // the backward map x_bottom = A x_above + F
+#pragma unroll
+    for (int c = 0; c < LZ; ++c) {
+        const X w = vadd<T, CV>(v[c], h);
+        h = vfma<T, CV>(dq[c], w, w);
+        v[c] = vmul<T, CV>(w, m[c]);
+    }
+    X F = zero;
+#pragma unroll
+    for (int c = LZ - 1; c >= 0; --c) F = vadd<T, CV>(F, vfma<T, CV>(dq[c], F, v[c]));
+    stv<T, CV>(sF + seg * QL * CV, 0u, F);
+    __syncthreads();
+    X x = zero;
+    for (int s = nseg - 1; s > seg; --s)
+        x = vfma<T, CV>(lds_v<T, CV>(sA + s * QL * CV), x, lds_v<T, CV>(sF + s * QL * CV));
+    const X om = splat<T, CV>(omega), om1 = splat<T, CV>(T(1) - omega);
+    T acc = 0;
+    off = first + (unsigned)(min(LZ, nz - k0) - 1) * plane;
+#pragma unroll
+    for (int c = LZ - 1; c >= 0; --c) {
+        x = vadd<T, CV>(x, vfma<T, CV>(dq[c], x, v[c]));
+        X uo = vmul<T, CV>(om, x);
+        if (GUESS) uo = vfma<T, CV>(om1, uc[c], uo);
+        if (k0 + c < nz) {
+            if (own < ncol) {
+                stv<T, CV>(uout, off, uo);
+                if (DOT) {
+                    const X bc = lds_v<T, CV>(sb + c * row);
+#pragma unroll
+                    for (int e = 0; e < CV; ++e) acc = fma(bc.a[e], uo.a[e], acc);
+                }
+            }
+            off -= plane;
+        }
+    }
+    return acc;
+}
+
+// The coarsest-level solve (`sweeps` sweeps from zero) by one block with u, b,
+// t_x and t_y of the level in shared memory, [layer][column] as in memory.
+// Thread (column, segment of LZ layers) keeps its factors in registers for
+// all sweeps; the forward and backward maps go through shared memory as in
+// sweep_tile, with A formed once.  The sweeps update u in place: every
+// coupling of a sweep is read before its first barrier, every value written
+// after its second.  sh: 4 n + 3 blockDim values.
+template <typename T, int LZ>
+__device__ __forceinline__ void coarse_sweeps(const LevelDev<T> &L, const T *__restrict__ b,
+                                              T *__restrict__ out, T omega, int sweeps, T *sh)
+{
+    const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
+    const int ncol = nlon * nlat, n = ncol * nz;
+    T *su = sh, *sb = sh + n, *stx = sh + 2 * n, *sty = sh + 3 * n;
+    T *sA = sh + 4 * n, *sC = sA + blockDim.x, *sF = sC + blockDim.x;
+    for (int g = threadIdx.x; g < n; g += blockDim.x) {
+        sb[g] = __ldg(b + g);
+        stx[g] = __ldg(L.tx + g);
+        sty[g] = __ldg(L.ty + g);
+    }
+    const int nseg = (nz + LZ - 1) / LZ;
+    const bool mine = threadIdx.x < ncol * nseg;
+    const int seg = mine ? threadIdx.x / ncol : 0, col = mine ? threadIdx.x - seg * ncol : 0;
+    const int k0 = seg * LZ;
+    const int j = col / nlon, i = col - j * nlon;
+    const int de = (i + 1 == nlon) ? -i : 1, dw = (i == 0) ? nlon - 1 : -1;
+    const bool hasN = j + 1 < nlat, hasS = j > 0;
+    T m[LZ], dq[LZ], A = 1;
+#pragma unroll
+    for (int c = 0; c < LZ; ++c) {
+        const int g = min(k0 + c, nz - 1) * ncol + col;
+        m[c] = k0 + c < nz ? __ldg(L.m + g) : T(0);
+        dq[c] = -__ldg(L.dq + g);
+        A = fma(dq[c], A, A);
+    }
+    sA[threadIdx.x] = A;
+    __syncthreads();
+    const T om1 = T(1) - omega;
+    for (int it = 0; it < sweeps; ++it) {
+        T v[LZ], C = 0;
+#pragma unroll
+        for (int c = 0; c < LZ; ++c) {
+            const int g = min(k0 + c, nz - 1) * ncol + col;
+            T x = sb[g];
+            if (it > 0) {
+                x = fma(stx[g], su[g + de], x);
+                x = fma(stx[g + dw], su[g + dw], x);
+                if (hasN) x = fma(sty[g], su[g + nlon], x);
+                if (hasS) x = fma(sty[g - nlon], su[g - nlon], x);
+            }
+            v[c] = x;
+            const T t = x + C;
+            C = fma(dq[c], t, t);
+        }
+        sC[threadIdx.x] = C;
+        __syncthreads();
+        T h = 0;
+        for (int s = 0; s < seg; ++s) h = fma(sA[s * ncol + col], h, sC[s * ncol + col]);
+#pragma unroll
+        for (int c = 0; c < LZ; ++c) {
+            const T w = v[c] + h;
+            h = fma(dq[c], w, w);
+            v[c] = w * m[c];
+        }
+        T F = 0;
+#pragma unroll
+        for (int c = LZ - 1; c >= 0; --c) F = F + fma(dq[c], F, v[c]);
+        sF[threadIdx.x] = F;
+        __syncthreads();
+        T x = 0;
+        for (int s = nseg - 1; s > seg; --s) x = fma(sA[s * ncol + col], x, sF[s * ncol + col]);
+#pragma unroll
+        for (int c = LZ - 1; c >= 0; --c) {
+            x = x + fma(dq[c], x, v[c]);
+            if (mine && k0 + c < nz) {
+                const int g = (k0 + c) * ncol + col;
+                su[g] = it > 0 ? fma(om1, su[g], omega * x) : omega * x;
+            }
+        }
+        __syncthreads();
+    }
+    for (int g = threadIdx.x; g < n; g += blockDim.x) out[g] = su[g];
+}
+
+}  // namespace tpmg
