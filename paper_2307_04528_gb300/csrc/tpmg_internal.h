@@ -76,6 +76,14 @@ int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgS
 //   u_out = (1 - omega) u_in + omega H_z^{-1} (b - dH u_in)
 // (u_in == nullptr: zero initial guess).
 template <typename T>
+// The FP64 stencil with a thread per 2 x 2 columns (tpmg_stencil.cu; the
+// values of launch_stencil): the number of blocks (and partial sums), or -1
+// for odd sizes or buffers not aligned to two values.
+int launch_stencil_quad(const LevelDev<double> &L, int mode, const double *b, const double *x,
+                        double *y, double *partial, cudaStream_t s, const int *flag);
+// Records the SM count.
+void stencil_prepare(int sms);
+
 cudaError_t launch_smooth(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
                           double omega, cudaStream_t s, const int *flag = nullptr);
 
@@ -235,6 +243,10 @@ int launch_residual_cast(const LevelDev<double> &L, const double *b, const doubl
 cudaError_t launch_cast_scaled(const double *r, float *r32, double inv_scale, size_t n,
                                cudaStream_t s);
 // x64 += scale * (double)e32
+// The same with a thread per 2 x 2 columns, or -1 as launch_stencil_quad.
+int launch_residual_cast_quad(const LevelDev<double> &L, const double *b, const double *x,
+                              float *r32, double inv_scale, bool narrow, double *partial,
+                              cudaStream_t s);
 cudaError_t launch_update_mixed(double *x, const float *e, double scale, size_t n,
                                 cudaStream_t s);
 
@@ -391,6 +403,9 @@ cudaError_t launch_ns_stencil(const NsView<T> &V, int mode, const T *b, const T 
 // after one sweep from zero, u = omega A_z^{-1} b).
 template <typename T>
 cudaError_t launch_ns_presmooth_resid(const NsView<T> &V, const T *b, const T *u, double omega,
+// The FP64 form with a thread per 2 x 2 columns, or -1 as launch_stencil_quad.
+int launch_ns_stencil_quad(const NsView<double> &V, int mode, const double *b, const double *x,
+                           double *y, cudaStream_t s);
                                       T *r, cudaStream_t s);
 // One sweep of Eq. (1), u_out = (1 - omega) u_in + omega A_z^{-1}(b - dA u_in)
 // (u_in == nullptr: zero guess).

@@ -126,6 +126,8 @@ int launch_residual_cast(const LevelDev<double> &L, const double *b, const doubl
     // significant entries are normal floats: |r| <= ||r|| < 2^10 / inv_scale
     // stays below 2^110, and entries down to 2^-56 ||r|| stay above 2^-126.
     const bool narrow = inv_scale >= 0x1p-100 && inv_scale <= 0x1p60;
+    const int blocks = launch_residual_cast_quad(L, b, x, r32, inv_scale, narrow, partial, s);
+    if (blocks >= 0) return blocks;
     if (narrow) k_resid_cast<true><<<grid, kBlock, 0, s>>>(L, b, x, r32, inv_scale, partial);
     else k_resid_cast<false><<<grid, kBlock, 0, s>>>(L, b, x, r32, inv_scale, partial);
     return grid;
@@ -149,6 +151,10 @@ template <typename T>
 int launch_stencil(const LevelDev<T> &L, int mode, const T *b, const T *x, T *y, double *partial,
                    cudaStream_t s, const int *flag)
 {
+    if constexpr (sizeof(T) == 8) {
+        const int blocks = launch_stencil_quad(L, mode, b, x, y, partial, s, flag);
+        if (blocks >= 0) return partial ? blocks : 0;
+    }
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (!partial && ncol < kCellParallelColumns) {
@@ -302,6 +308,7 @@ cudaError_t smooth_prepare()
         cudaSuccess)
         return e;
     if (sms > 0) g_sms = sms;
+    stencil_prepare(sms);
     if (lim > 0) g_smem_optin = lim;
     const void *kernels[] = {(const void *)k_smooth<double>,     (const void *)k_smooth<float>,
                              (const void *)k_smooth0<double>,    (const void *)k_smooth0<float>,

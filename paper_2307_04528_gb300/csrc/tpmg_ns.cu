@@ -444,6 +444,8 @@ template <typename T>
 cudaError_t launch_ns_stencil(const NsView<T> &V, int mode, const T *b, const T *x, T *y,
                               cudaStream_t s)
 {
+    if constexpr (sizeof(T) == 8)
+        if (launch_ns_stencil_quad(V, mode, b, x, y, s) >= 0) return cudaGetLastError();
     if (mode)
         k_ns_stencil<T, 1><<<col_blocks(V, kBlock), kBlock, 0, s>>>(V, b, x, y);
     else
