@@ -131,6 +131,9 @@ void coarsen_rows(const LevelShape &f, int nlon_c, double alpha_c, LevelShape &c
         }
         K.rptr[J + 1] = (int)K.rrow.size();
     }
+    K.w0f.assign(K.w0.begin(), K.w0.end());
+    K.w1f.assign(K.w1.begin(), K.w1.end());
+    K.rwf.assign(K.rw.begin(), K.rw.end());
     // coarse north-face distance ratio
     K.sy.assign(nc, 0.0);
     for (int J = 0; J + 1 < nc; ++J) {
@@ -279,11 +282,14 @@ static size_t carve(mg_handle *H, void *base)
             D.nlat_c = K.nlat_c;
             D.j0 = cv.take<int>(K.j0.size());
             D.w0 = cv.take<double>(K.w0.size());
+            D.w0f = cv.take<float>(K.w0f.size());
             D.j1 = cv.take<int>(K.j1.size());
             D.w1 = cv.take<double>(K.w1.size());
+            D.w1f = cv.take<float>(K.w1f.size());
             D.rptr = cv.take<int>(K.rptr.size());
             D.rrow = cv.take<int>(K.rrow.size());
             D.rw = cv.take<double>(K.rw.size());
+            D.rwf = cv.take<float>(K.rwf.size());
             D.cfirst = cv.take<int>(K.cfirst.size());
             D.ccnt = cv.take<int>(K.ccnt.size());
             D.sy = cv.take<double>(K.sy.size());
@@ -435,11 +441,14 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
             const LinkDev &D = v.linkdev;
             CHK(upload(K.j0, D.j0, s));
             CHK(upload(K.w0, D.w0, s));
+            CHK(upload(K.w0f, D.w0f, s));
             CHK(upload(K.j1, D.j1, s));
             CHK(upload(K.w1, D.w1, s));
+            CHK(upload(K.w1f, D.w1f, s));
             CHK(upload(K.rptr, D.rptr, s));
             CHK(upload(K.rrow, D.rrow, s));
             CHK(upload(K.rw, D.rw, s));
+            CHK(upload(K.rwf, D.rwf, s));
             CHK(upload(K.cfirst, D.cfirst, s));
             CHK(upload(K.ccnt, D.ccnt, s));
             CHK(upload(K.sy, D.sy, s));

@@ -915,6 +915,26 @@ __device__ __forceinline__ void smooth_staged(const LevelDev<T> &L, const T *__r
 }
 
 // ------------------------------------------------------------------ transfers
+// A link's weights in the precision of the transfer.
+template <typename T>
+__device__ __forceinline__ const T *near_weights(const LinkDev &K)
+{
+    if constexpr (sizeof(T) == 4) return K.w0f;
+    else return K.w0;
+}
+template <typename T>
+__device__ __forceinline__ const T *far_weights(const LinkDev &K)
+{
+    if constexpr (sizeof(T) == 4) return K.w1f;
+    else return K.w1;
+}
+template <typename T>
+__device__ __forceinline__ const T *row_weights(const LinkDev &K)
+{
+    if constexpr (sizeof(T) == 4) return K.rwf;
+    else return K.rw;
+}
+
 // Restriction R = P^T as a gather: coarse (I, J, k) sums, over the fine rows
 // listed for J with their latitude weights, the fine residuals at longitudes
 // 2I-1, 2I, 2I+1, 2I+2 (mod nlon) with weights 1/4, 3/4, 3/4, 1/4.
@@ -948,7 +968,7 @@ __device__ __forceinline__ void restrict_layers(const LevelDev<T> &F, const Link
 #pragma unroll
     for (int a = 0; a < kMaxRestrictRows; ++a) {
         off[a] = a < cnt ? __ldg(K.rrow + p0 + a) * nf : 0;
-        w[a] = a < cnt ? (T)__ldg(K.rw + p0 + a) : T(0);
+        w[a] = a < cnt ? __ldg(row_weights<T>(K) + p0 + a) : T(0);
     }
     const T q1 = T(0.25), q3 = T(0.75);
 #pragma unroll 1
@@ -985,8 +1005,8 @@ __device__ __forceinline__ void prolong_layers(const LevelDev<T> &F, const LinkD
     const int Ja = __ldg(K.j0 + j), Jb = __ldg(K.j1 + j);
     const size_t plane_c = (size_t)nc * K.nlat_c, plane_f = (size_t)nf * F.nlat;
     const T q1 = T(0.25), q3 = T(0.75);
-    const T wa = (T)__ldg(K.w0 + j);
-    const T wb = Jb >= 0 ? (T)__ldg(K.w1 + j) : T(0);
+    const T wa = __ldg(near_weights<T>(K) + j);
+    const T wb = Jb >= 0 ? __ldg(far_weights<T>(K) + j) : T(0);
     const size_t oa = (size_t)Ja * nc, ob = (size_t)(Jb >= 0 ? Jb : Ja) * nc;
     const size_t of = (size_t)j * nf + 2 * I;
 #pragma unroll 1
@@ -1172,14 +1192,14 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
         }
         const int J0 = __ldg(K.j0 + j), J1 = __ldg(K.j1 + j);
         if (J0 >= Jb && J0 < Je) {
-            const T w = (T)__ldg(K.w0 + j);
+            const T w = __ldg(near_weights<T>(K) + j);
             const int d = J0 - Jlo;
             if (d == 0) a0 = fma(w, sv, a0);
             else if (d == 1) a1 = fma(w, sv, a1);
             else a2 = fma(w, sv, a2);
         }
         if (J1 >= Jb && J1 < Je) {
-            const T w = (T)__ldg(K.w1 + j);
+            const T w = __ldg(far_weights<T>(K) + j);
             const int d = J1 - Jlo;
             if (d == 0) a0 = fma(w, sv, a0);
             else if (d == 1) a1 = fma(w, sv, a1);

@@ -29,6 +29,7 @@ struct LinkHost {
     int nlat_c = 0;
     std::vector<int> cfirst, ccnt, j0, j1, rptr, rrow;
     std::vector<double> w0, w1, rw, sy;
+    std::vector<float> w0f, w1f, rwf;  // their FP32 roundings
 };
 
 }  // namespace tpmg

@@ -31,6 +31,10 @@ struct LinkDev {
     const int *cfirst;          // [nlat_c] first fine row of coarse row J
     const int *ccnt;            // [nlat_c] 1 or 2 fine rows
     const double *sy;           // [nlat_c] coarse north-face distance ratio
+    // the FP32 roundings of w0, w1 and rw: a conversion in a kernel issues on
+    // the FP64 pipe, which the FP32 residual + restriction kept 45 % busy
+    // with its two conversions per row
+    const float *w0f, *w1f, *rwf;
 };
 
 // Device-side scalars of a conjugate-gradient iteration.

@@ -191,11 +191,14 @@ size_t ns_carve(mg_ns_handle *H, void *base)
             D.nlat_c = K.nlat_c;
             D.j0 = cv.take<int>(K.j0.size());
             D.w0 = cv.take<double>(K.w0.size());
+            D.w0f = cv.take<float>(K.w0f.size());
             D.j1 = cv.take<int>(K.j1.size());
             D.w1 = cv.take<double>(K.w1.size());
+            D.w1f = cv.take<float>(K.w1f.size());
             D.rptr = cv.take<int>(K.rptr.size());
             D.rrow = cv.take<int>(K.rrow.size());
             D.rw = cv.take<double>(K.rw.size());
+            D.rwf = cv.take<float>(K.rwf.size());
             D.cfirst = cv.take<int>(K.cfirst.size());
             D.ccnt = cv.take<int>(K.ccnt.size());
             D.sy = cv.take<double>(K.sy.size());
@@ -295,11 +298,14 @@ int ns_setup(mg_ns_handle *H, const mg_ns_coeffs *co, void *ws, size_t ws_bytes,
             const LinkDev &D = v.linkdev;
             CHK(upload(K.j0, D.j0, s));
             CHK(upload(K.w0, D.w0, s));
+            CHK(upload(K.w0f, D.w0f, s));
             CHK(upload(K.j1, D.j1, s));
             CHK(upload(K.w1, D.w1, s));
+            CHK(upload(K.w1f, D.w1f, s));
             CHK(upload(K.rptr, D.rptr, s));
             CHK(upload(K.rrow, D.rrow, s));
             CHK(upload(K.rw, D.rw, s));
+            CHK(upload(K.rwf, D.rwf, s));
             CHK(upload(K.cfirst, D.cfirst, s));
             CHK(upload(K.ccnt, D.ccnt, s));
             CHK(upload(K.sy, D.sy, s));
