@@ -76,10 +76,6 @@ template <typename T>
 int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgScalars *sc,
                      T *d_new, T *q, double *partial, cudaStream_t s, const int *flag = nullptr);
 
-// One smoother sweep of Eq. (1) in the arrangement
-//   u_out = (1 - omega) u_in + omega H_z^{-1} (b - dH u_in)
-// (u_in == nullptr: zero initial guess).
-template <typename T>
 // The FP64 stencil with a thread per 2 x 2 columns (tpmg_stencil.cu; the
 // values of launch_stencil): the number of blocks (and partial sums), or -1
 // for odd sizes or buffers not aligned to two values.
@@ -88,6 +84,10 @@ int launch_stencil_quad(const LevelDev<double> &L, int mode, const double *b, co
 // Records the SM count.
 void stencil_prepare(int sms);
 
+// One smoother sweep of Eq. (1) in the arrangement
+//   u_out = (1 - omega) u_in + omega H_z^{-1} (b - dH u_in)
+// (u_in == nullptr: zero initial guess).
+template <typename T>
 cudaError_t launch_smooth(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
                           double omega, cudaStream_t s, const int *flag = nullptr);
 
@@ -243,14 +243,14 @@ cudaError_t launch_hdiag(const LevelDev<double> &L, double *dh, cudaStream_t s);
 // partial sums.
 int launch_residual_cast(const LevelDev<double> &L, const double *b, const double *x, float *r32,
                          double inv_scale, double *partial, cudaStream_t s);
-// r32 = (float)(r64 * inv_scale)
-cudaError_t launch_cast_scaled(const double *r, float *r32, double inv_scale, size_t n,
-                               cudaStream_t s);
-// x64 += scale * (double)e32
 // The same with a thread per 2 x 2 columns, or -1 as launch_stencil_quad.
 int launch_residual_cast_quad(const LevelDev<double> &L, const double *b, const double *x,
                               float *r32, double inv_scale, bool narrow, double *partial,
                               cudaStream_t s);
+// r32 = (float)(r64 * inv_scale)
+cudaError_t launch_cast_scaled(const double *r, float *r32, double inv_scale, size_t n,
+                               cudaStream_t s);
+// x64 += scale * (double)e32
 cudaError_t launch_update_mixed(double *x, const float *e, double scale, size_t n,
                                 cudaStream_t s);
 
@@ -403,13 +403,13 @@ struct NsView {
 template <typename T>
 cudaError_t launch_ns_stencil(const NsView<T> &V, int mode, const T *b, const T *x, T *y,
                               cudaStream_t s);
+// The FP64 form with a thread per 2 x 2 columns, or -1 as launch_stencil_quad.
+int launch_ns_stencil_quad(const NsView<double> &V, int mode, const double *b, const double *x,
+                           double *y, cudaStream_t s);
 // r = (1 - omega) b plus the four horizontal couplings of u (the residual
 // after one sweep from zero, u = omega A_z^{-1} b).
 template <typename T>
 cudaError_t launch_ns_presmooth_resid(const NsView<T> &V, const T *b, const T *u, double omega,
-// The FP64 form with a thread per 2 x 2 columns, or -1 as launch_stencil_quad.
-int launch_ns_stencil_quad(const NsView<double> &V, int mode, const double *b, const double *x,
-                           double *y, cudaStream_t s);
                                       T *r, cudaStream_t s);
 // One sweep of Eq. (1), u_out = (1 - omega) u_in + omega A_z^{-1}(b - dA u_in)
 // (u_in == nullptr: zero guess).
