@@ -643,7 +643,7 @@ template <typename T>
 static int smooth_from_zero(mg_handle *H, int l, const LevelDev<T> &D, const T *b, T *out,
                             T *scratch, int sweeps, double omega, cudaStream_t s)
 {
-    if (coarse_solve_fits(D.nlon, D.nlat, D.nz, sizeof(T))) {  // all sweeps in one launch
+    if (coarse_solve_fits<T>(D.nlon, D.nlat, D.nz)) {  // all sweeps in one launch
         KRUN(K_SMOOTH0, l, prec_of<T>(), launch_coarse_solve<T>(D, b, out, omega, sweeps, s));
         return MG_OK;
     }

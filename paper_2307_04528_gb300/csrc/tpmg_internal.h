@@ -109,9 +109,10 @@ int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *u_in, T *u_ou
 // Shared-memory limits of the segmented sweeps (before any stream capture).
 cudaError_t sweep_prepare();
 
-// The coarsest-level solve: `sweeps` sweeps from a zero guess in one
-// one-block launch, for the coarsest levels that coarse_solve_fits.
-bool coarse_solve_fits(int nlon, int nlat, int nz, size_t value_bytes);
+// The coarsest-level solve: `sweeps` sweeps from a zero guess in one launch of
+// a thread-block cluster, for the levels that coarse_solve_fits.
+template <typename T>
+bool coarse_solve_fits(int nlon, int nlat, int nz);
 template <typename T>
 cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
                                 cudaStream_t s);

@@ -144,12 +144,49 @@ cudaError_t allow_smem()
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, need);
 }
 
+constexpr int kClusterBlocks = 8;  // the portable cluster size
+
+// Threads of a block of the coarsest-level solve: what its registers allow.
 template <typename T, int LZ>
-__global__ void __launch_bounds__(kCoarseSolveThreads, 1)
-k_coarse_sweeps(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps)
+constexpr int kClusterThreads = sizeof(T) == 4 ? 512 : LZ <= 4 ? 384 : 256;
+
+template <typename T, int LZ>
+__global__ void __launch_bounds__(kClusterThreads<T, LZ>, 1)
+k_coarse_cluster(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
+                 int R)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    coarse_sweeps<T, LZ>(L, b, out, omega, sweeps, reinterpret_cast<T *>(smraw));
+    coarse_cluster<T, LZ>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
+}
+
+// Layers per segment, balancing the dependent steps: about ten operations a
+// layer against two a segment, plus in FP32 (4 clocks an operation, FP64 ten
+// times that) the reads of the exchange.
+template <typename T>
+int cluster_lz(int nz)
+{
+    if (sizeof(T) == 8) return nz <= 24 ? 2 : nz <= 48 ? 3 : nz <= 96 ? 4 : 6;
+    return nz <= 16 ? 4 : nz <= 40 ? 6 : nz <= 72 ? 8 : 12;
+}
+
+struct ClusterShape {
+    int lz, R, blocks, threads;
+    size_t values;  // of shared memory
+};
+
+template <typename T>
+ClusterShape cluster_shape(int nlon, int nlat, int nz)
+{
+    ClusterShape c;
+    c.lz = cluster_lz<T>(nz);
+    // at least 128 cells to a block
+    const int blocks = (int)std::min<long long>(
+        kClusterBlocks, std::max<long long>((long long)nlon * nlat * nz / 128, 1));
+    c.R = (nlat + blocks - 1) / blocks;
+    c.blocks = (nlat + c.R - 1) / c.R;
+    c.threads = (c.R * nlon * ((nz + c.lz - 1) / c.lz) + 31) / 32 * 32;
+    c.values = 2 * (size_t)c.R * nlon * nz + 3 * (size_t)c.threads;
+    return c;
 }
 
 // The shape for a level and its buffers, or -1 where the column walk is the
@@ -195,63 +232,70 @@ int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *uin, T *uout)
     return n >= 0 ? n : (L.nlon * L.nlat + kBlock - 1) / kBlock;
 }
 
-// The one-block coarsest-level solve: FP32 levels of at most 8192 cells and
-// 1024 columns (a sweep costs ~1.5 us where a launch per sweep costs ~3), FP64
-// levels of at most 512 cells (one SM retires 2 FP64 operations a clock, 17
-// per cell and sweep).
-bool coarse_solve_fits(int nlon, int nlat, int nz, size_t value_bytes)
+// Levels whose rows fit eight blocks' threads take the cluster (up to 448
+// columns of 70 layers in FP32, 168 in FP64).  Per sweep, FP32: 1.35 us at 11
+// x 18 x 37 and 1.7 us at 6 x 14 x 70, against 4.5 and 4.1 us for one block
+// with the level's factors in registers and ~3 us for a launch per sweep.
+template <typename T>
+bool coarse_solve_fits(int nlon, int nlat, int nz)
 {
-    const long long ncol = (long long)nlon * nlat;
-    return ncol <= 1024 && ncol * nz <= (value_bytes == 4 ? 8192 : 512);
+    if (nlon > 512) return false;
+    const ClusterShape c = cluster_shape<T>(nlon, nlat, nz);
+    const int most = sizeof(T) == 4 ? kClusterThreads<float, 4>
+                     : c.lz <= 4    ? kClusterThreads<double, 4>
+                                    : kClusterThreads<double, 6>;
+    return c.threads <= most && c.values * sizeof(T) <= 160 * 1024;
 }
 
 template <typename T>
 cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
                                 cudaStream_t s)
 {
-    const int ncol = L.nlon * L.nlat, n = ncol * L.nz;
+    const ClusterShape c = cluster_shape<T>(L.nlon, L.nlat, L.nz);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c.blocks);
+    cfg.blockDim = dim3(c.threads);
+    cfg.dynamicSmemBytes = c.values * sizeof(T);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c.blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const T om = (T)omega;
     auto run = [&](auto lz) {
-        constexpr int LZ = decltype(lz)::value;
-        const int threads = (ncol * ((L.nz + LZ - 1) / LZ) + 31) / 32 * 32;
-        const size_t smem = (4 * (size_t)n + 3 * (size_t)threads) * sizeof(T);
-        k_coarse_sweeps<T, LZ><<<1, threads, smem, s>>>(L, b, out, (T)omega, sweeps);
-        return cudaGetLastError();
+        return cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, decltype(lz)::value>, L, b, out, om,
+                                  sweeps, c.R);
     };
-    auto holds = [&](int lz) { return ncol * ((L.nz + lz - 1) / lz) <= kCoarseSolveThreads; };
-    // the shortest segments whose threads one block holds (ncol nz <= 8192
-    // and ncol <= 1024 leave at most 16 layers per thread)
-    if constexpr (sizeof(T) == 8) {  // at most 512 cells
-        return run(std::integral_constant<int, 2>{});
+    if constexpr (sizeof(T) == 8) {
+        if (c.lz == 2) return run(std::integral_constant<int, 2>{});
+        if (c.lz == 3) return run(std::integral_constant<int, 3>{});
+        if (c.lz == 4) return run(std::integral_constant<int, 4>{});
+        return run(std::integral_constant<int, 6>{});
     } else {
-        if (holds(2)) return run(std::integral_constant<int, 2>{});
-        if (holds(4)) return run(std::integral_constant<int, 4>{});
-        if (holds(6)) return run(std::integral_constant<int, 6>{});
-        if (holds(8)) return run(std::integral_constant<int, 8>{});
-        if (holds(12)) return run(std::integral_constant<int, 12>{});
-        return run(std::integral_constant<int, 16>{});
+        if (c.lz == 4) return run(std::integral_constant<int, 4>{});
+        if (c.lz == 6) return run(std::integral_constant<int, 6>{});
+        if (c.lz == 8) return run(std::integral_constant<int, 8>{});
+        return run(std::integral_constant<int, 12>{});
     }
 }
 
 cudaError_t sweep_prepare()
 {
     cudaError_t e;
-    int dev = 0, lim = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
-        cudaSuccess)
-        return e;
     for (cudaError_t q : {allow_smem<float, Large, true>(), allow_smem<float, Large5, true>(),
                           allow_smem<float, Mid, true>(), allow_smem<float, SmallTall, true>(),
                           allow_smem<double, Mid64, true>(), allow_smem<double, SmallTall, true>()})
         if (q != cudaSuccess) return q;
     const void *coarse[] = {
-        (const void *)k_coarse_sweeps<float, 2>, (const void *)k_coarse_sweeps<float, 4>,
-        (const void *)k_coarse_sweeps<float, 6>, (const void *)k_coarse_sweeps<float, 8>,
-        (const void *)k_coarse_sweeps<float, 12>,
-        (const void *)k_coarse_sweeps<float, 16>};
+        (const void *)k_coarse_cluster<float, 4>,  (const void *)k_coarse_cluster<float, 6>,
+        (const void *)k_coarse_cluster<float, 8>,  (const void *)k_coarse_cluster<float, 12>,
+        (const void *)k_coarse_cluster<double, 2>, (const void *)k_coarse_cluster<double, 3>,
+        (const void *)k_coarse_cluster<double, 4>, (const void *)k_coarse_cluster<double, 6>};
     for (const void *k : coarse)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      std::min(lim, 4 * 8192 * 4 + 3 * 1024 * 4))) != cudaSuccess)
+                                      160 * 1024)) != cudaSuccess)
             return e;
     return cudaSuccess;
 }
@@ -260,6 +304,7 @@ cudaError_t sweep_prepare()
     template int launch_sweep<T>(const LevelDev<T> &, const T *, const T *, T *, double, double *, \
                                  cudaStream_t, const int *);                                     \
     template int smooth_dot_partials<T>(const LevelDev<T> &, const T *, const T *, T *);           \
+    template bool coarse_solve_fits<T>(int, int, int);                                             \
     template cudaError_t launch_coarse_solve<T>(const LevelDev<T> &, const T *, T *, double, int, \
                                                 cudaStream_t);
 TPMG_SWEEP_INST(double)

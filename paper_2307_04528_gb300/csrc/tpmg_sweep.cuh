@@ -22,6 +22,7 @@
 // re-runs its layers with the serial formulas.  Each array is read once.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "tpmg_device.cuh"
@@ -329,55 +330,68 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
     return acc;
 }
 
-// The coarsest-level solve (`sweeps` sweeps from zero) by one block with u, b,
-// t_x and t_y of the level in shared memory, [layer][column] as in memory.
-// Thread (column, segment of LZ layers) keeps its factors in registers for
-// all sweeps; the forward and backward maps go through shared memory as in
-// sweep_tile, with A formed once.  The sweeps update u in place: every
-// coupling of a sweep is read before its first barrier, every value written
-// after its second.  sh: 4 n + 3 blockDim values.
+// The coarsest-level solve (`sweeps` sweeps from zero) by one thread-block
+// cluster: block r owns the latitude rows [r R, r R + R), and a thread (column,
+// segment of LZ layers) of them keeps its factors, couplings and right-hand
+// side in registers for all sweeps.  u lives in the blocks' shared memory, two
+// copies written in turn; the rows beside a block's own are read from its
+// neighbours' shared memory, and one cluster barrier separates the sweeps.
+// The forward and backward maps of the segments are exchanged as in
+// sweep_tile, the factor A once.  sh: 2 R nlon nz + 3 blockDim values.
 template <typename T, int LZ>
-__device__ __forceinline__ void coarse_sweeps(const LevelDev<T> &L, const T *__restrict__ b,
-                                              T *__restrict__ out, T omega, int sweeps, T *sh)
+__device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__restrict__ b,
+                                               T *__restrict__ out, T omega, int sweeps, int R,
+                                               T *sh)
 {
-    const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
-    const int ncol = nlon * nlat, n = ncol * nz;
-    T *su = sh, *sb = sh + n, *stx = sh + 2 * n, *sty = sh + 3 * n;
-    T *sA = sh + 4 * n, *sC = sA + blockDim.x, *sF = sC + blockDim.x;
-    for (int g = threadIdx.x; g < n; g += blockDim.x) {
-        sb[g] = __ldg(b + g);
-        stx[g] = __ldg(L.tx + g);
-        sty[g] = __ldg(L.ty + g);
-    }
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int nlon = L.nlon, nlat = L.nlat, nz = L.nz, plane = nlon * nlat;
+    const int rank = (int)cl.block_rank(), j0 = rank * R;
+    const int rows = max(0, min(R, nlat - j0)), cols = rows * nlon, part = R * nlon;
+    T *u0 = sh, *u1 = sh + part * nz;
+    T *sA = sh + 2 * part * nz, *sC = sA + blockDim.x, *sF = sC + blockDim.x;
     const int nseg = (nz + LZ - 1) / LZ;
-    const bool mine = threadIdx.x < ncol * nseg;
-    const int seg = mine ? threadIdx.x / ncol : 0, col = mine ? threadIdx.x - seg * ncol : 0;
+    const bool mine = (int)threadIdx.x < cols * nseg;
+    const int seg = mine ? threadIdx.x / cols : 0, lc = mine ? threadIdx.x - seg * cols : 0;
     const int k0 = seg * LZ;
-    const int j = col / nlon, i = col - j * nlon;
+    const int r = lc / nlon, i = lc - r * nlon, j = min(j0 + r, nlat - 1);
     const int de = (i + 1 == nlon) ? -i : 1, dw = (i == 0) ? nlon - 1 : -1;
     const bool hasN = j + 1 < nlat, hasS = j > 0;
-    T m[LZ], dq[LZ], A = 1;
+    // the cells north and south of this column's first layer, in both copies
+    const T *n0 = u0 + lc, *s0 = u0 + lc;
+    if (hasN)
+        n0 = r + 1 < rows ? u0 + lc + nlon : cl.map_shared_rank(u0, rank + 1) + i;
+    if (hasS)
+        s0 = r > 0 ? u0 + lc - nlon : cl.map_shared_rank(u0, rank - 1) + (R - 1) * nlon + i;
+    T m[LZ], dq[LZ], bb[LZ], te[LZ], tw[LZ], tn[LZ], ts[LZ], uc[LZ], A = 1;
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
-        const int g = min(k0 + c, nz - 1) * ncol + col;
+        const int g = min(k0 + c, nz - 1) * plane + j * nlon + i;
+        bb[c] = __ldg(b + g);
+        te[c] = __ldg(L.tx + g);
+        tw[c] = __ldg(L.tx + g + dw);
+        tn[c] = hasN ? __ldg(L.ty + g) : T(0);
+        ts[c] = hasS ? __ldg(L.ty + g - nlon) : T(0);
         m[c] = k0 + c < nz ? __ldg(L.m + g) : T(0);
         dq[c] = -__ldg(L.dq + g);
+        uc[c] = 0;
         A = fma(dq[c], A, A);
     }
     sA[threadIdx.x] = A;
-    __syncthreads();
     const T om1 = T(1) - omega;
     for (int it = 0; it < sweeps; ++it) {
+        const int cur = (it & 1) * part * nz;  // the copy read; the other is written
+        T *nxt = (it & 1) ? u0 : u1;
         T v[LZ], C = 0;
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
-            const int g = min(k0 + c, nz - 1) * ncol + col;
-            T x = sb[g];
+            T x = bb[c];
             if (it > 0) {
-                x = fma(stx[g], su[g + de], x);
-                x = fma(stx[g + dw], su[g + dw], x);
-                if (hasN) x = fma(sty[g], su[g + nlon], x);
-                if (hasS) x = fma(sty[g - nlon], su[g - nlon], x);
+                const int o = cur + min(k0 + c, nz - 1) * part;
+                x = fma(te[c], u0[o + lc + de], x);
+                x = fma(tw[c], u0[o + lc + dw], x);
+                x = fma(tn[c], n0[o], x);
+                x = fma(ts[c], s0[o], x);
             }
             v[c] = x;
             const T t = x + C;
@@ -386,7 +400,8 @@ __device__ __forceinline__ void coarse_sweeps(const LevelDev<T> &L, const T *__r
         sC[threadIdx.x] = C;
         __syncthreads();
         T h = 0;
-        for (int s = 0; s < seg; ++s) h = fma(sA[s * ncol + col], h, sC[s * ncol + col]);
+#pragma unroll 4
+        for (int s = 0; s < seg; ++s) h = fma(sA[s * cols + lc], h, sC[s * cols + lc]);
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
             const T w = v[c] + h;
@@ -399,18 +414,21 @@ __device__ __forceinline__ void coarse_sweeps(const LevelDev<T> &L, const T *__r
         sF[threadIdx.x] = F;
         __syncthreads();
         T x = 0;
-        for (int s = nseg - 1; s > seg; --s) x = fma(sA[s * ncol + col], x, sF[s * ncol + col]);
+#pragma unroll 4
+        for (int s = nseg - 1; s > seg; --s) x = fma(sA[s * cols + lc], x, sF[s * cols + lc]);
 #pragma unroll
         for (int c = LZ - 1; c >= 0; --c) {
             x = x + fma(dq[c], x, v[c]);
+            uc[c] = fma(om1, uc[c], omega * x);
             if (mine && k0 + c < nz) {
-                const int g = (k0 + c) * ncol + col;
-                su[g] = it > 0 ? fma(om1, su[g], omega * x) : omega * x;
+                if (it + 1 < sweeps)
+                    nxt[(k0 + c) * part + lc] = uc[c];
+                else
+                    out[(k0 + c) * plane + j * nlon + i] = uc[c];
             }
         }
-        __syncthreads();
+        cl.sync();  // the sweep is complete, in every block, before the next reads it
     }
-    for (int g = threadIdx.x; g < n; g += blockDim.x) out[g] = su[g];
 }
 
 }  // namespace tpmg
