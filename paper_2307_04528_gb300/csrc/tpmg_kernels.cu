@@ -372,17 +372,18 @@ bool resid_restrict_fits(const void *b, const void *u, size_t value_bytes)
     return (uintptr_t)b % (2 * value_bytes) == 0 && (uintptr_t)u % (2 * value_bytes) == 0;
 }
 
-// Coarse rows per band of the fused residual + restriction: the widest
-// band (of kRRBand, 4, 2, 1; FP64, bound by the operations spent on band-edge
-// rows formed twice, from 2 kRRBand) whose warps still make two waves of 48
-// per SM.
+// Coarse rows per band of the fused residual + restriction: the widest band
+// (of kRRBand, 4, 2, 1) whose warps still make two waves of 48 per SM.  FP64,
+// bound by the operations spent on band-edge rows that are formed twice,
+// starts from 2 kRRBand and narrows only below 16 warps per SM (256 x 128 x
+// 32: bands of one row would form every fine row 2.4 times).
 template <typename T>
 int rr_band(const LevelDev<T> &F, const LinkDev &K)
 {
     const long long warps = (F.nlon / 2 + kRROwned - 1) / kRROwned;
+    const long long enough = (sizeof(T) == 8 ? 16LL : 2LL * 48) * g_sms;
     int band = sizeof(T) == 8 ? 2 * kRRBand : kRRBand;
-    while (band > 1 && warps * F.nz * ((K.nlat_c + band - 1) / band) < 2LL * 48 * g_sms)
-        band /= 2;
+    while (band > 1 && warps * F.nz * ((K.nlat_c + band - 1) / band) < enough) band /= 2;
     return band;
 }
 
