@@ -409,7 +409,6 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
         return fail(MG_ERR_WORKSPACE, "workspace %zu bytes < %zu needed", ws_bytes, need);
     carve(H, ws);
     CU(smooth_prepare());
-    CU(tma_prepare());
     {
         int dev = 0, lim = 0;
         CU(cudaGetDevice(&dev));
@@ -625,16 +624,6 @@ extern "C" int mg_profile_read(mg_handle *H, int kind, int level, int prec, int 
 extern "C" unsigned long long mg_launch_count(void) { return g_launches.load(); }
 
 static int level_check(mg_handle *H, int level, int prec, bool need_coarser);
-
-// A staged kernel that gave up waiting on its copies (tpmg_tma.cu) turns the
-// solve's status into MG_ERR_TIMEOUT.
-int tpmg::check_timeouts(int rc, cudaStream_t s)
-{
-    const int n = tma_timeouts(s, true);
-    if (n > 0) return fail(MG_ERR_TIMEOUT, "%d blocks gave up waiting on their copies", n);
-    if (n < 0) return fail(MG_ERR_CUDA, "reading the copy-timeout flag failed");
-    return rc;
-}
 
 // ------------------------------------------------------------------ V-cycle
 // Smoother sweeps from a zero guess, alternating between two buffers so that
@@ -1148,7 +1137,7 @@ extern "C" int mg_solve(mg_handle *H, const double *b, double *x, double tol, mg
     const int rc = solve_impl<double>(H, b, x, tol, H->p.maxit, H->p.method, &hist, &its, &rel,
                                       (cudaStream_t)stream, false, xmax == 0.0);
     fill_stats(st, hist, its, 0, rel);
-    return check_timeouts(rc, (cudaStream_t)stream);
+    return rc;
 }
 
 extern "C" int mg_solve_mixed(mg_handle *H, const double *b, double *x, double tol, mg_stats *st,
@@ -1240,7 +1229,7 @@ extern "C" int mg_solve_mixed(mg_handle *H, const double *b, double *x, double t
         ++outer;
     }
     fill_stats(st, hist, outer, inner, rel);
-    return check_timeouts(rc, s);
+    return rc;
 }
 
 extern "C" int mg_solve_single(mg_handle *H, const float *b, float *x, double tol, mg_stats *st,
@@ -1265,7 +1254,8 @@ extern "C" int mg_solve_single(mg_handle *H, const float *b, float *x, double to
     const int rc = solve_impl<float>(H, b, x, tol, H->p.maxit, H->p.method, &hist, &its, &rel, s);
     KRUN(K_VEC, 0, 1, launch_scale<float>(x, H->scale32, f.n, s));
     fill_stats(st, hist, its, 0, rel);
-    return check_timeouts(rc, s);
+    CU(cudaStreamSynchronize(s));
+    return rc;
 }
 
 // ------------------------------------------------------------------ C ABI: operators

@@ -62,7 +62,7 @@ int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgS
                      T *d_new, T *q, double *partial, cudaStream_t s, const int *flag)
 {
     if constexpr (sizeof(T) == 4) {
-        const int g = launch_dir_apply_tma(L, z, d_old, sc, d_new, q, partial, s, flag);
+        const int g = launch_dir_quad(L, z, d_old, sc, d_new, q, partial, s, flag);
         if (g >= 0) return g;
     }
     const int ncol = L.nlon * L.nlat;
@@ -309,6 +309,7 @@ cudaError_t smooth_prepare()
         return e;
     if (sms > 0) g_sms = sms;
     stencil_prepare(sms);
+    dir_prepare(sms);
     if (lim > 0) g_smem_optin = lim;
     const void *kernels[] = {(const void *)k_smooth<double>,     (const void *)k_smooth<float>,
                              (const void *)k_smooth0<double>,    (const void *)k_smooth0<float>,
@@ -536,7 +537,7 @@ int dir_apply_partials(const LevelDev<T> &L, const T *z, const T *d_old, const T
                        const T *q)
 {
     if constexpr (sizeof(T) == 4) {
-        const int g = dir_apply_tma_grid(L, z, d_old, d_new, q);
+        const int g = dir_quad_blocks(L, z, d_old, d_new, q);
         if (g >= 0) return g;
     }
     return (L.nlon * L.nlat + kBlock - 1) / kBlock;
