@@ -43,11 +43,15 @@ struct Loads {
 
 template <bool BZ>
 __global__ void __launch_bounds__(kBlock, 4)
-k_dir_quad(LevelDev<float> L, const float *__restrict__ z, const float *__restrict__ dold,
-           const CgScalars *__restrict__ sc, float *__restrict__ dnew, float *__restrict__ q,
-           int kz, double *__restrict__ partial, const int *__restrict__ flag)
+k_dir_quad(LevelDev<float> L, const float *__restrict__ z, const float *__restrict__ d_even,
+           const CgScalars *__restrict__ sc, float *__restrict__ d_to, float *__restrict__ q,
+           int kz, double *__restrict__ partial, const int *__restrict__ flag,
+           const CgLoop *__restrict__ loop)
 {
     if (flag && !*flag) return;
+    const bool odd = loop && (loop->its & 1);
+    const float *__restrict__ dold = loop && loop->its == 0 ? z : odd ? d_to : d_even;
+    float *__restrict__ dnew = odd ? const_cast<float *>(d_even) : d_to;
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz, nq = nlon / 4;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     float acc = 0.f;
@@ -169,17 +173,17 @@ int dir_quad_blocks(const LevelDev<float> &L, const float *z, const float *d_old
 
 int launch_dir_quad(const LevelDev<float> &L, const float *z, const float *d_old,
                     const CgScalars *sc, float *d_new, float *q, double *partial, cudaStream_t s,
-                    const int *flag)
+                    const int *flag, const CgLoop *loop)
 {
     const int blocks = dir_quad_blocks(L, z, d_old, d_new, q);
     if (blocks < 0) return -1;
     const Shape g = shape_of(L);
     if (d_old)
         k_dir_quad<false><<<dim3(g.gx, g.gy), kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, g.kz,
-                                                              partial, flag);
+                                                              partial, flag, loop);
     else
         k_dir_quad<true><<<dim3(g.gx, g.gy), kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, g.kz,
-                                                             partial, flag);
+                                                             partial, flag, loop);
     return blocks;
 }
 

@@ -114,6 +114,10 @@ struct mg_handle {
     // vector pair: 0 r -> z (conjugate gradients, stationary), 1 p -> ph and
     // 2 s -> sh (BiCGStab)
     VGraph vg[2][3];
+    // the conjugate-gradient loop of each precision (a conditional node whose
+    // body is one iteration), captured on first use
+    VGraph loop[2];
+    bool use_loops = true;
     mg_grid grid{};
     mg_params p{};
     int L = 0;
@@ -124,6 +128,7 @@ struct mg_handle {
     CgScalars *sc = nullptr;
     CgScalars *sc_coarse = nullptr;  // scalars of the PCG coarse solve
     BicgScalars *bsc = nullptr;      // scalars of BiCGStab
+    tpmg::CgLoop *cg_loop = nullptr; // state of the conjugate-gradient loop
     int *flag = nullptr;
     double scale32 = 0.0;
     double cheb_mu = 0.0;  // Chebyshev coarse solve: lower end of the spectrum of H_z^{-1} H

@@ -42,6 +42,18 @@ struct CgScalars {
     double rz, rz_new, dAd, rr, alpha, beta, maxabs, pad;
 };
 
+// State of a conjugate-gradient run whose iterations are a device-side loop
+// (a conditional graph node): set by the host, advanced by the loop's last
+// kernel.  Iteration `its` (0, 1, ...) writes its direction to d0 when even,
+// to d1 when odd; x is the caller's vector.
+constexpr int kLoopHist = 256;
+struct CgLoop {
+    double stop, grow;  // the loop ends at ||r|| <= stop or ||r||^2 > grow
+    int its, limit;     // iterations done, and where this launch ends
+    void *x;
+    double hist[kLoopHist];  // ||r||^2 of iteration i in hist[i % kLoopHist]
+};
+
 // Device-side scalars of a BiCGStab iteration (brk: a breakdown was met).
 struct BicgScalars {
     double rho, alpha, omega, beta, rv, ts, tt, rr, brk, pad;
@@ -71,10 +83,13 @@ int launch_stencil(const LevelDev<T> &L, int mode, const T *b, const T *x, T *y,
 
 // d_new = z + beta d_old (beta read from sc; d_old == nullptr: d_new = z) and
 // q = H d_new in one pass, with per-block partial sums of <d_new, q>; returns
-// the number of partial sums.
+// the number of partial sums.  loop: d_old and d_new are the directions of
+// its even iterations' predecessor and result (exchanged in the odd ones),
+// and z stands in for d_old in iteration 0 (beta = 0).
 template <typename T>
 int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgScalars *sc,
-                     T *d_new, T *q, double *partial, cudaStream_t s, const int *flag = nullptr);
+                     T *d_new, T *q, double *partial, cudaStream_t s, const int *flag = nullptr,
+                     const CgLoop *loop = nullptr);
 
 // The FP32 direction update + apply with a thread per four columns
 // (tpmg_dir.cu; the values of launch_dir_apply): the number of blocks (and
@@ -83,7 +98,7 @@ int dir_quad_blocks(const LevelDev<float> &L, const float *z, const float *d_old
                     const float *d_new, const float *q);
 int launch_dir_quad(const LevelDev<float> &L, const float *z, const float *d_old,
                     const CgScalars *sc, float *d_new, float *q, double *partial, cudaStream_t s,
-                    const int *flag);
+                    const int *flag, const CgLoop *loop);
 // Records the SM count.
 void dir_prepare(int sms);
 
@@ -181,12 +196,22 @@ int launch_maxabs(const T *a, size_t n, double *partial, cudaStream_t s);
 // x += alpha d; r -= alpha Ad; partial sum(r*r).  alpha from sc->alpha.
 template <typename T>
 int launch_cg_update(T *x, T *r, const T *d, const T *Ad, size_t n, const CgScalars *sc,
-                     double *partial, cudaStream_t s);
+                     double *partial, cudaStream_t s, const CgLoop *loop = nullptr,
+                     const T *d_odd = nullptr);
 
-// d_out = z + beta d_in (beta from sc->beta; beta_zero: d_out = z).
+// d_out = z + beta d_in (beta from sc->beta; beta_zero: d_out = z).  loop: d_in
+// is not read in its iteration 0 (z stands in for it, beta = 0).
 template <typename T>
 cudaError_t launch_cg_direction(const T *z, const T *d_in, T *d_out, size_t n,
-                                const CgScalars *sc, bool beta_zero, cudaStream_t s);
+                                const CgScalars *sc, bool beta_zero, cudaStream_t s,
+                                const CgLoop *loop = nullptr);
+
+// The reductions of a device-side conjugate-gradient loop: LOOP_RZ <r, z> and
+// beta (0 in iteration 0), LOOP_ALPHA <d, A d> and alpha, LOOP_CHECK ||r||^2,
+// its entry in hist, its + 1, and whether `cond` runs another iteration.
+enum { LOOP_RZ = 0, LOOP_ALPHA = 1, LOOP_CHECK = 2 };
+cudaError_t launch_loop_finalize(const double *partial, int n, CgScalars *sc, int op,
+                                 CgLoop *loop, cudaGraphConditionalHandle cond, cudaStream_t s);
 
 // Grid of the vector kernels for n elements (one wave of full occupancy).
 int vec_grid(size_t n);

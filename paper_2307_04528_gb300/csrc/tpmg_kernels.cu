@@ -46,11 +46,15 @@ k_stencil(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ x, T *__
 // scalars; BZ: first direction d_new = z), with the block sums of <d_new, q>.
 template <typename T, bool BZ>
 __global__ void __launch_bounds__(kBlock)
-k_dir_apply(LevelDev<T> L, const T *__restrict__ z, const T *__restrict__ dold,
-            const CgScalars *__restrict__ sc, T *__restrict__ dnew, T *__restrict__ q,
-            double *__restrict__ partial, const int *__restrict__ flag)
+k_dir_apply(LevelDev<T> L, const T *__restrict__ z, const T *__restrict__ d_even,
+            const CgScalars *__restrict__ sc, T *__restrict__ d_to, T *__restrict__ q,
+            double *__restrict__ partial, const int *__restrict__ flag,
+            const CgLoop *__restrict__ loop)
 {
     if (flag && !*flag) return;
+    const bool odd = loop && (loop->its & 1);
+    const T *__restrict__ dold = loop && loop->its == 0 ? z : odd ? d_to : d_even;
+    T *__restrict__ dnew = odd ? const_cast<T *>(d_even) : d_to;
     const T beta = BZ ? T(0) : (T)sc->beta;
     const T acc = dir_apply_column<T, BZ>(L, z, dold, beta, dnew, q,
                                           blockIdx.x * blockDim.x + threadIdx.x);
@@ -59,18 +63,21 @@ k_dir_apply(LevelDev<T> L, const T *__restrict__ z, const T *__restrict__ dold,
 
 template <typename T>
 int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgScalars *sc,
-                     T *d_new, T *q, double *partial, cudaStream_t s, const int *flag)
+                     T *d_new, T *q, double *partial, cudaStream_t s, const int *flag,
+                     const CgLoop *loop)
 {
     if constexpr (sizeof(T) == 4) {
-        const int g = launch_dir_quad(L, z, d_old, sc, d_new, q, partial, s, flag);
+        const int g = launch_dir_quad(L, z, d_old, sc, d_new, q, partial, s, flag, loop);
         if (g >= 0) return g;
     }
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (d_old == nullptr)
-        k_dir_apply<T, true><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag);
+        k_dir_apply<T, true><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
+                                                     loop);
     else
-        k_dir_apply<T, false><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag);
+        k_dir_apply<T, false><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
+                                                      loop);
     return grid;
 }
 
@@ -618,9 +625,12 @@ int launch_maxabs(const T *a, size_t n, double *partial, cudaStream_t s)
 
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_cg_update(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ d, const T *__restrict__ Ad,
-            size_t n, const CgScalars *sc, double *partial)
+k_cg_update(T *__restrict__ xv, T *__restrict__ r, const T *__restrict__ d_even,
+            const T *__restrict__ Ad, size_t n, const CgScalars *sc, double *partial,
+            const CgLoop *__restrict__ loop, const T *__restrict__ d_odd)
 {
+    T *__restrict__ x = loop ? static_cast<T *>(loop->x) : xv;
+    const T *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
     const T alpha = (T)sc->alpha;
     T acc = 0;
 #pragma unroll 4
@@ -635,10 +645,12 @@ k_cg_update(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ d, const
 }
 
 __global__ void __launch_bounds__(kBlock)
-k_cg_update_f4(float4 *__restrict__ x, float4 *__restrict__ r, const float4 *__restrict__ d,
-               const float4 *__restrict__ Ad, size_t n4, const CgScalars *sc,
-               double *partial)
+k_cg_update_f4(float4 *__restrict__ xv0, float4 *__restrict__ r, const float4 *__restrict__ d_even,
+               const float4 *__restrict__ Ad, size_t n4, const CgScalars *sc, double *partial,
+               const CgLoop *__restrict__ loop, const float4 *__restrict__ d_odd)
 {
+    float4 *__restrict__ x = loop ? static_cast<float4 *>(loop->x) : xv0;
+    const float4 *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
     const float alpha = (float)sc->alpha;
     float acc = 0.f;
 #pragma unroll 2
@@ -666,27 +678,28 @@ k_cg_update_f4(float4 *__restrict__ x, float4 *__restrict__ r, const float4 *__r
 
 template <typename T>
 int launch_cg_update(T *x, T *r, const T *d, const T *Ad, size_t n, const CgScalars *sc,
-                     double *partial, cudaStream_t s)
+                     double *partial, cudaStream_t s, const CgLoop *loop, const T *d_odd)
 {
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
-        if (vec4_ok(n, x, r, d, Ad)) {
+        if (vec4_ok(n, x, r, d, Ad) && vec4_ok(n, d_odd)) {
             k_cg_update_f4<<<g, kBlock, 0, s>>>(
                 reinterpret_cast<float4 *>(x), reinterpret_cast<float4 *>(r),
                 reinterpret_cast<const float4 *>(d), reinterpret_cast<const float4 *>(Ad), n / 4,
-                sc, partial);
+                sc, partial, loop, reinterpret_cast<const float4 *>(d_odd));
             return g;
         }
     }
-    k_cg_update<T><<<g, kBlock, 0, s>>>(x, r, d, Ad, n, sc, partial);
+    k_cg_update<T><<<g, kBlock, 0, s>>>(x, r, d, Ad, n, sc, partial, loop, d_odd);
     return g;
 }
 
 template <typename T, bool BZ>
 __global__ void __launch_bounds__(kBlock)
-k_cg_direction(const T *__restrict__ z, const T *__restrict__ din, T *__restrict__ dout, size_t n,
-               const CgScalars *sc)
+k_cg_direction(const T *__restrict__ z, const T *din, T *dout, size_t n, const CgScalars *sc,
+               const CgLoop *__restrict__ loop)
 {
+    if (loop && loop->its == 0) din = z;
     const T beta = BZ ? T(0) : (T)sc->beta;
 #pragma unroll 4
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
@@ -696,9 +709,10 @@ k_cg_direction(const T *__restrict__ z, const T *__restrict__ din, T *__restrict
 
 template <bool BZ>
 __global__ void __launch_bounds__(kBlock)
-k_cg_direction_f4(const float4 *__restrict__ z, const float4 *__restrict__ din,
-                  float4 *__restrict__ dout, size_t n4, const CgScalars *sc)
+k_cg_direction_f4(const float4 *__restrict__ z, const float4 *din, float4 *dout, size_t n4,
+                  const CgScalars *sc, const CgLoop *__restrict__ loop)
 {
+    if (loop && loop->its == 0) din = z;
     const float beta = BZ ? 0.f : (float)sc->beta;
 #pragma unroll 2
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n4;
@@ -716,7 +730,7 @@ k_cg_direction_f4(const float4 *__restrict__ z, const float4 *__restrict__ din,
 
 template <typename T>
 cudaError_t launch_cg_direction(const T *z, const T *d_in, T *d_out, size_t n, const CgScalars *sc,
-                                bool beta_zero, cudaStream_t s)
+                                bool beta_zero, cudaStream_t s, const CgLoop *loop)
 {
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
@@ -724,13 +738,13 @@ cudaError_t launch_cg_direction(const T *z, const T *d_in, T *d_out, size_t n, c
             const float4 *z4 = reinterpret_cast<const float4 *>(z);
             const float4 *di = reinterpret_cast<const float4 *>(d_in);
             float4 *dw = reinterpret_cast<float4 *>(d_out);
-            if (beta_zero) k_cg_direction_f4<true><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc);
-            else k_cg_direction_f4<false><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc);
+            if (beta_zero) k_cg_direction_f4<true><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
+            else k_cg_direction_f4<false><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
             return cudaGetLastError();
         }
     }
-    if (beta_zero) k_cg_direction<T, true><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc);
-    else k_cg_direction<T, false><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc);
+    if (beta_zero) k_cg_direction<T, true><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
+    else k_cg_direction<T, false><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
     return cudaGetLastError();
 }
 
@@ -857,6 +871,44 @@ cudaError_t launch_finalize(const double *partial, int n, CgScalars *sc, int whi
                             cudaStream_t s)
 {
     k_finalize<<<1, 1024, 0, s>>>(partial, n, sc, which, op);
+    return cudaGetLastError();
+}
+
+// Fixed-order sum of the partials and a step of a device-side loop (LOOP_*).
+__global__ void __launch_bounds__(1024)
+k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op, CgLoop *loop,
+                cudaGraphConditionalHandle cond)
+{
+    __shared__ double ws[32];
+    double v = 0;
+    for (int c = threadIdx.x; c < n; c += blockDim.x) v += partial[c];
+    v = warp_reduce<0>(v);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane == 0) ws[w] = v;
+    __syncthreads();
+    if (w != 0) return;
+    v = warp_reduce<0>(lane < (int)(blockDim.x >> 5) ? ws[lane] : 0.0);
+    if (lane != 0) return;
+    if (op == LOOP_RZ) {
+        sc->beta = loop->its > 0 && sc->rz != 0.0 ? v / sc->rz : 0.0;
+        sc->rz = v;
+    } else if (op == LOOP_ALPHA) {
+        sc->dAd = v;
+        sc->alpha = v != 0.0 ? sc->rz / v : 0.0;
+    } else {
+        sc->rr = v;
+        loop->hist[loop->its % kLoopHist] = v;
+        const int its = ++loop->its;
+        // a NaN compares false and ends the loop, as does an infinity
+        const bool more = sqrt(v) > loop->stop && v <= loop->grow && its < loop->limit;
+        cudaGraphSetConditional(cond, more ? 1u : 0u);
+    }
+}
+
+cudaError_t launch_loop_finalize(const double *partial, int n, CgScalars *sc, int op,
+                                 CgLoop *loop, cudaGraphConditionalHandle cond, cudaStream_t s)
+{
+    k_loop_finalize<<<1, 1024, 0, s>>>(partial, n, sc, op, loop, cond);
     return cudaGetLastError();
 }
 
@@ -1040,12 +1092,14 @@ cudaError_t launch_coeff_grad(int nlon, int nlat, int nz, const double *lam, con
     template int launch_dot<T>(const T *, const T *, size_t, double *, cudaStream_t);             \
     template int launch_maxabs<T>(const T *, size_t, double *, cudaStream_t);                     \
     template int launch_cg_update<T>(T *, T *, const T *, const T *, size_t, const CgScalars *,    \
-                                     double *, cudaStream_t);                                     \
+                                     double *, cudaStream_t, const CgLoop *, const T *);          \
     template cudaError_t launch_cg_direction<T>(const T *, const T *, T *, size_t,                \
-                                                const CgScalars *, bool, cudaStream_t);           \
+                                                const CgScalars *, bool, cudaStream_t,            \
+                                                const CgLoop *);                                  \
     template cudaError_t launch_add<T>(T *, const T *, size_t, cudaStream_t);                    \
     template int launch_dir_apply<T>(const LevelDev<T> &, const T *, const T *, const CgScalars *, \
-                                     T *, T *, double *, cudaStream_t, const int *);            \
+                                     T *, T *, double *, cudaStream_t, const int *,              \
+                                     const CgLoop *);                                            \
     template int dir_apply_partials<T>(const LevelDev<T> &, const T *, const T *, const T *,      \
                                        const T *);
 
