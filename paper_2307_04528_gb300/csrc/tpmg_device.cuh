@@ -1072,8 +1072,10 @@ __device__ __forceinline__ typename Pair<T>::type ld_pair(const T *p)
 // omega b cancels everything else; om1 = 1 - omega): the same walk without
 // h, t_z and the layers above and below, terms added east, west, north,
 // south.
-template <typename T, bool PRE = false>
-__device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const LinkDev &K,
+// Level: LevelDev, or (PRE) NsView, whose couplings from the west and the
+// south are arrays of their own.
+template <typename T, bool PRE = false, typename Level = LevelDev<T>>
+__device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDev &K,
                                                     const T *__restrict__ b,
                                                     const T *__restrict__ u, T *__restrict__ bc,
                                                     int warp, int lane, int Jb, int k,
@@ -1090,8 +1092,11 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
     const size_t plane = (size_t)nf * nlat, plane_c = (size_t)nc * ncJ;
     const size_t o = (size_t)k * plane + 2 * I;
     const bool up = k + 1 < nz, dn = k > 0;
-    const T *uk = u + o, *bk = b + o, *hk = F.h + o, *txk = F.tx + o, *tyk = F.ty + o;
-    const T *tzk = F.tz + o;
+    constexpr bool NS = kDirected<Level>;
+    static_assert(PRE || !NS, "the full residual is the symmetric level's");
+    const T *uk = u + o, *bk = b + o, *hk = mass_of(F) + o, *txk = east_of(F) + o;
+    const T *tyk = north_of(F) + o, *tzk = up_of(F) + o;
+    const T *wk = west_of(F) + o, *sk = south_of(F) + o;
     const T *uu = up ? uk + plane : uk, *ud = dn ? uk - plane : uk, *tzd = dn ? tzk - plane : tzk;
     T *out = bc + (size_t)k * plane_c + (owned ? Iown : 0);
     const int jfirst = __ldg(K.rrow + __ldg(K.rptr + Jb));
@@ -1103,31 +1108,39 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
     P2 zero;
     zero.x = zero.y = T(0);
     P2 Us = jfirst > 0 ? ld_pair(uk + (size_t)(jfirst - 1) * nf) : zero;
-    P2 Tys = jfirst > 0 ? ld_pair(tyk + (size_t)(jfirst - 1) * nf) : zero;
+    P2 Tys = jfirst > 0 ? ld_pair(sk + (size_t)(jfirst - 1) * nf) : zero;
     P2 Uc = ld_pair(uk + (size_t)jfirst * nf);
     // The FP32 PRE form has little arithmetic per row to cover its loads, so
     // it issues the next row's loads (u and t_y one row north, b and t_x on
     // the row) before combining this one: two rows in flight per thread.  The
     // full residual, and FP64 (ALU-bound), keep one row.
     constexpr bool kAhead = PRE && sizeof(T) == 4;
-    P2 nUn = zero, nB = zero, nTX = zero, nTYN = zero;
+    P2 nUn = zero, nB = zero, nTX = zero, nTYN = zero, nTW = zero, nTS = zero;
     if (kAhead) {
         const size_t o0 = (size_t)jfirst * nf;
         nUn = jfirst + 1 < nlat ? ld_pair(uk + o0 + nf) : zero;
         nB = ld_pair(bk + o0);
         nTX = ld_pair(txk + o0);
         nTYN = jfirst + 1 < nlat ? ld_pair(tyk + o0) : zero;
+        if (NS) {
+            nTW = ld_pair(wk + o0);
+            nTS = ld_pair(sk + o0);
+        }
     }
 #pragma unroll 1
     for (int j = jfirst; j <= jlast; ++j) {
         const bool hasN = j + 1 < nlat, hasS = j > 0;
         const size_t oj = (size_t)j * nf;
-        P2 Un, B, TX, TYN;
+        P2 Un, B, TX, TYN, TW, TS;
         if (kAhead) {
             Un = nUn;
             B = nB;
             TX = nTX;
             TYN = nTYN;
+            if (NS) {
+                TW = nTW;
+                TS = nTS;
+            }
             if (j < jlast) {
                 const size_t o1 = oj + nf;
                 const bool n1 = j + 2 < nlat;
@@ -1135,16 +1148,28 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
                 nB = ld_pair(bk + o1);
                 nTX = ld_pair(txk + o1);
                 nTYN = n1 ? ld_pair(tyk + o1) : zero;
+                if (NS) {
+                    nTW = ld_pair(wk + o1);
+                    nTS = ld_pair(sk + o1);
+                }
             }
         } else {
             Un = hasN ? ld_pair(uk + oj + nf) : zero;
             B = ld_pair(bk + oj);
             TX = ld_pair(txk + oj);
             TYN = hasN ? ld_pair(tyk + oj) : zero;
+            if (NS) {
+                TW = ld_pair(wk + oj);
+                TS = ld_pair(sk + oj);
+            }
+        }
+        if (!NS) {
+            TW = TX;
+            TS = TYN;
         }
         const T uw = __shfl_up_sync(kAll, Uc.y, 1);    // u[2I-1]
         const T ue = __shfl_down_sync(kAll, Uc.x, 1);  // u[2I+2]
-        const T txw = __shfl_up_sync(kAll, TX.y, 1);   // t_x[2I-1], west face of 2I
+        const T txw = __shfl_up_sync(kAll, TW.y, 1);   // t_x[2I-1], west face of 2I
         T r0, r1;
         if (PRE) {
             r0 = om1 * B.x;
@@ -1154,7 +1179,7 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
             if (hasS) r0 = fma(Tys.x, Us.x, r0);
             r1 = om1 * B.y;
             r1 = fma(TX.y, ue, r1);
-            r1 = fma(TX.x, Uc.x, r1);
+            r1 = fma(TW.x, Uc.x, r1);
             if (hasN) r1 = fma(TYN.y, Un.y, r1);
             if (hasS) r1 = fma(Tys.y, Us.y, r1);
         } else {
@@ -1207,7 +1232,7 @@ __device__ __forceinline__ void resid_restrict_band(const LevelDev<T> &F, const 
         }
         Us = Uc;
         Uc = Un;
-        Tys = TYN;
+        Tys = TS;
     }
     while (Jlo < Je) {
         if (owned) out[(size_t)Jlo * nc] = a0;

@@ -418,6 +418,60 @@ struct NsView {
     const T *m, *dq;
 };
 
+// The arrays of a level by the face they couple a cell across: a cell's own
+// coupling east / north, and its western / southern neighbour's row (the cell
+// one west, one south in the array), the same array in a symmetric level.
+template <typename T>
+__host__ __device__ inline const T *mass_of(const LevelDev<T> &L) { return L.h; }
+template <typename T>
+__host__ __device__ inline const T *mass_of(const NsView<T> &V) { return V.h; }
+template <typename T>
+__host__ __device__ inline const T *east_of(const LevelDev<T> &L) { return L.tx; }
+template <typename T>
+__host__ __device__ inline const T *east_of(const NsView<T> &V) { return V.e; }
+template <typename T>
+__host__ __device__ inline const T *west_of(const LevelDev<T> &L) { return L.tx; }
+template <typename T>
+__host__ __device__ inline const T *west_of(const NsView<T> &V) { return V.w; }
+template <typename T>
+__host__ __device__ inline const T *north_of(const LevelDev<T> &L) { return L.ty; }
+template <typename T>
+__host__ __device__ inline const T *north_of(const NsView<T> &V) { return V.n; }
+template <typename T>
+__host__ __device__ inline const T *south_of(const LevelDev<T> &L) { return L.ty; }
+template <typename T>
+__host__ __device__ inline const T *south_of(const NsView<T> &V) { return V.s; }
+template <typename T>
+__host__ __device__ inline const T *up_of(const LevelDev<T> &L) { return L.tz; }
+template <typename T>
+__host__ __device__ inline const T *up_of(const NsView<T> &V) { return V.u; }
+// the coupling of the row above down to the cell
+template <typename T>
+__host__ __device__ inline const T *down_of(const LevelDev<T> &L) { return L.tz; }
+template <typename T>
+__host__ __device__ inline const T *down_of(const NsView<T> &V) { return V.d; }
+template <typename V>
+constexpr bool kDirected = false;
+template <typename T>
+constexpr bool kDirected<NsView<T>> = true;
+
+// One sweep of Eq. (1) of a directed level by segments of layers (u_in ==
+// nullptr: from zero); -1 where the column walk is the faster form.
+template <typename T>
+int launch_ns_sweep(const NsView<T> &V, const T *b, const T *u_in, T *u_out, double omega,
+                    cudaStream_t s);
+// Coarsest-level solve on one thread-block cluster, where it fits.
+template <typename T>
+bool ns_coarse_fits(const NsView<T> &V);
+template <typename T>
+cudaError_t launch_ns_coarse(const NsView<T> &V, const T *b, T *out, double omega, int sweeps,
+                             cudaStream_t s);
+// The residual after one sweep from zero, restricted (b and u aligned to two
+// values: resid_restrict_fits).
+template <typename T>
+cudaError_t launch_ns_presmooth_restrict(const NsView<T> &V, const LinkDev &K, const T *b,
+                                         const T *u, T *bc, double omega, cudaStream_t s);
+
 // y = A x (mode 0) or b - A x (mode 1) in the directed flux form.
 template <typename T>
 cudaError_t launch_ns_stencil(const NsView<T> &V, int mode, const T *b, const T *x, T *y,

@@ -375,6 +375,18 @@ k_resid_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ b, const T *__r
                                 (band0 + (int)blockIdx.z) * band, blockIdx.y, om1, band);
 }
 
+// The same over a directed level (two more arrays, two more pairs in flight).
+template <typename T>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 8 : 0)
+k_ns_presmooth_restrict(NsView<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
+                        T *__restrict__ bc, T om1, int band0, int band)
+{
+    const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+    if (warp * kRROwned >= F.nlon / 2) return;  // whole warps
+    resid_restrict_band<T, true>(F, K, b, u, bc, warp, threadIdx.x & 31,
+                                 (band0 + (int)blockIdx.z) * band, blockIdx.y, om1, band);
+}
+
 bool resid_restrict_fits(const void *b, const void *u, size_t value_bytes)
 {
     return (uintptr_t)b % (2 * value_bytes) == 0 && (uintptr_t)u % (2 * value_bytes) == 0;
@@ -386,13 +398,33 @@ bool resid_restrict_fits(const void *b, const void *u, size_t value_bytes)
 // starts from 2 kRRBand and narrows only below 16 warps per SM (256 x 128 x
 // 32: bands of one row would form every fine row 2.4 times).
 template <typename T>
-int rr_band(const LevelDev<T> &F, const LinkDev &K)
+static int rr_band(int nlon, int nz, const LinkDev &K)
 {
-    const long long warps = (F.nlon / 2 + kRROwned - 1) / kRROwned;
+    const long long warps = (nlon / 2 + kRROwned - 1) / kRROwned;
     const long long enough = (sizeof(T) == 8 ? 16LL : 2LL * 48) * g_sms;
     int band = sizeof(T) == 8 ? 2 * kRRBand : kRRBand;
-    while (band > 1 && warps * F.nz * ((K.nlat_c + band - 1) / band) < enough) band /= 2;
+    while (band > 1 && warps * nz * ((K.nlat_c + band - 1) / band) < enough) band /= 2;
     return band;
+}
+
+template <typename T>
+int rr_band(const LevelDev<T> &F, const LinkDev &K)
+{
+    return rr_band<T>(F.nlon, F.nz, K);
+}
+
+template <typename T>
+cudaError_t launch_ns_presmooth_restrict(const NsView<T> &F, const LinkDev &K, const T *b,
+                                         const T *u, T *bc, double omega, cudaStream_t s)
+{
+    const int warps = (F.nlon / 2 + kRROwned - 1) / kRROwned;
+    const int band = rr_band<T>(F.nlon, F.nz, K), bands = (K.nlat_c + band - 1) / band;
+    for (int band0 = 0; band0 < bands; band0 += 65535) {  // grid z limit
+        const dim3 grid((warps * 32 + kBlock - 1) / kBlock, F.nz, std::min(65535, bands - band0));
+        k_ns_presmooth_restrict<T><<<grid, kBlock, 0, s>>>(F, K, b, u, bc, T(1) - (T)omega, band0,
+                                                           band);
+    }
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -1085,6 +1117,9 @@ cudaError_t launch_coeff_grad(int nlon, int nlat, int nz, const double *lam, con
                                                   const T *, T *, cudaStream_t, const int *, bool, \
                                                   double);                                        \
     template int rr_band<T>(const LevelDev<T> &, const LinkDev &);                                 \
+    template cudaError_t launch_ns_presmooth_restrict<T>(const NsView<T> &, const LinkDev &,       \
+                                                         const T *, const T *, T *, double,        \
+                                                         cudaStream_t);                            \
     template cudaError_t launch_restrict<T>(const LevelDev<T> &, const LinkDev &, const T *, T *,  \
                                             cudaStream_t, const int *);                           \
     template cudaError_t launch_prolong_add<T>(const LevelDev<T> &, const LinkDev &, const T *,    \

@@ -465,6 +465,7 @@ template <typename T>
 cudaError_t launch_ns_smooth(const NsView<T> &V, const T *b, const T *u_in, T *u_out,
                              double omega, cudaStream_t s)
 {
+    if (launch_ns_sweep<T>(V, b, u_in, u_out, omega, s) >= 0) return cudaGetLastError();
     const int grid = col_blocks(V, kNsSmoothBlock);
     if (u_in)
         k_ns_smooth<T><<<grid, kNsSmoothBlock, 0, s>>>(V, b, u_in, u_out, (T)omega);

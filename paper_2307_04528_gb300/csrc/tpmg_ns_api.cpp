@@ -274,6 +274,7 @@ int ns_setup(mg_ns_handle *H, const mg_ns_coeffs *co, void *ws, size_t ws_bytes,
     if (ws_bytes < need)
         return fail(MG_ERR_WORKSPACE, "workspace %zu bytes < %zu needed", ws_bytes, need);
     ns_carve(H, ws);
+    CU(smooth_prepare());
     NsLevel &f = H->lev[0];
     const size_t bytes0 = f.n * sizeof(double);
     const double *src[7] = {co->h, co->tx, co->ty, co->tz, co->txr, co->tyr, co->tzr};
@@ -366,18 +367,27 @@ int ns_vcycle_level(mg_ns_handle *H, int l, bool tr, const T *b, T *out, cudaStr
     const NsView<T> V = view<T>(v, tr);
     const double om = H->p.omega;
     const int nu1 = H->p.nu1, nu2 = H->p.nu2;
-    if (l == H->L - 1) return ns_sweeps<T>(V, b, nullptr, H->p.coarse_iters, out, a.w, om, s);
+    if (l == H->L - 1) {
+        if (H->p.coarse_iters < 2 || !ns_coarse_fits<T>(V))
+            return ns_sweeps<T>(V, b, nullptr, H->p.coarse_iters, out, a.w, om, s);
+        NRUN(launch_ns_coarse<T>(V, b, out, om, H->p.coarse_iters, s));
+        return MG_OK;
+    }
     // the pre-smoothed iterate lives where nu2 post-sweeps alternating with
     // a.w end in out: a.w for odd nu2, out for even
     T *pre = (nu2 % 2 == 1) ? a.w : out;
     CHK(ns_sweeps<T>(V, b, nullptr, nu1, pre, pre == out ? a.w : out, om, s));
-    if (nu1 == 1)
-        NRUN(launch_ns_presmooth_resid<T>(V, b, pre, om, a.r, s));
-    else
-        NRUN(launch_ns_stencil<T>(V, 1, b, pre, a.r, s));
     NsLevel &c = H->lev[l + 1];
     NsArrays<T> &ca = arr<T>(c);
-    NRUN(launch_restrict<T>(shape_of<T>(v), v.linkdev, a.r, ca.b, s));
+    if (nu1 == 1 && resid_restrict_fits(b, pre, sizeof(T))) {
+        NRUN(launch_ns_presmooth_restrict<T>(V, v.linkdev, b, pre, ca.b, om, s));
+    } else {
+        if (nu1 == 1)
+            NRUN(launch_ns_presmooth_resid<T>(V, b, pre, om, a.r, s));
+        else
+            NRUN(launch_ns_stencil<T>(V, 1, b, pre, a.r, s));
+        NRUN(launch_restrict<T>(shape_of<T>(v), v.linkdev, a.r, ca.b, s));
+    }
     CHK(ns_vcycle_level<T>(H, l + 1, tr, ca.b, ca.u, s));
     NRUN(launch_prolong_add<T>(shape_of<T>(v), v.linkdev, ca.u, pre, s));
     if (nu2 > 0) CHK(ns_sweeps<T>(V, b, pre, nu2, out, a.w, om, s));

@@ -16,9 +16,10 @@ namespace {
 // more tiles than there are slots for partial sums.  (The loop also has the
 // compiler issue a tile's loads in one run: 0.534 ms against 0.698 without it
 // at 1536 x 1152 x 70, the same instructions otherwise.)
-template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB>
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB,
+          typename Level>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_sweep(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
+k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
         T omega, double *__restrict__ partial, const int *__restrict__ flag)
 {
     if (flag && !*flag) return;
@@ -67,10 +68,15 @@ using SmallTall = Shape<1, 3, 8, 512, 1>;  // more than 72 layers
 // 43.8 -> 20.3 us, Small 26.2; 64 x 32 x 16: 9.6 -> 7.6, Small 4.1)
 using Mid64 = Shape<1, 9, 8, 192, 1>;
 
-template <typename T, typename S, bool GUESS, bool DOT>
+// Directed FP32 levels that fill the GPU: one more array per layer in
+// registers, two more read around it.
+using NsLarge0 = Shape<2, 9, 32, 256, 2, false>;
+using NsLarge = Shape<4, 5, 16, 256, 2>;
+
+template <typename T, typename S, bool GUESS, bool DOT, typename Level = LevelDev<T>>
 constexpr auto kernel_of()
 {
-    return k_sweep<T, S::CV, S::LZ, S::QL, GUESS, DOT, S::MAXT, S::MINB>;
+    return k_sweep<T, S::CV, S::LZ, S::QL, GUESS, DOT, S::MAXT, S::MINB, Level>;
 }
 
 template <typename S>
@@ -79,14 +85,14 @@ int threads_of(int nz)  // whole warps: a segment past the last owns no layer
     return ((nz + S::LZ - 1) / S::LZ * S::QL + 31) / 32 * 32;
 }
 
-template <typename T, typename S, bool DOT>
+template <typename T, typename S, bool DOT, typename Level = LevelDev<T>>
 size_t smem_of(int threads)
 {
-    return (size_t)(3 + (DOT ? S::LZ : 0)) * threads * S::CV * sizeof(T);
+    return (size_t)(3 + kDirected<Level> + (DOT ? S::LZ : 0)) * threads * S::CV * sizeof(T);
 }
 
-template <typename T, typename S>
-bool suits(const LevelDev<T> &L, uintptr_t ptrs)
+template <typename T, typename S, typename Level>
+bool suits(const Level &L, uintptr_t ptrs)
 {
     return L.nlon % S::CV == 0 && threads_of<S>(L.nz) <= S::MAXT && ptrs % (S::CV * sizeof(T)) == 0;
 }
@@ -103,8 +109,8 @@ struct Sweep {
     bool dot, count;
 };
 
-template <typename T, typename S>
-int go(const LevelDev<T> &L, const Sweep<T> &a)
+template <typename T, typename S, typename Level>
+int go(const Level &L, const Sweep<T> &a)
 {
     const long long per = S::QL * S::CV;
     const long long tiles = ((long long)L.nlon * L.nlat + per - 1) / per;
@@ -117,14 +123,17 @@ int go(const LevelDev<T> &L, const Sweep<T> &a)
     const cudaStream_t s = a.s;
     const int *flag = a.flag;
     if (!uin)
-        kernel_of<T, S, false, false>()<<<grid, threads, smem_of<T, S, false>(threads), s>>>(
+        kernel_of<T, S, false, false, Level>()<<<grid, threads,
+                                                 smem_of<T, S, false, Level>(threads), s>>>(
             L, b, uin, uout, (T)omega, partial, flag);
     if constexpr (S::GUESS) {
-        if (uin && partial)
-            kernel_of<T, S, true, true>()<<<grid, threads, smem_of<T, S, true>(threads), s>>>(
-                L, b, uin, uout, (T)omega, partial, flag);
-        else if (uin)
-            kernel_of<T, S, true, false>()<<<grid, threads, smem_of<T, S, false>(threads), s>>>(
+        if constexpr (!kDirected<Level>)
+            if (uin && partial)
+                kernel_of<T, S, true, true>()<<<grid, threads, smem_of<T, S, true>(threads), s>>>(
+                    L, b, uin, uout, (T)omega, partial, flag);
+        if (uin && !partial)
+            kernel_of<T, S, true, false, Level>()<<<grid, threads,
+                                                    smem_of<T, S, false, Level>(threads), s>>>(
                 L, b, uin, uout, (T)omega, partial, flag);
     }
     return grid;
@@ -135,28 +144,30 @@ int waste(int nz, int lz) { return ((nz + lz - 1) / lz * lz - nz) * 100 / nz; }
 
 constexpr int kSmallColumns = 2048, kMidColumns = 8192;
 
-template <typename T, typename S, bool DOT>
+template <typename T, typename S, bool DOT, typename Level = LevelDev<T>>
 cudaError_t allow_smem()
 {
-    const int need = (int)smem_of<T, S, DOT>(S::MAXT);
+    const int need = (int)smem_of<T, S, DOT, Level>(S::MAXT);
     if (need <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute((const void *)kernel_of<T, S, true, DOT>(),
+    return cudaFuncSetAttribute((const void *)kernel_of<T, S, true, DOT, Level>(),
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, need);
 }
 
 constexpr int kClusterBlocks = 8;  // the portable cluster size
 
 // Threads of a block of the coarsest-level solve: what its registers allow.
-template <typename T, int LZ>
-constexpr int kClusterThreads = sizeof(T) == 4 ? 512 : LZ <= 4 ? 384 : 256;
+template <typename T, int LZ, typename Level>
+constexpr int kClusterThreads = sizeof(T) == 4 && !kDirected<Level> ? 512
+                                : sizeof(T) == 4 || LZ <= 4         ? 384
+                                                                    : 256;
 
-template <typename T, int LZ>
-__global__ void __launch_bounds__(kClusterThreads<T, LZ>, 1)
-k_coarse_cluster(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
+template <typename T, int LZ, typename Level>
+__global__ void __launch_bounds__(kClusterThreads<T, LZ, Level>, 1)
+k_coarse_cluster(Level L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
                  int R)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    coarse_cluster<T, LZ>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
+    coarse_cluster<T, LZ, Level>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
 }
 
 // Layers per segment, balancing the dependent steps: about ten operations a
@@ -185,7 +196,7 @@ ClusterShape cluster_shape(int nlon, int nlat, int nz)
     c.R = (nlat + blocks - 1) / blocks;
     c.blocks = (nlat + c.R - 1) / c.R;
     c.threads = (c.R * nlon * ((nz + c.lz - 1) / c.lz) + 31) / 32 * 32;
-    c.values = 2 * (size_t)c.R * nlon * nz + 3 * (size_t)c.threads;
+    c.values = 2 * (size_t)c.R * nlon * nz + 4 * (size_t)c.threads;
     return c;
 }
 
@@ -194,18 +205,23 @@ ClusterShape cluster_shape(int nlon, int nlat, int nz)
 // operations per cell against 10, and the walk is bound by the FP64 pipe),
 // FP32 levels that fill the GPU with rows of no whole quad, and layer counts
 // beyond the shapes' registers.
-template <typename T>
-int pick(const LevelDev<T> &L, const Sweep<T> &a)
+template <typename T, typename Level>
+int pick(const Level &L, const Sweep<T> &a)
 {
     const long long ncol = (long long)L.nlon * L.nlat;
     if ((unsigned long long)ncol * L.nz * sizeof(T) >= 1ull << 32) return -1;  // 32-bit offsets
     const uintptr_t ptrs = (uintptr_t)a.b | (uintptr_t)a.uin | (uintptr_t)a.uout |
-                           (uintptr_t)L.tx | (uintptr_t)L.ty | (uintptr_t)L.m | (uintptr_t)L.dq;
+                           (uintptr_t)east_of(L) | (uintptr_t)north_of(L) |
+                           (uintptr_t)west_of(L) | (uintptr_t)south_of(L) |
+                           (uintptr_t)down_of(L) | (uintptr_t)L.m | (uintptr_t)L.dq;
     if constexpr (sizeof(T) == 8) {
         if (ncol > kMidColumns) return -1;
         if (ncol * L.nz >= 1 << 16 && suits<T, Mid64>(L, ptrs)) return go<T, Mid64>(L, a);
     } else if (ncol < kMidColumns) {
         if (ncol >= kSmallColumns && suits<T, Mid>(L, ptrs)) return go<T, Mid>(L, a);
+    } else if constexpr (kDirected<Level>) {
+        if (a.uin) return suits<T, NsLarge>(L, ptrs) ? go<T, NsLarge>(L, a) : -1;
+        return suits<T, NsLarge0>(L, ptrs) ? go<T, NsLarge0>(L, a) : -1;
     } else {
         if (waste(L.nz, 9) >= waste(L.nz, 5) + 8 && suits<T, Large5>(L, ptrs))
             return go<T, Large5>(L, a);
@@ -241,14 +257,23 @@ bool coarse_solve_fits(int nlon, int nlat, int nz)
 {
     if (nlon > 512) return false;
     const ClusterShape c = cluster_shape<T>(nlon, nlat, nz);
-    const int most = sizeof(T) == 4 ? kClusterThreads<float, 4>
-                     : c.lz <= 4    ? kClusterThreads<double, 4>
-                                    : kClusterThreads<double, 6>;
+    const int most = c.lz <= 4 ? kClusterThreads<T, 4, LevelDev<T>>
+                               : kClusterThreads<T, 6, LevelDev<T>>;
     return c.threads <= most && c.values * sizeof(T) <= 160 * 1024;
 }
 
 template <typename T>
-cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
+bool ns_coarse_fits(const NsView<T> &V)
+{
+    if (V.nlon > 512) return false;
+    const ClusterShape c = cluster_shape<T>(V.nlon, V.nlat, V.nz);
+    const int most = c.lz <= 4 ? kClusterThreads<T, 4, NsView<T>>
+                               : kClusterThreads<T, 6, NsView<T>>;
+    return c.threads <= most && c.values * sizeof(T) <= 160 * 1024;
+}
+
+template <typename T, typename Level>
+static cudaError_t coarse_solve(const Level &L, const T *b, T *out, double omega, int sweeps,
                                 cudaStream_t s)
 {
     const ClusterShape c = cluster_shape<T>(L.nlon, L.nlat, L.nz);
@@ -265,8 +290,8 @@ cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double
     cfg.numAttrs = 1;
     const T om = (T)omega;
     auto run = [&](auto lz) {
-        return cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, decltype(lz)::value>, L, b, out, om,
-                                  sweeps, c.R);
+        return cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, decltype(lz)::value, Level>, L, b, out,
+                                  om, sweeps, c.R);
     };
     if constexpr (sizeof(T) == 8) {
         if (c.lz == 2) return run(std::integral_constant<int, 2>{});
@@ -281,22 +306,52 @@ cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double
     }
 }
 
+template <typename T>
+cudaError_t launch_coarse_solve(const LevelDev<T> &L, const T *b, T *out, double omega, int sweeps,
+                                cudaStream_t s)
+{
+    return coarse_solve<T>(L, b, out, omega, sweeps, s);
+}
+
+template <typename T>
+cudaError_t launch_ns_coarse(const NsView<T> &V, const T *b, T *out, double omega, int sweeps,
+                             cudaStream_t s)
+{
+    return coarse_solve<T>(V, b, out, omega, sweeps, s);
+}
+
+template <typename T>
+int launch_ns_sweep(const NsView<T> &V, const T *b, const T *u_in, T *u_out, double omega,
+                    cudaStream_t s)
+{
+    return pick<T>(V, {b, u_in, u_out, omega, nullptr, s, nullptr, false, false});
+}
+
+template <typename T, typename Level>
+static cudaError_t allow_coarse_smem()
+{
+    const void *k4[] = {(const void *)k_coarse_cluster<T, 4, Level>,
+                        (const void *)k_coarse_cluster<T, 6, Level>,
+                        (const void *)k_coarse_cluster<T, sizeof(T) == 4 ? 8 : 2, Level>,
+                        (const void *)k_coarse_cluster<T, sizeof(T) == 4 ? 12 : 3, Level>};
+    for (const void *k : k4) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t sweep_prepare()
 {
-    cudaError_t e;
     for (cudaError_t q : {allow_smem<float, Large, true>(), allow_smem<float, Large5, true>(),
                           allow_smem<float, Mid, true>(), allow_smem<float, SmallTall, true>(),
-                          allow_smem<double, Mid64, true>(), allow_smem<double, SmallTall, true>()})
+                          allow_smem<double, Mid64, true>(), allow_smem<double, SmallTall, true>(),
+                          allow_coarse_smem<float, LevelDev<float>>(),
+                          allow_coarse_smem<double, LevelDev<double>>(),
+                          allow_coarse_smem<float, NsView<float>>(),
+                          allow_coarse_smem<double, NsView<double>>()})
         if (q != cudaSuccess) return q;
-    const void *coarse[] = {
-        (const void *)k_coarse_cluster<float, 4>,  (const void *)k_coarse_cluster<float, 6>,
-        (const void *)k_coarse_cluster<float, 8>,  (const void *)k_coarse_cluster<float, 12>,
-        (const void *)k_coarse_cluster<double, 2>, (const void *)k_coarse_cluster<double, 3>,
-        (const void *)k_coarse_cluster<double, 4>, (const void *)k_coarse_cluster<double, 6>};
-    for (const void *k : coarse)
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      160 * 1024)) != cudaSuccess)
-            return e;
     return cudaSuccess;
 }
 
@@ -306,7 +361,12 @@ cudaError_t sweep_prepare()
     template int smooth_dot_partials<T>(const LevelDev<T> &, const T *, const T *, T *);           \
     template bool coarse_solve_fits<T>(int, int, int);                                             \
     template cudaError_t launch_coarse_solve<T>(const LevelDev<T> &, const T *, T *, double, int, \
-                                                cudaStream_t);
+                                                cudaStream_t);                                    \
+    template int launch_ns_sweep<T>(const NsView<T> &, const T *, const T *, T *, double,          \
+                                    cudaStream_t);                                                \
+    template bool ns_coarse_fits<T>(const NsView<T> &);                                            \
+    template cudaError_t launch_ns_coarse<T>(const NsView<T> &, const T *, T *, double, int,       \
+                                             cudaStream_t);
 TPMG_SWEEP_INST(double)
 TPMG_SWEEP_INST(float)
 #undef TPMG_SWEEP_INST

@@ -205,17 +205,29 @@ __device__ __forceinline__ Vals<T, CV> lds_v(const T *p)
     return r;
 }
 
+// w of the layer's map h_out = F w: (1 - q/p) w, or in a directed level f w
+// with f = d m (the coupling down of the row above times 1/p).
+template <bool NS, typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> carry(const Vals<T, CV> &ndq, const Vals<T, CV> &f,
+                                             const Vals<T, CV> &w)
+{
+    if constexpr (NS) return vmul<T, CV>(f, w);
+    else return vfma<T, CV>(ndq, w, w);
+}
+
 // One tile of QL CV columns.  DOT: returns the thread's part of <b, u_out>,
 // b waiting for the last pass in the thread's own slots of shared memory.
-// Byte offsets are 32-bit (sweep_fits).  sh: 3 blockDim CV values, and LZ
-// blockDim CV more for DOT.
-template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT>
-__device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restrict__ b,
+// Byte offsets are 32-bit (pick).  sh: 3 blockDim CV values (4 in a directed
+// level), and LZ blockDim CV more for DOT.
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, typename Level>
+__device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
                                         const T *__restrict__ uin, T *__restrict__ uout, T omega,
                                         int tile, T *sh)
 {
     using X = Vals<T, CV>;
     constexpr unsigned SZ = sizeof(T);
+    constexpr bool NS = kDirected<Level>;
+    static_assert(!(NS && DOT), "no <b, u_out> of a directed level");
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat;
     const int q = threadIdx.x % QL, seg = threadIdx.x / QL, nseg = blockDim.x / QL;
@@ -227,7 +239,7 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
     const int row = blockDim.x * CV;  // values per slot row of shared memory
     T *sb = sh + 3 * row + threadIdx.x * CV;
 
-    X v[LZ], m[LZ], dq[LZ], uc[GUESS ? LZ : 1];
+    X v[LZ], m[LZ], dq[LZ], uc[GUESS ? LZ : 1], f[NS ? LZ : 1];
     // No load sits behind a branch: layers past the top re-read the last one.
     unsigned off = first;
 #pragma unroll
@@ -236,6 +248,7 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
         dq[c] = ldv<T, CV>(L.dq, off);
         v[c] = ldv<T, CV>(b, off);
         if (GUESS) uc[c] = ldv<T, CV>(uin, off);
+        if constexpr (NS) f[c] = ldv<T, CV>(down_of(L), off);
         off += k0 + c + 1 < nz ? plane : 0u;
     }
     if (GUESS) {
@@ -244,20 +257,23 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
         // rows past a pole read the cell itself
         const T *ue = uin + (i + CV == nlon ? -i : CV), *uw = uin + (i == 0 ? nlon - 1 : -1);
         const T *un = uin + (hasN ? nlon : 0), *us = uin - (hasS ? nlon : 0);
-        const T *tw = L.tx + (i == 0 ? nlon - 1 : -1), *ts = L.ty - (hasS ? nlon : 0);
+        const T *tw = west_of(L) + (i == 0 ? nlon - 1 : -1);
+        const T *ts = south_of(L) - (hasS ? nlon : 0);
         off = first;
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
-            const X t = ldv<T, CV>(L.tx, off);
+            const X t = ldv<T, CV>(east_of(L), off);
+            X tb = t;  // the couplings of the cells to the west
+            if constexpr (NS && CV > 1) tb = ldv<T, CV>(west_of(L), off);
             const X N = ldv<T, CV>(un, off), S = ldv<T, CV>(us, off);
-            const X tn = ldv<T, CV>(L.ty, off), tS = ldv<T, CV>(ts, off);
+            const X tn = ldv<T, CV>(north_of(L), off), tS = ldv<T, CV>(ts, off);
             const T E = ldv<T, 1>(ue, off).a[0], W = ldv<T, 1>(uw, off).a[0];
             const T tW = ldv<T, 1>(tw, off).a[0];
             if (DOT) stv<T, CV>(sb + c * row, 0u, v[c]);
 #pragma unroll
             for (int e = 0; e < CV; ++e) {
                 v[c].a[e] = fma(t.a[e], e + 1 < CV ? uc[c].a[e + 1 < CV ? e + 1 : e] : E, v[c].a[e]);
-                v[c].a[e] = fma(e > 0 ? t.a[e > 0 ? e - 1 : 0] : tW,
+                v[c].a[e] = fma(e > 0 ? tb.a[e > 0 ? e - 1 : 0] : tW,
                                 e > 0 ? uc[c].a[e > 0 ? e - 1 : 0] : W, v[c].a[e]);
             }
             const X vn = vfma<T, CV>(tn, N, v[c]);
@@ -274,17 +290,24 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
     for (int c = 0; c < LZ; ++c) {
         m[c] = k0 + c < nz ? m[c] : zero;
         dq[c] = vneg<T, CV>(dq[c]);
+        if constexpr (NS) f[c] = vmul<T, CV>(f[c], m[c]);
     }
 
-    // forward: the segment's map h_out = A h_in + C
-    X A = splat<T, CV>(T(1)), C = zero;
+    // forward: the segment's map h_out = A h_in + C; backward factor B (= A in
+    // a symmetric level)
+    X A = splat<T, CV>(T(1)), C = zero, B = A;
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const X t = vadd<T, CV>(v[c], C);
-        C = vfma<T, CV>(dq[c], t, t);
-        A = vfma<T, CV>(dq[c], A, A);
+        C = carry<NS, T, CV>(dq[c], f[NS ? c : 0], t);
+        A = carry<NS, T, CV>(dq[c], f[NS ? c : 0], A);
+        if constexpr (NS) B = vfma<T, CV>(dq[c], B, B);
     }
-    T *sA = sh + q * CV, *sC = sA + row, *sF = sC + row;
+    T *sA = sh + q * CV, *sC = sA + row, *sF = sC + row, *sB = sA;
+    if constexpr (NS) {
+        sB = sh + (3 + (DOT ? LZ : 0)) * row + q * CV;
+        stv<T, CV>(sB + seg * QL * CV, 0u, B);
+    }
     stv<T, CV>(sA + seg * QL * CV, 0u, A);
     stv<T, CV>(sC + seg * QL * CV, 0u, C);
     __syncthreads();
@@ -296,7 +319,7 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const X w = vadd<T, CV>(v[c], h);
-        h = vfma<T, CV>(dq[c], w, w);
+        h = carry<NS, T, CV>(dq[c], f[NS ? c : 0], w);
         v[c] = vmul<T, CV>(w, m[c]);
     }
     X F = zero;
@@ -306,7 +329,7 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
     __syncthreads();
     X x = zero;
     for (int s = nseg - 1; s > seg; --s)
-        x = vfma<T, CV>(lds_v<T, CV>(sA + s * QL * CV), x, lds_v<T, CV>(sF + s * QL * CV));
+        x = vfma<T, CV>(lds_v<T, CV>(sB + s * QL * CV), x, lds_v<T, CV>(sF + s * QL * CV));
     const X om = splat<T, CV>(omega), om1 = splat<T, CV>(T(1) - omega);
     T acc = 0;
     off = first + (unsigned)(min(LZ, nz - k0) - 1) * plane;
@@ -337,19 +360,21 @@ __device__ __forceinline__ T sweep_tile(const LevelDev<T> &L, const T *__restric
 // copies written in turn; the rows beside a block's own are read from its
 // neighbours' shared memory, and one cluster barrier separates the sweeps.
 // The forward and backward maps of the segments are exchanged as in
-// sweep_tile, the factor A once.  sh: 2 R nlon nz + 3 blockDim values.
-template <typename T, int LZ>
-__device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__restrict__ b,
+// sweep_tile, their factors once.  sh: 2 R nlon nz + 4 blockDim values.
+template <typename T, int LZ, typename Level>
+__device__ __forceinline__ void coarse_cluster(const Level &L, const T *__restrict__ b,
                                                T *__restrict__ out, T omega, int sweeps, int R,
                                                T *sh)
 {
     namespace cg = cooperative_groups;
+    constexpr bool NS = kDirected<Level>;
     cg::cluster_group cl = cg::this_cluster();
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz, plane = nlon * nlat;
     const int rank = (int)cl.block_rank(), j0 = rank * R;
     const int rows = max(0, min(R, nlat - j0)), cols = rows * nlon, part = R * nlon;
     T *u0 = sh, *u1 = sh + part * nz;
     T *sA = sh + 2 * part * nz, *sC = sA + blockDim.x, *sF = sC + blockDim.x;
+    T *sB = NS ? sF + blockDim.x : sA;
     const int nseg = (nz + LZ - 1) / LZ;
     const bool mine = (int)threadIdx.x < cols * nseg;
     const int seg = mine ? threadIdx.x / cols : 0, lc = mine ? threadIdx.x - seg * cols : 0;
@@ -363,21 +388,24 @@ __device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__
         n0 = r + 1 < rows ? u0 + lc + nlon : cl.map_shared_rank(u0, rank + 1) + i;
     if (hasS)
         s0 = r > 0 ? u0 + lc - nlon : cl.map_shared_rank(u0, rank - 1) + (R - 1) * nlon + i;
-    T m[LZ], dq[LZ], bb[LZ], te[LZ], tw[LZ], tn[LZ], ts[LZ], uc[LZ], A = 1;
+    T m[LZ], dq[LZ], bb[LZ], te[LZ], tw[LZ], tn[LZ], ts[LZ], uc[LZ], f[NS ? LZ : 1], A = 1, B = 1;
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const int g = min(k0 + c, nz - 1) * plane + j * nlon + i;
         bb[c] = __ldg(b + g);
-        te[c] = __ldg(L.tx + g);
-        tw[c] = __ldg(L.tx + g + dw);
-        tn[c] = hasN ? __ldg(L.ty + g) : T(0);
-        ts[c] = hasS ? __ldg(L.ty + g - nlon) : T(0);
+        te[c] = __ldg(east_of(L) + g);
+        tw[c] = __ldg(west_of(L) + g + dw);
+        tn[c] = hasN ? __ldg(north_of(L) + g) : T(0);
+        ts[c] = hasS ? __ldg(south_of(L) + g - nlon) : T(0);
         m[c] = k0 + c < nz ? __ldg(L.m + g) : T(0);
         dq[c] = -__ldg(L.dq + g);
         uc[c] = 0;
-        A = fma(dq[c], A, A);
+        if constexpr (NS) f[c] = __ldg(down_of(L) + g) * m[c];
+        A = NS ? f[NS ? c : 0] * A : fma(dq[c], A, A);
+        B = fma(dq[c], B, B);
     }
     sA[threadIdx.x] = A;
+    if (NS) sB[threadIdx.x] = B;
     const T om1 = T(1) - omega;
     for (int it = 0; it < sweeps; ++it) {
         const int cur = (it & 1) * part * nz;  // the copy read; the other is written
@@ -395,7 +423,7 @@ __device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__
             }
             v[c] = x;
             const T t = x + C;
-            C = fma(dq[c], t, t);
+            C = NS ? f[NS ? c : 0] * t : fma(dq[c], t, t);
         }
         sC[threadIdx.x] = C;
         __syncthreads();
@@ -405,7 +433,7 @@ __device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
             const T w = v[c] + h;
-            h = fma(dq[c], w, w);
+            h = NS ? f[NS ? c : 0] * w : fma(dq[c], w, w);
             v[c] = w * m[c];
         }
         T F = 0;
@@ -415,7 +443,7 @@ __device__ __forceinline__ void coarse_cluster(const LevelDev<T> &L, const T *__
         __syncthreads();
         T x = 0;
 #pragma unroll 4
-        for (int s = nseg - 1; s > seg; --s) x = fma(sA[s * cols + lc], x, sF[s * cols + lc]);
+        for (int s = nseg - 1; s > seg; --s) x = fma(sB[s * cols + lc], x, sF[s * cols + lc]);
 #pragma unroll
         for (int c = LZ - 1; c >= 0; --c) {
             x = x + fma(dq[c], x, v[c]);
