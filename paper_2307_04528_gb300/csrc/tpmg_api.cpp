@@ -1283,7 +1283,12 @@ extern "C" int mg_solve_mixed(mg_handle *H, const double *b, double *x, double t
     if (!H || !b || !x) return fail(MG_ERR_ARG, "null argument");
     if (!H->p.mixed) return fail(MG_ERR_ARG, "handle built without the FP32 hierarchy (mixed=0)");
     if (!(tol >= 0)) return fail(MG_ERR_ARG, "tol must be >= 0");
-    cudaStream_t s = (cudaStream_t)stream;
+    return solve_mixed(H, b, x, tol, H->p.method, st, (cudaStream_t)stream);
+}
+
+int tpmg::solve_mixed(mg_handle *H, const double *b, double *x, double tol, int method, mg_stats *st,
+                cudaStream_t s)
+{
     LevelHost &f = H->lev[0];
     LevelDev<double> D = dev<double>(f);
     D.h = f.dh;  // the refinement residual takes the horizontal diagonal (launch_residual_cast)
@@ -1353,8 +1358,8 @@ extern "C" int mg_solve_mixed(mg_handle *H, const double *b, double *x, double t
         double rel_in = 0;
         // solve no further than the outer target still needs (safety 0.3)
         const double itol = inner_tolerance(H->p.inner_tol, tol, rel);
-        const int rin = solve_impl<float>(H, f.b32, H->cg32.x, itol, H->p.inner_maxit,
-                                          H->p.method, nullptr, &its_in, &rel_in, s, true);
+        const int rin = solve_impl<float>(H, f.b32, H->cg32.x, itol, H->p.inner_maxit, method,
+                                          nullptr, &its_in, &rel_in, s, true);
         if (rin != MG_OK && rin != MG_ERR_NOT_CONVERGED && rin != MG_ERR_DIVERGED) {
             rc = rin;
             break;

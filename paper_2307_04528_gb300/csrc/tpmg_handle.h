@@ -222,4 +222,8 @@ int handle_plan(const mg_grid *g, const mg_params *p, void *ws, size_t *bytes, m
 int handle_setup(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_bytes, cudaStream_t s);
 int read_scalars(mg_handle *H, int which, double *out, cudaStream_t s);
 double inner_tolerance(double inner_tol, double tol, double rel);
+
+// mg_solve_mixed with the inner iteration named (MG_METHOD_*).
+int solve_mixed(mg_handle *H, const double *b, double *x, double tol, int method, mg_stats *st,
+                cudaStream_t s);
 }  // namespace tpmg
