@@ -246,6 +246,14 @@ template <typename T>
 cudaError_t launch_scale(T *x, double f, size_t n, cudaStream_t s);
 // per-block maxima of (h + horizontal couplings) / h over the level
 int launch_hz_ratio(const LevelDev<double> &L, double *partial, cudaStream_t s);
+// A Chebyshev step in one pass: r_out = r - H d, x += d (first: x = d), d_out =
+// c1 d + c2 H_z^{-1} r_out (last: x takes it too), where the segmented sweeps
+// take the level and the buffers (cheb_sweep_fits).  r_out may be r.
+template <typename T>
+bool cheb_sweep_fits(const LevelDev<T> &L, const T *r, const T *d, T *d_out, T *r_out, T *x);
+template <typename T>
+cudaError_t launch_cheb_sweep(const LevelDev<T> &L, const T *r, const T *d, T *d_out, T *r_out,
+                              T *x, double c1, double c2, bool first, bool last, cudaStream_t s);
 // Chebyshev step: x += d, d = c1 d + c2 z (first: d = c2 z)
 template <typename T>
 cudaError_t launch_cheb_step(T *x, T *d, const T *z, double c1, double c2, size_t n, bool first,

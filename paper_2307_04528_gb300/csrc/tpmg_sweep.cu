@@ -34,6 +34,21 @@ k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restri
     if (DOT) block_store<0>((double)acc, partial);
 }
 
+// A Chebyshev step of the coarsest-level solve as one sweep (launch_cheb_sweep).
+template <typename T, int CV, int LZ, int QL, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+k_sweep_cheb(LevelDev<T> L, const T *b, const T *__restrict__ uin,
+             T *__restrict__ uout, ChebStep<T> ch)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int tiles = (L.nlon * L.nlat + QL * CV - 1) / (QL * CV);
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        if (tile != (int)blockIdx.x) __syncthreads();  // the last tile's maps have been read
+        sweep_tile<T, CV, LZ, QL, true, false, true>(L, b, uin, uout, T(1), tile,
+                                                     reinterpret_cast<T *>(smraw), ch);
+    }
+}
+
 // A shape of the sweep: CV columns per thread, LZ layers per segment, QL
 // lanes along longitude, MAXT threads at most, MINB blocks per SM.
 template <int CV_, int LZ_, int QL_, int MAXT_, int MINB_, bool GUESS_ = true>
@@ -107,6 +122,7 @@ struct Sweep {
     cudaStream_t s;
     const int *flag;
     bool dot, count;
+    const ChebStep<T> *ch = nullptr;  // a Chebyshev step
 };
 
 template <typename T, typename S, typename Level>
@@ -126,6 +142,13 @@ int go(const Level &L, const Sweep<T> &a)
         kernel_of<T, S, false, false, Level>()<<<grid, threads,
                                                  smem_of<T, S, false, Level>(threads), s>>>(
             L, b, uin, uout, (T)omega, partial, flag);
+    if constexpr (S::GUESS && !kDirected<Level>) {
+        if (a.ch) {
+            k_sweep_cheb<T, S::CV, S::LZ, S::QL, S::MAXT, S::MINB>
+                <<<grid, threads, smem_of<T, S, false>(threads), s>>>(L, b, uin, uout, *a.ch);
+            return grid;
+        }
+    }
     if constexpr (S::GUESS) {
         if constexpr (!kDirected<Level>)
             if (uin && partial)
@@ -213,7 +236,9 @@ int pick(const Level &L, const Sweep<T> &a)
     const uintptr_t ptrs = (uintptr_t)a.b | (uintptr_t)a.uin | (uintptr_t)a.uout |
                            (uintptr_t)east_of(L) | (uintptr_t)north_of(L) |
                            (uintptr_t)west_of(L) | (uintptr_t)south_of(L) |
-                           (uintptr_t)down_of(L) | (uintptr_t)L.m | (uintptr_t)L.dq;
+                           (uintptr_t)down_of(L) | (uintptr_t)L.m | (uintptr_t)L.dq |
+                           (uintptr_t)mass_of(L) | (uintptr_t)up_of(L) |
+                           (a.ch ? (uintptr_t)a.ch->r_out | (uintptr_t)a.ch->x : 0);
     if constexpr (sizeof(T) == 8) {
         if (ncol > kMidColumns) return -1;
         if (ncol * L.nz >= 1 << 16 && suits<T, Mid64>(L, ptrs)) return go<T, Mid64>(L, a);
@@ -239,6 +264,22 @@ int launch_sweep(const LevelDev<T> &L, const T *b, const T *uin, T *uout, double
                  double *partial, cudaStream_t s, const int *flag)
 {
     return pick<T>(L, {b, uin, uout, omega, partial, s, flag, partial != nullptr, false});
+}
+
+template <typename T>
+bool cheb_sweep_fits(const LevelDev<T> &L, const T *b, const T *d, T *d_out, T *r_out, T *x)
+{
+    const ChebStep<T> ch{r_out, x, T(0), T(0), false, false};
+    return pick<T>(L, {b, d, d_out, 1.0, nullptr, nullptr, nullptr, false, true, &ch}) >= 0;
+}
+
+template <typename T>
+cudaError_t launch_cheb_sweep(const LevelDev<T> &L, const T *b, const T *d, T *d_out, T *r_out,
+                              T *x, double c1, double c2, bool first, bool last, cudaStream_t s)
+{
+    const ChebStep<T> ch{r_out, x, (T)c1, (T)c2, first, last};
+    pick<T>(L, {b, d, d_out, 1.0, nullptr, s, nullptr, false, false, &ch});
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -358,6 +399,9 @@ cudaError_t sweep_prepare()
 #define TPMG_SWEEP_INST(T)                                                                       \
     template int launch_sweep<T>(const LevelDev<T> &, const T *, const T *, T *, double, double *, \
                                  cudaStream_t, const int *);                                     \
+    template bool cheb_sweep_fits<T>(const LevelDev<T> &, const T *, const T *, T *, T *, T *);    \
+    template cudaError_t launch_cheb_sweep<T>(const LevelDev<T> &, const T *, const T *, T *, T *, \
+                                              T *, double, double, bool, bool, cudaStream_t);     \
     template int smooth_dot_partials<T>(const LevelDev<T> &, const T *, const T *, T *);           \
     template bool coarse_solve_fits<T>(int, int, int);                                             \
     template cudaError_t launch_coarse_solve<T>(const LevelDev<T> &, const T *, T *, double, int, \

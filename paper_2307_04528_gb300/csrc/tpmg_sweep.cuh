@@ -71,6 +71,27 @@ __device__ __forceinline__ Vals<T, CV> ldv(const T *__restrict__ p, unsigned byt
     return r;
 }
 
+// The same for values this kernel also writes (not through the read-only path).
+template <typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> ldv_own(const T *p, unsigned byte)
+{
+    Vals<T, CV> r;
+    const char *q = reinterpret_cast<const char *>(p) + byte;
+    if constexpr (CV == 1) {
+        r.a[0] = *reinterpret_cast<const T *>(q);
+    } else {
+        using V = typename VecOf<T, CV>::type;
+        const V v = *reinterpret_cast<const V *>(q);
+        r.a[0] = v.x;
+        r.a[1] = v.y;
+        if constexpr (CV == 4) {
+            r.a[2] = v.z;
+            r.a[3] = v.w;
+        }
+    }
+    return r;
+}
+
 template <typename T, int CV>
 __device__ __forceinline__ void stv(T *__restrict__ p, unsigned byte, const Vals<T, CV> &x)
 {
@@ -215,14 +236,26 @@ __device__ __forceinline__ Vals<T, CV> carry(const Vals<T, CV> &ndq, const Vals<
     else return vfma<T, CV>(ndq, w, w);
 }
 
+// A Chebyshev step instead of a sweep: with b the residual and u_in the step d,
+// r_out = b - H d, x += d (first: x = d) and u_out = c1 d + c2 H_z^{-1} r_out;
+// last: x takes the new step too.  Each cell of r_out (may be b) and x is its
+// own thread's.
+template <typename T>
+struct ChebStep {
+    T *r_out, *x;
+    T c1, c2;
+    bool first, last;
+};
+
 // One tile of QL CV columns.  DOT: returns the thread's part of <b, u_out>,
 // b waiting for the last pass in the thread's own slots of shared memory.
 // Byte offsets are 32-bit (pick).  sh: 3 blockDim CV values (4 in a directed
 // level), and LZ blockDim CV more for DOT.
-template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, typename Level>
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, bool CHEB = false,
+          typename Level>
 __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
                                         const T *__restrict__ uin, T *__restrict__ uout, T omega,
-                                        int tile, T *sh)
+                                        int tile, T *sh, const ChebStep<T> &ch = {})
 {
     using X = Vals<T, CV>;
     constexpr unsigned SZ = sizeof(T);
@@ -246,7 +279,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
     for (int c = 0; c < LZ; ++c) {
         m[c] = ldv<T, CV>(L.m, off);
         dq[c] = ldv<T, CV>(L.dq, off);
-        v[c] = ldv<T, CV>(b, off);
+        v[c] = CHEB ? ldv_own<T, CV>(b, off) : ldv<T, CV>(b, off);
         if (GUESS) uc[c] = ldv<T, CV>(uin, off);
         if constexpr (NS) f[c] = ldv<T, CV>(down_of(L), off);
         off += k0 + c + 1 < nz ? plane : 0u;
@@ -260,6 +293,14 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
         const T *tw = west_of(L) + (i == 0 ? nlon - 1 : -1);
         const T *ts = south_of(L) - (hasS ? nlon : 0);
         off = first;
+        // CHEB: t_z and d of the layer below the segment, d of the one above
+        X tzd = splat<T, CV>(T(0)), ud = tzd, ua = tzd;
+        if constexpr (CHEB) {
+            const unsigned dn = k0 > 0 ? plane : 0u;
+            tzd = ldv<T, CV>(up_of(L), first - dn);
+            ud = ldv<T, CV>(uin, first - dn);
+            ua = ldv<T, CV>(uin, first + (k0 + LZ < nz ? LZ * plane : 0u));
+        }
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
             const X t = ldv<T, CV>(east_of(L), off);
@@ -269,6 +310,29 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
             const X tn = ldv<T, CV>(north_of(L), off), tS = ldv<T, CV>(ts, off);
             const T E = ldv<T, 1>(ue, off).a[0], W = ldv<T, 1>(uw, off).a[0];
             const T tW = ldv<T, 1>(tw, off).a[0];
+            if constexpr (CHEB) {
+                // r = b - H d in flux form
+                const X hm = ldv<T, CV>(mass_of(L), off), tz = ldv<T, CV>(up_of(L), off);
+                const X &U = c + 1 < LZ ? uc[c + 1 < LZ ? c + 1 : c] : ua;
+                const X &D = c > 0 ? uc[c > 0 ? c - 1 : 0] : ud;
+#pragma unroll
+                for (int e = 0; e < CV; ++e) {
+                    const T x = uc[c].a[e];
+                    T s = hm.a[e] * x;
+                    s = fma(t.a[e], x - (e + 1 < CV ? uc[c].a[e + 1 < CV ? e + 1 : e] : E), s);
+                    s = fma(e > 0 ? t.a[e > 0 ? e - 1 : 0] : tW,
+                            x - (e > 0 ? uc[c].a[e > 0 ? e - 1 : 0] : W), s);
+                    if (hasN) s = fma(tn.a[e], x - N.a[e], s);
+                    if (hasS) s = fma(tS.a[e], x - S.a[e], s);
+                    if (k0 + c + 1 < nz) s = fma(tz.a[e], x - U.a[e], s);
+                    if (k0 + c > 0) s = fma(tzd.a[e], x - D.a[e], s);
+                    v[c].a[e] -= s;
+                }
+                tzd = tz;
+                if (own < ncol && k0 + c < nz) stv<T, CV>(ch.r_out, off, v[c]);
+                off += k0 + c + 1 < nz ? plane : 0u;
+                continue;
+            }
             if (DOT) stv<T, CV>(sb + c * row, 0u, v[c]);
 #pragma unroll
             for (int e = 0; e < CV; ++e) {
@@ -322,6 +386,15 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
         h = carry<NS, T, CV>(dq[c], f[NS ? c : 0], w);
         v[c] = vmul<T, CV>(w, m[c]);
     }
+    X xv[CHEB ? LZ : 1];
+    if constexpr (CHEB) {
+        off = first;
+#pragma unroll
+        for (int c = 0; c < LZ; ++c) {
+            xv[c] = ch.first ? zero : ldv_own<T, CV>(ch.x, off);
+            off += k0 + c + 1 < nz ? plane : 0u;
+        }
+    }
     X F = zero;
 #pragma unroll
     for (int c = LZ - 1; c >= 0; --c) F = vadd<T, CV>(F, vfma<T, CV>(dq[c], F, v[c]));
@@ -336,10 +409,18 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
 #pragma unroll
     for (int c = LZ - 1; c >= 0; --c) {
         x = vadd<T, CV>(x, vfma<T, CV>(dq[c], x, v[c]));
-        X uo = vmul<T, CV>(om, x);
-        if (GUESS) uo = vfma<T, CV>(om1, uc[c], uo);
+        X uo;
+        if constexpr (CHEB) {
+            uo = vfma<T, CV>(splat<T, CV>(ch.c2), x, vmul<T, CV>(splat<T, CV>(ch.c1), uc[c]));
+            xv[c] = vadd<T, CV>(xv[c], uc[c]);
+            if (ch.last) xv[c] = vadd<T, CV>(xv[c], uo);
+        } else {
+            uo = vmul<T, CV>(om, x);
+            if (GUESS) uo = vfma<T, CV>(om1, uc[c], uo);
+        }
         if (k0 + c < nz) {
             if (own < ncol) {
+                if constexpr (CHEB) stv<T, CV>(ch.x, off, xv[c]);
                 stv<T, CV>(uout, off, uo);
                 if (DOT) {
                     const X bc = lds_v<T, CV>(sb + c * row);
