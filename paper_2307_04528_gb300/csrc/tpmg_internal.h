@@ -42,6 +42,52 @@ struct CgScalars {
     double rz, rz_new, dAd, rr, alpha, beta, maxabs, pad;
 };
 
+// A kernel launched so that its blocks may be placed while the kernel before it
+// on the stream drains (programmatic dependent launch): it waits at its top,
+// in after_previous(), for that kernel's results, which hides the launch
+// latency between the short kernels of the coarse levels (the FP32 V-cycle at
+// 1024 x 768 x 70 1.085 -> 1.014 ms, those of H and H^T at 512 x 384 x 70 and
+// two applies 1.62 -> 1.50).  Not under capture: in the body of the device-side
+// loop such edges cost more than plain ones (24 Chebyshev steps per coarse solve:
+// 39.9 -> 40.9 ms; 256 x 128 x 32 in FP64: 12.6 -> 13.2).
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous()
+{
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+
+inline cudaLaunchAttribute after_attribute()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+
+inline bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(s, &st);
+    return st != cudaStreamCaptureStatusNone;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                         cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = after_attribute();
+    cfg.attrs = &at;
+    cfg.numAttrs = capturing(s) ? 0 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // State of a conjugate-gradient run whose iterations are a device-side loop
 // (a conditional graph node): set by the host, advanced by the loop's last
 // kernel.  Iteration `its` (0, 1, ...) writes its direction to d0 when even,

@@ -51,6 +51,7 @@ k_dir_apply(LevelDev<T> L, const T *__restrict__ z, const T *__restrict__ d_even
             double *__restrict__ partial, const int *__restrict__ flag,
             const CgLoop *__restrict__ loop)
 {
+    after_previous();
     if (flag && !*flag) return;
     const bool odd = loop && (loop->its & 1);
     const T *__restrict__ dold = loop && loop->its == 0 ? z : odd ? d_to : d_even;
@@ -73,11 +74,11 @@ int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgS
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (d_old == nullptr)
-        k_dir_apply<T, true><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
-                                                     loop);
+        launch_after(k_dir_apply<T, true>, grid, kBlock, 0, s, L, z, d_old, sc, d_new, q, partial,
+                     flag, loop);
     else
-        k_dir_apply<T, false><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
-                                                      loop);
+        launch_after(k_dir_apply<T, false>, grid, kBlock, 0, s, L, z, d_old, sc, d_new, q, partial,
+                     flag, loop);
     return grid;
 }
 
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kBlock)
 k_smooth(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
          T omega, const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     smooth_column<T, false, 0, kYOut<T>>(L, b, uin, uout, omega,
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(kBlock)
 k_smooth0(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ uout, T omega,
           const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     smooth_staged<T, true>(L, b, nullptr, uout, omega, blockIdx.x * blockDim.x + threadIdx.x,
@@ -233,6 +236,7 @@ k_smooth_dot(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin,
              T *__restrict__ uout, T omega, double *__restrict__ partial,
              const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     T acc = 0;
@@ -250,7 +254,8 @@ int launch_smooth_dot(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
     const size_t smem = kYOut<T> ? 0 : (size_t)L.nz * kBlock * sizeof(T);
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
-    k_smooth_dot<T><<<grid, kBlock, smem, s>>>(L, b, u_in, u_out, (T)omega, partial, flag);
+    launch_after(k_smooth_dot<T>, grid, kBlock, smem, s, L, b, u_in, u_out, (T)omega, partial,
+                 flag);
     return grid;
 }
 
@@ -283,10 +288,10 @@ cudaError_t launch_smooth_walk(const LevelDev<T> &L, const T *b, const T *u_in, 
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (u_in == nullptr) {
         const size_t smem = ring_smem_bytes<T, true>(L.nz, kBlock);
-        k_smooth0<T><<<grid, kBlock, smem, s>>>(L, b, u_out, (T)omega, flag);
+        launch_after(k_smooth0<T>, grid, kBlock, smem, s, L, b, u_out, (T)omega, flag);
     } else {
         const size_t smem = kYOut<T> ? 0 : (size_t)L.nz * kBlock * sizeof(T);
-        k_smooth<T><<<grid, kBlock, smem, s>>>(L, b, u_in, u_out, (T)omega, flag);
+        launch_after(k_smooth<T>, grid, kBlock, smem, s, L, b, u_in, u_out, (T)omega, flag);
     }
     return cudaGetLastError();
 }
@@ -368,6 +373,7 @@ __global__ void __launch_bounds__(kBlock, (PRE && sizeof(T) == 4) ? 12 : 0)
 k_resid_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
                  T *__restrict__ bc, T om1, int band0, int band, const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     if (warp * kRROwned >= F.nlon / 2) return;  // whole warps
@@ -381,6 +387,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 8 : 0)
 k_ns_presmooth_restrict(NsView<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
                         T *__restrict__ bc, T om1, int band0, int band)
 {
+    after_previous();
     const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     if (warp * kRROwned >= F.nlon / 2) return;  // whole warps
     resid_restrict_band<T, true>(F, K, b, u, bc, warp, threadIdx.x & 31,
@@ -421,8 +428,8 @@ cudaError_t launch_ns_presmooth_restrict(const NsView<T> &F, const LinkDev &K, c
     const int band = rr_band<T>(F.nlon, F.nz, K), bands = (K.nlat_c + band - 1) / band;
     for (int band0 = 0; band0 < bands; band0 += 65535) {  // grid z limit
         const dim3 grid((warps * 32 + kBlock - 1) / kBlock, F.nz, std::min(65535, bands - band0));
-        k_ns_presmooth_restrict<T><<<grid, kBlock, 0, s>>>(F, K, b, u, bc, T(1) - (T)omega, band0,
-                                                           band);
+        launch_after(k_ns_presmooth_restrict<T>, grid, kBlock, 0, s, F, K, b, u, bc,
+                     T(1) - (T)omega, band0, band);
     }
     return cudaGetLastError();
 }
@@ -440,11 +447,11 @@ cudaError_t launch_resid_restrict(const LevelDev<T> &F, const LinkDev &K, const 
     for (int band0 = 0; band0 < bands; band0 += 65535) {  // grid z limit
         const dim3 grid((warps * 32 + kBlock - 1) / kBlock, F.nz, std::min(65535, bands - band0));
         if (presmooth)
-            k_resid_restrict<T, true><<<grid, kBlock, 0, s>>>(F, K, b, u, bc, om1, band0, band,
-                                                              flag);
+            launch_after(k_resid_restrict<T, true>, grid, kBlock, 0, s, F, K, b, u, bc, om1, band0,
+                         band, flag);
         else
-            k_resid_restrict<T, false><<<grid, kBlock, 0, s>>>(F, K, b, u, bc, om1, band0, band,
-                                                               flag);
+            launch_after(k_resid_restrict<T, false>, grid, kBlock, 0, s, F, K, b, u, bc, om1, band0,
+                         band, flag);
     }
     return cudaGetLastError();
 }
@@ -482,6 +489,7 @@ __global__ void __launch_bounds__(kBlock)
 k_prolong_add(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict__ u, int kz,
               const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     const int k0 = blockIdx.y * kz;
     prolong_layers<T>(F, K, ec, u, blockIdx.x * blockDim.x + threadIdx.x, k0, min(F.nz, k0 + kz));
@@ -499,6 +507,7 @@ __global__ void __launch_bounds__(kBlock)
 k_prolong_quad(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict__ u, int kz,
                const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     using P2 = typename Pair<T>::type;
     constexpr unsigned kAll = 0xffffffffu;
@@ -544,13 +553,13 @@ cudaError_t launch_prolong_add(const LevelDev<T> &F, const LinkDev &K, const T *
         const int quads = (F.nlon / 4) * F.nlat;
         const int kz = layers_per_thread(quads, F.nz);
         const dim3 grid((quads + kBlock - 1) / kBlock, (F.nz + kz - 1) / kz);
-        k_prolong_quad<T><<<grid, kBlock, 0, s>>>(F, K, ec, u, kz, flag);
+        launch_after(k_prolong_quad<T>, grid, kBlock, 0, s, F, K, ec, u, kz, flag);
         return cudaGetLastError();
     }
     const int npair = (F.nlon / 2) * F.nlat;
     const int kz = layers_per_thread(npair, F.nz);
     const dim3 grid((npair + kBlock - 1) / kBlock, (F.nz + kz - 1) / kz);
-    k_prolong_add<T><<<grid, kBlock, 0, s>>>(F, K, ec, u, kz, flag);
+    launch_after(k_prolong_add<T>, grid, kBlock, 0, s, F, K, ec, u, kz, flag);
     return cudaGetLastError();
 }
 
@@ -586,6 +595,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock)
 k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, double *partial)
 {
+    after_previous();
     T acc = 0;
 #pragma unroll 4
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
@@ -608,6 +618,7 @@ static bool vec4_ok(size_t n, const void *a, const void *b = nullptr, const void
 __global__ void __launch_bounds__(kBlock)
 k_dot_f4(const float4 *__restrict__ a, const float4 *__restrict__ b, size_t n4, double *partial)
 {
+    after_previous();
     float acc = 0.f;
 #pragma unroll 2
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n4;
@@ -627,12 +638,12 @@ int launch_dot(const T *a, const T *b, size_t n, double *partial, cudaStream_t s
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
         if (vec4_ok(n, a, b)) {
-            k_dot_f4<<<g, kBlock, 0, s>>>(reinterpret_cast<const float4 *>(a),
-                                          reinterpret_cast<const float4 *>(b), n / 4, partial);
+            launch_after(k_dot_f4, g, kBlock, 0, s, reinterpret_cast<const float4 *>(a),
+                         reinterpret_cast<const float4 *>(b), n / 4, partial);
             return g;
         }
     }
-    k_dot<T><<<g, kBlock, 0, s>>>(a, b, n, partial);
+    launch_after(k_dot<T>, g, kBlock, 0, s, a, b, n, partial);
     return g;
 }
 
@@ -661,6 +672,7 @@ k_cg_update(T *__restrict__ xv, T *__restrict__ r, const T *__restrict__ d_even,
             const T *__restrict__ Ad, size_t n, const CgScalars *sc, double *partial,
             const CgLoop *__restrict__ loop, const T *__restrict__ d_odd)
 {
+    after_previous();
     T *__restrict__ x = loop ? static_cast<T *>(loop->x) : xv;
     const T *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
     const T alpha = (T)sc->alpha;
@@ -681,6 +693,7 @@ k_cg_update_f4(float4 *__restrict__ xv0, float4 *__restrict__ r, const float4 *_
                const float4 *__restrict__ Ad, size_t n4, const CgScalars *sc, double *partial,
                const CgLoop *__restrict__ loop, const float4 *__restrict__ d_odd)
 {
+    after_previous();
     float4 *__restrict__ x = loop ? static_cast<float4 *>(loop->x) : xv0;
     const float4 *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
     const float alpha = (float)sc->alpha;
@@ -715,14 +728,14 @@ int launch_cg_update(T *x, T *r, const T *d, const T *Ad, size_t n, const CgScal
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
         if (vec4_ok(n, x, r, d, Ad) && vec4_ok(n, d_odd)) {
-            k_cg_update_f4<<<g, kBlock, 0, s>>>(
-                reinterpret_cast<float4 *>(x), reinterpret_cast<float4 *>(r),
-                reinterpret_cast<const float4 *>(d), reinterpret_cast<const float4 *>(Ad), n / 4,
-                sc, partial, loop, reinterpret_cast<const float4 *>(d_odd));
+            launch_after(k_cg_update_f4, g, kBlock, 0, s, reinterpret_cast<float4 *>(x),
+                         reinterpret_cast<float4 *>(r), reinterpret_cast<const float4 *>(d),
+                         reinterpret_cast<const float4 *>(Ad), n / 4, sc, partial, loop,
+                         reinterpret_cast<const float4 *>(d_odd));
             return g;
         }
     }
-    k_cg_update<T><<<g, kBlock, 0, s>>>(x, r, d, Ad, n, sc, partial, loop, d_odd);
+    launch_after(k_cg_update<T>, g, kBlock, 0, s, x, r, d, Ad, n, sc, partial, loop, d_odd);
     return g;
 }
 
@@ -731,6 +744,7 @@ __global__ void __launch_bounds__(kBlock)
 k_cg_direction(const T *__restrict__ z, const T *din, T *dout, size_t n, const CgScalars *sc,
                const CgLoop *__restrict__ loop)
 {
+    after_previous();
     if (loop && loop->its == 0) din = z;
     const T beta = BZ ? T(0) : (T)sc->beta;
 #pragma unroll 4
@@ -744,6 +758,7 @@ __global__ void __launch_bounds__(kBlock)
 k_cg_direction_f4(const float4 *__restrict__ z, const float4 *din, float4 *dout, size_t n4,
                   const CgScalars *sc, const CgLoop *__restrict__ loop)
 {
+    after_previous();
     if (loop && loop->its == 0) din = z;
     const float beta = BZ ? 0.f : (float)sc->beta;
 #pragma unroll 2
@@ -770,13 +785,16 @@ cudaError_t launch_cg_direction(const T *z, const T *d_in, T *d_out, size_t n, c
             const float4 *z4 = reinterpret_cast<const float4 *>(z);
             const float4 *di = reinterpret_cast<const float4 *>(d_in);
             float4 *dw = reinterpret_cast<float4 *>(d_out);
-            if (beta_zero) k_cg_direction_f4<true><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
-            else k_cg_direction_f4<false><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
+            if (beta_zero) launch_after(k_cg_direction_f4<true>, g, kBlock, 0, s, z4, di, dw, n / 4,
+                                        sc, loop);
+            else launch_after(k_cg_direction_f4<false>, g, kBlock, 0, s, z4, di, dw, n / 4, sc,
+                              loop);
             return cudaGetLastError();
         }
     }
-    if (beta_zero) k_cg_direction<T, true><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
-    else k_cg_direction<T, false><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
+    if (beta_zero) launch_after(k_cg_direction<T, true>, g, kBlock, 0, s, z, d_in, d_out, n, sc,
+                                loop);
+    else launch_after(k_cg_direction<T, false>, g, kBlock, 0, s, z, d_in, d_out, n, sc, loop);
     return cudaGetLastError();
 }
 
@@ -911,6 +929,7 @@ __global__ void __launch_bounds__(1024)
 k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op, CgLoop *loop,
                 cudaGraphConditionalHandle cond)
 {
+    after_previous();
     __shared__ double ws[32];
     double v = 0;
     for (int c = threadIdx.x; c < n; c += blockDim.x) v += partial[c];
@@ -940,7 +959,7 @@ k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op
 cudaError_t launch_loop_finalize(const double *partial, int n, CgScalars *sc, int op,
                                  CgLoop *loop, cudaGraphConditionalHandle cond, cudaStream_t s)
 {
-    k_loop_finalize<<<1, 1024, 0, s>>>(partial, n, sc, op, loop, cond);
+    launch_after(k_loop_finalize, 1, 1024, 0, s, partial, n, sc, op, loop, cond);
     return cudaGetLastError();
 }
 

@@ -61,6 +61,7 @@ k_stencil_quad(StencilView V, const double *__restrict__ b, const double *__rest
                void *__restrict__ yout, double scale, int kz, double *__restrict__ partial,
                const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     const int nlon = V.nlon, nlat = V.nlat, nz = V.nz, half = nlon / 2;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -215,17 +216,17 @@ int launch_view(const StencilView &V, int mode, const double *b, const double *x
     if (!quad_fits(V, {V.h, V.e, V.n, V.u, V.w, V.s, V.d, b, x, y}, g)) return -1;
     const dim3 grid(g.gx, g.gy);
     if (mode && partial)
-        k_stencil_quad<SYM, true, true, false, false, false>
-            <<<grid, kBlock, 0, s>>>(V, b, x, y, 1.0, g.kz, partial, flag);
+        launch_after(k_stencil_quad<SYM, true, true, false, false, false>, grid, kBlock, 0, s, V, b,
+                     x, y, 1.0, g.kz, partial, flag);
     else if (mode)
-        k_stencil_quad<SYM, true, false, false, false, false>
-            <<<grid, kBlock, 0, s>>>(V, b, x, y, 1.0, g.kz, nullptr, flag);
+        launch_after(k_stencil_quad<SYM, true, false, false, false, false>, grid, kBlock, 0, s, V,
+                     b, x, y, 1.0, g.kz, nullptr, flag);
     else if (partial)
-        k_stencil_quad<SYM, false, true, false, false, false>
-            <<<grid, kBlock, 0, s>>>(V, b, x, y, 1.0, g.kz, partial, flag);
+        launch_after(k_stencil_quad<SYM, false, true, false, false, false>, grid, kBlock, 0, s, V,
+                     b, x, y, 1.0, g.kz, partial, flag);
     else
-        k_stencil_quad<SYM, false, false, false, false, false>
-            <<<grid, kBlock, 0, s>>>(V, b, x, y, 1.0, g.kz, nullptr, flag);
+        launch_after(k_stencil_quad<SYM, false, false, false, false, false>, grid, kBlock, 0, s, V,
+                     b, x, y, 1.0, g.kz, nullptr, flag);
     return g.gx * g.gy;
 }
 
@@ -263,11 +264,11 @@ int launch_residual_cast_quad(const LevelDev<double> &L, const double *b, const 
     if (!quad_fits(V, {V.h, V.e, V.n, V.u, b, x, r32}, g)) return -1;
     const dim3 grid(g.gx, g.gy);
     if (narrow)
-        k_stencil_quad<true, true, true, true, true, true>
-            <<<grid, kBlock, 0, s>>>(V, b, x, r32, inv_scale, g.kz, partial, nullptr);
+        launch_after(k_stencil_quad<true, true, true, true, true, true>, grid, kBlock, 0, s, V, b,
+                     x, r32, inv_scale, g.kz, partial, nullptr);
     else
-        k_stencil_quad<true, true, true, true, false, true>
-            <<<grid, kBlock, 0, s>>>(V, b, x, r32, inv_scale, g.kz, partial, nullptr);
+        launch_after(k_stencil_quad<true, true, true, true, false, true>, grid, kBlock, 0, s, V, b,
+                     x, r32, inv_scale, g.kz, partial, nullptr);
     return g.gx * g.gy;
 }
 

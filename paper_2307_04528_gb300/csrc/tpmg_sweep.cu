@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
 k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
         T omega, double *__restrict__ partial, const int *__restrict__ flag)
 {
+    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int tiles = (L.nlon * L.nlat + QL * CV - 1) / (QL * CV);
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
 k_sweep_cheb(LevelDev<T> L, const T *b, const T *__restrict__ uin,
              T *__restrict__ uout, ChebStep<T> ch)
 {
+    after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
     const int tiles = (L.nlon * L.nlat + QL * CV - 1) / (QL * CV);
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
@@ -139,25 +141,26 @@ int go(const Level &L, const Sweep<T> &a)
     const cudaStream_t s = a.s;
     const int *flag = a.flag;
     if (!uin)
-        kernel_of<T, S, false, false, Level>()<<<grid, threads,
-                                                 smem_of<T, S, false, Level>(threads), s>>>(
-            L, b, uin, uout, (T)omega, partial, flag);
+        launch_after(kernel_of<T, S, false, false, Level>(), grid, threads,
+                     smem_of<T, S, false, Level>(threads), s, L, b, uin, uout, (T)omega, partial,
+                     flag);
     if constexpr (S::GUESS && !kDirected<Level>) {
         if (a.ch) {
-            k_sweep_cheb<T, S::CV, S::LZ, S::QL, S::MAXT, S::MINB>
-                <<<grid, threads, smem_of<T, S, false>(threads), s>>>(L, b, uin, uout, *a.ch);
+            launch_after(k_sweep_cheb<T, S::CV, S::LZ, S::QL, S::MAXT, S::MINB>, grid, threads,
+                         smem_of<T, S, false>(threads), s, L, b, uin, uout, *a.ch);
             return grid;
         }
     }
     if constexpr (S::GUESS) {
         if constexpr (!kDirected<Level>)
             if (uin && partial)
-                kernel_of<T, S, true, true>()<<<grid, threads, smem_of<T, S, true>(threads), s>>>(
-                    L, b, uin, uout, (T)omega, partial, flag);
+                launch_after(kernel_of<T, S, true, true>(), grid, threads,
+                             smem_of<T, S, true>(threads), s, L, b, uin, uout, (T)omega, partial,
+                             flag);
         if (uin && !partial)
-            kernel_of<T, S, true, false, Level>()<<<grid, threads,
-                                                    smem_of<T, S, false, Level>(threads), s>>>(
-                L, b, uin, uout, (T)omega, partial, flag);
+            launch_after(kernel_of<T, S, true, false, Level>(), grid, threads,
+                         smem_of<T, S, false, Level>(threads), s, L, b, uin, uout, (T)omega,
+                         partial, flag);
     }
     return grid;
 }
@@ -189,6 +192,7 @@ __global__ void __launch_bounds__(kClusterThreads<T, LZ, Level>, 1)
 k_coarse_cluster(Level L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
                  int R)
 {
+    after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
     coarse_cluster<T, LZ, Level>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
 }
@@ -323,12 +327,13 @@ static cudaError_t coarse_solve(const Level &L, const T *b, T *out, double omega
     cfg.blockDim = dim3(c.threads);
     cfg.dynamicSmemBytes = c.values * sizeof(T);
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = c.blocks;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1] = after_attribute();
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = capturing(s) ? 1 : 2;
     const T om = (T)omega;
     auto run = [&](auto lz) {
         return cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, decltype(lz)::value, Level>, L, b, out,
