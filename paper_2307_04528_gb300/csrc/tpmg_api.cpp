@@ -1094,6 +1094,14 @@ static bool cg_loop_ready(mg_handle *H, const T *x)
     cudaGraph_t captured = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(s, &captured);
     if (st != MG_OK || ec != cudaSuccess) return give_up();
+    if constexpr (sizeof(T) == 4) {
+        if (cudaStreamBeginCaptureToGraph(s, g.graph, &node, nullptr, 1,
+                                          cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+            return give_up();
+        const cudaError_t ef = launch_cg_flush(cg.d0, n, H->sc, H->cg_loop, s);
+        const cudaError_t eg = cudaStreamEndCapture(s, &captured);
+        if (ef != cudaSuccess || eg != cudaSuccess) return give_up();
+    }
     if (cudaGraphInstantiate(&g.exec, g.graph, 0) != cudaSuccess) {
         g.exec = nullptr;
         return give_up();
@@ -1173,14 +1181,15 @@ static int solve_impl(mg_handle *H, const T *b, T *x, double tol, int maxit, int
             while (!over) {
                 const int from = st.its;
                 st.limit = std::min(left, from + kLoopHist);
-                CU(cudaMemcpyAsync(H->cg_loop, &st, offsetof(CgLoop, hist),
+                CU(cudaMemcpyAsync(H->cg_loop, &st, offsetof(CgLoop, alpha_even),
                                    cudaMemcpyHostToDevice, s));
                 CU(cudaGraphLaunch(H->loop[P].exec, s));
                 CU(cudaMemcpyAsync(&st, H->cg_loop, sizeof st, cudaMemcpyDeviceToHost, s));
                 CU(cudaStreamSynchronize(s));
                 if (st.its <= from || st.its > st.limit)
                     return fail(MG_ERR_CUDA, "the device-side iteration did not advance");
-                g_launches.fetch_add(H->loop[P].kernels * (unsigned long long)(st.its - from),
+                g_launches.fetch_add(H->loop[P].kernels * (unsigned long long)(st.its - from) +
+                                         (P == MG_PREC_FP32),
                                      std::memory_order_relaxed);
                 for (int i = from; i < st.its; ++i) {
                     ++its;

@@ -97,6 +97,7 @@ struct CgLoop {
     double stop, grow;  // the loop ends at ||r|| <= stop or ||r||^2 > grow
     int its, limit;     // iterations done, and where this launch ends
     void *x;
+    double alpha_even;  // the last even iteration's alpha
     double hist[kLoopHist];  // ||r||^2 of iteration i in hist[i % kLoopHist]
 };
 
@@ -245,6 +246,9 @@ int launch_cg_update(T *x, T *r, const T *d, const T *Ad, size_t n, const CgScal
                      double *partial, cudaStream_t s, const CgLoop *loop = nullptr,
                      const T *d_odd = nullptr);
 
+// After an FP32 loop: x += alpha d of a last even iteration.
+cudaError_t launch_cg_flush(const float *d, size_t n, const CgScalars *sc, const CgLoop *loop,
+                            cudaStream_t s);
 // d_out = z + beta d_in (beta from sc->beta; beta_zero: d_out = z).  loop: d_in
 // is not read in its iteration 0 (z stands in for it, beta = 0).
 template <typename T>

