@@ -221,8 +221,8 @@ def run_reference(args):
 # (reads + writes of distinct arrays; horizontal neighbours counted once)
 KERNEL_WORDS = {
     # (kind, prec): (name, words per cell)
-    (0, 1): ("smooth fp32 (+ <r, z>)", 8),            # u b tx ty tz m dq -> u
-    (1, 1): ("smooth fp32 zero guess", 5),            # b tz m dq -> u
+    (0, 1): ("smooth fp32 (+ <r, z>)", 7),            # u b tx ty m dq -> u
+    (1, 1): ("smooth fp32 zero guess", 4),            # b m dq -> u
     (2, 1): ("residual + restriction fp32", 6),       # u b tx ty tz h -> b_c (+ coarse write;
                                                       # u b tx ty after a sweep from zero)
     (3, 1): ("direction update + apply fp32", 8),     # z d tx ty tz h -> d q
@@ -234,13 +234,13 @@ KERNEL_WORDS = {
 }
 
 
-# DRAM bytes per fine cell of one k_smooth_dot<float> launch (ncu capture at
-# 512x384x70: 397.3 MB read + 34.8 MB written for 13,762,560 cells)
-SMOOTH_DOT_DRAM_BYTES_PER_CELL = (397.266944e6 + 34.799616e6) / (512 * 384 * 70)
+# DRAM bytes per fine cell of one launch of the FP32 sweep with <r, z> (ncu
+# capture at 512x384x70: 330.3 MB read + 40.7 MB written for 13,762,560 cells)
+SMOOTH_DOT_DRAM_BYTES_PER_CELL = (330.349056e6 + 40.736e6) / (512 * 384 * 70)
 # DRAM bytes per fine cell of one k_resid_restrict<float> launch in its
-# presmoothing form on the finest level (ncu capture at 512x384x70: 232.6 MB
-# read + 16.1 MB written for 13,762,560 fine cells)
-RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.561408e6 + 16.097536e6) / (512 * 384 * 70)
+# presmoothing form on the finest level (ncu capture at 512x384x70: 232.5 MB
+# read + 13.0 MB written for 13,762,560 fine cells)
+RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.47872e6 + 13.043456e6) / (512 * 384 * 70)
 
 
 def kernel_table(H, L, N):
@@ -428,12 +428,12 @@ def run_ours(args):
 
     peak, peak_kind = load_peaks()
     # the kernel with the largest share of the mixed solve: the V-cycle's last
-    # fine-level sweep with <r, z> fused (reads u, b, tx, ty, tz, m, dq; writes
-    # u: 8 x 4 B per cell)
-    sm_bytes = 32 * N
+    # fine-level sweep with <r, z> fused (reads u, b, tx, ty, m, dq; writes u:
+    # 7 x 4 B per cell)
+    sm_bytes = 28 * N
     sm_avg_ms = sm_ms / max(sm_calls, 1)
     achieved = sm_bytes / (sm_avg_ms * 1e-3) / 1e9 if sm_calls else None
-    roofline = {"kernel": "k_smooth_dot<float>: fine-level block-Jacobi sweep of Eq. (1) "
+    roofline = {"kernel": "k_sweep<float>: fine-level block-Jacobi sweep of Eq. (1) "
                           "(last sweep of the V-cycle, CG inner product fused)", "bound": "hbm",
                 "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,

@@ -373,8 +373,8 @@ __device__ __forceinline__ void stencil_cell(const LevelDev<T> &L, const T *__re
 // pivots p_k = q_k + t_k, on the setup factors m_k = 1/p_k and dq_k = q_k/p_k:
 //   forward   y_k = (v_k + t_{k-1} y_{k-1}) m_k,  v_k = b_k + sum_h T u_in,nb
 //   backward  x_k = x_{k+1} + (y_k - dq_k x_{k+1})
-// This is the sweep on a non-zero guess; sweeps from a zero guess are
-// smooth_staged (large levels) and smooth_warp_column (small FP32 levels).
+// This is the column walk on a non-zero guess; from a zero guess it is
+// smooth_staged.  Most levels sweep by segments instead (sweep_tile).
 // The forward values y wait in shared memory for the backward sweep
 // (blockDim x nz values).
 //
@@ -654,8 +654,7 @@ __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], 
 // lane's own layers are consecutive words (bank-conflict free for an odd
 // layers-per-lane count).  The level is staged once from its [layer][column]
 // arrays and the result written back once; the sweeps in between touch no
-// global memory.  Same arithmetic, same order as the sweeps from global
-// memory (smooth_warp_column).  Called by every thread of the block; sh:
+// global memory.  Called by every thread of the block; sh:
 // kCoarseShArrays * ncol * nz values of dynamic shared memory.
 constexpr int kCoarseShArrays = 8;
 

@@ -1,7 +1,10 @@
-// CUDA kernels of the tensor-product multigrid (sm_103a).
+// CUDA kernels of the tensor-product multigrid (sm_103a): the column walks,
+// transfers, vector kernels and setup.  (The segmented sweeps, the FP64
+// stencils by 2 x 2 columns and the FP32 direction update + apply by quads,
+// which take most levels, have files of their own.)
 //
-// Data layout: every field is [nz][nlat][nlon], longitude fastest.  One
-// thread owns one vertical column (i, j) and walks k, so at every k the
+// Data layout: every field is [nz][nlat][nlon], longitude fastest.  In the
+// column walks one thread owns one vertical column (i, j) and walks k, so at every k the
 // threads of a warp touch consecutive addresses (coalesced, one 128-byte
 // line per warp per array in FP32, two in FP64).  Horizontal neighbours
 // (i +- 1, j +- 1) are re-reads of lines that neighbouring threads of the
@@ -381,7 +384,10 @@ k_resid_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ b, const T *__r
                                 (band0 + (int)blockIdx.z) * band, blockIdx.y, om1, band);
 }
 
-// The same over a directed level (two more arrays, two more pairs in flight).
+// The same over a directed level: two more arrays, so two more pairs in flight
+// per row and 8 blocks per SM (64 registers, no spills).  Against the plain
+// column walk and a restriction of its own, seven levels of 512 x 384 x 70 in
+// FP32: 74 -> 21 us on average.
 template <typename T>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 8 : 0)
 k_ns_presmooth_restrict(NsView<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
