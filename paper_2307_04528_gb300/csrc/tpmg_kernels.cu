@@ -980,6 +980,10 @@ k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op
 {
     after_previous();
     __shared__ double ws[32];
+    // the scalars of the last step, in flight while the partials are summed
+    // (loaded after the sum: 64 x 32 x 16 in FP64 1.944 ms a solve instead of 1.925)
+    const double rz = sc->rz, stop = loop->stop, grow = loop->grow;
+    const int it = loop->its, limit = loop->limit;
     double v = 0;
     for (int c = threadIdx.x; c < n; c += blockDim.x) v += partial[c];
     v = warp_reduce<0>(v);
@@ -990,18 +994,19 @@ k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op
     v = warp_reduce<0>(lane < (int)(blockDim.x >> 5) ? ws[lane] : 0.0);
     if (lane != 0) return;
     if (op == LOOP_RZ) {
-        sc->beta = loop->its > 0 && sc->rz != 0.0 ? v / sc->rz : 0.0;
+        sc->beta = it > 0 && rz != 0.0 ? v / rz : 0.0;
         sc->rz = v;
     } else if (op == LOOP_ALPHA) {
         sc->dAd = v;
-        sc->alpha = v != 0.0 ? sc->rz / v : 0.0;
-        if (!(loop->its & 1)) loop->alpha_even = sc->alpha;
+        const double alpha = v != 0.0 ? rz / v : 0.0;
+        sc->alpha = alpha;
+        if (!(it & 1)) loop->alpha_even = alpha;
     } else {
         sc->rr = v;
-        loop->hist[loop->its % kLoopHist] = v;
-        const int its = ++loop->its;
+        loop->hist[it % kLoopHist] = v;
+        loop->its = it + 1;
         // a NaN compares false and ends the loop, as does an infinity
-        const bool more = sqrt(v) > loop->stop && v <= loop->grow && its < loop->limit;
+        const bool more = sqrt(v) > stop && v <= grow && it + 1 < limit;
         cudaGraphSetConditional(cond, more ? 1u : 0u);
     }
 }
