@@ -293,10 +293,11 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
         const T *tw = west_of(L) + (i == 0 ? nlon - 1 : -1);
         const T *ts = south_of(L) - (hasS ? nlon : 0);
         off = first;
-        // CHEB: t_z and d of the layer below the segment, d of the one above
+        // CHEB: t_z and d of the layer below the segment, d of the one above (a
+        // segment past the top has none: with one layer there is none to read)
         X tzd = splat<T, CV>(T(0)), ud = tzd, ua = tzd;
         if constexpr (CHEB) {
-            const unsigned dn = k0 > 0 ? plane : 0u;
+            const unsigned dn = k0 > 0 && k0 < nz ? plane : 0u;
             tzd = ldv<T, CV>(up_of(L), first - dn);
             ud = ldv<T, CV>(uin, first - dn);
             ua = ldv<T, CV>(uin, first + (k0 + LZ < nz ? LZ * plane : 0u));
