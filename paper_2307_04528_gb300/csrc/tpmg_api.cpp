@@ -711,21 +711,24 @@ static int coarse_chebyshev(mg_handle *H, int l, const LevelDev<T> &D, const T *
     const int m = H->p.coarse_iters;
     // One launch per step where the segmented sweeps take the level: the
     // residual r - H d, the column solve and the updates of d and x in one pass
-    // over two copies of d (64 x 98 x 70 in FP32: 4.7 us a step, against
+    // over two copies of d and of r (64 x 98 x 70 in FP32: 4.7 us a step, against
     // 10.1 as three kernels).  The terms and their order are the separate
     // kernels'.  (Carrying x instead of r, z = H_z^{-1}(b + the horizontal
     // couplings of x) - x, took 4.4 us, but the difference lost a factor of 4
     // to 12 in accuracy.)
     if (m > 1 && cheb_sweep_fits<T>(D, b, d, z, r, out)) {
         T *dn = z;
+        const T *rk = b;
         double rho = 1.0 / sigma;
         KRUN(K_SMOOTH0, l, P, launch_smooth<T>(D, b, nullptr, d, 1.0 / theta, s));
         for (int k = 0; k + 1 < m; ++k) {
             const double rho_new = 1.0 / (2.0 * sigma - rho);
+            T *rn = (rk == r) ? r2 : r;
             KRUN(K_SMOOTH, l, P,
-                 launch_cheb_sweep<T>(D, k == 0 ? b : r, d, dn, r, out, rho_new * rho,
+                 launch_cheb_sweep<T>(D, rk, d, dn, rn, out, rho_new * rho,
                                       2.0 * rho_new / delta, k == 0, k + 2 == m, s));
             std::swap(d, dn);
+            rk = rn;
             rho = rho_new;
         }
         return MG_OK;

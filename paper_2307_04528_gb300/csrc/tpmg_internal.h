@@ -298,7 +298,7 @@ cudaError_t launch_scale(T *x, double f, size_t n, cudaStream_t s);
 int launch_hz_ratio(const LevelDev<double> &L, double *partial, cudaStream_t s);
 // A Chebyshev step in one pass: r_out = r - H d, x += d (first: x = d), d_out =
 // c1 d + c2 H_z^{-1} r_out (last: x takes it too), where the segmented sweeps
-// take the level and the buffers (cheb_sweep_fits).  r_out may be r.
+// take the level and the buffers (cheb_sweep_fits).  No output is an input.
 template <typename T>
 bool cheb_sweep_fits(const LevelDev<T> &L, const T *r, const T *d, T *d_out, T *r_out, T *x);
 template <typename T>

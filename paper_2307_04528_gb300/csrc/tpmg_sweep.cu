@@ -38,7 +38,7 @@ k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restri
 // A Chebyshev step of the coarsest-level solve as one sweep (launch_cheb_sweep).
 template <typename T, int CV, int LZ, int QL, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_sweep_cheb(LevelDev<T> L, const T *b, const T *__restrict__ uin,
+k_sweep_cheb(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin,
              T *__restrict__ uout, ChebStep<T> ch)
 {
     after_previous();

@@ -238,8 +238,7 @@ __device__ __forceinline__ Vals<T, CV> carry(const Vals<T, CV> &ndq, const Vals<
 
 // A Chebyshev step instead of a sweep: with b the residual and u_in the step d,
 // r_out = b - H d, x += d (first: x = d) and u_out = c1 d + c2 H_z^{-1} r_out;
-// last: x takes the new step too.  Each cell of r_out (may be b) and x is its
-// own thread's.
+// last: x takes the new step too.  Each cell of x is its own thread's.
 template <typename T>
 struct ChebStep {
     T *r_out, *x;
@@ -279,7 +278,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
     for (int c = 0; c < LZ; ++c) {
         m[c] = ldv<T, CV>(L.m, off);
         dq[c] = ldv<T, CV>(L.dq, off);
-        v[c] = CHEB ? ldv_own<T, CV>(b, off) : ldv<T, CV>(b, off);
+        v[c] = ldv<T, CV>(b, off);
         if (GUESS) uc[c] = ldv<T, CV>(uin, off);
         if constexpr (NS) f[c] = ldv<T, CV>(down_of(L), off);
         off += k0 + c + 1 < nz ? plane : 0u;

@@ -31,3 +31,15 @@ def check(shape, steps):
                          ids=lambda s: "x".join(map(str, s)))
 def test_one_layer(shape):
     check(shape, 5)
+
+
+# The shapes of a step, whose residual has two copies, written in turn: pairs and
+# 9-layer segments of single columns, quads in segments of 9 and 5, ragged tiles and
+# last segments, single columns, more than 72 layers, and sizes that take the
+# separate kernels.
+@pytest.mark.parametrize("steps", [2, 3, 7, 24])
+@pytest.mark.parametrize("shape", [(64, 34, 37), (64, 98, 70), (132, 64, 10), (128, 66, 37),
+                                   (65, 34, 12), (6, 4, 100), (10, 6, 2), (129, 64, 9)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_steps(shape, steps):
+    check(shape, steps)
