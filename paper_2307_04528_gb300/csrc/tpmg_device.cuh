@@ -992,8 +992,8 @@ __device__ __forceinline__ void restrict_layers(const LevelDev<T> &F, const Link
 // the prolongation and correction, the row links read once.
 template <typename T>
 __device__ __forceinline__ void prolong_layers(const LevelDev<T> &F, const LinkDev &K,
-                                               const T *__restrict__ ec, T *__restrict__ u, int t,
-                                               int k0, int k1)
+                                               const T *ec, T *__restrict__ u, int t, int k0,
+                                               int k1)
 {
     const int nf = F.nlon, nc = nf / 2;
     const int npair = nc * F.nlat;
@@ -1012,14 +1012,14 @@ __device__ __forceinline__ void prolong_layers(const LevelDev<T> &F, const LinkD
     for (int k = k0; k < k1; ++k) {
         const T *ek = ec + (size_t)k * plane_c;
         const T *ea = ek + oa;
-        const T ca = __ldg(ea + I);
-        T a0 = wa * fma(q3, ca, q1 * __ldg(ea + Im));
-        T a1 = wa * fma(q3, ca, q1 * __ldg(ea + Ip));
+        const T ca = ea[I];
+        T a0 = wa * fma(q3, ca, q1 * ea[Im]);
+        T a1 = wa * fma(q3, ca, q1 * ea[Ip]);
         if (Jb >= 0) {
             const T *eb = ek + ob;
-            const T cb = __ldg(eb + I);
-            a0 = fma(wb, fma(q3, cb, q1 * __ldg(eb + Im)), a0);
-            a1 = fma(wb, fma(q3, cb, q1 * __ldg(eb + Ip)), a1);
+            const T cb = eb[I];
+            a0 = fma(wb, fma(q3, cb, q1 * eb[Im]), a0);
+            a1 = fma(wb, fma(q3, cb, q1 * eb[Ip]), a1);
         }
         T *uk = u + (size_t)k * plane_f + of;
         uk[0] += a0;
@@ -1043,6 +1043,14 @@ template <typename T>
 __device__ __forceinline__ typename Pair<T>::type ld_pair(const T *p)
 {
     return __ldg(reinterpret_cast<const typename Pair<T>::type *>(p));
+}
+
+// The same of a vector that the kernel before this one may have written
+// (after_previous).
+template <typename T>
+__device__ __forceinline__ typename Pair<T>::type ld_pair_of(const T *p)
+{
+    return *reinterpret_cast<const typename Pair<T>::type *>(p);
 }
 
 // a_d += w v of three open sums, d warp-uniform.  FP64: one operation on the
@@ -1093,8 +1101,7 @@ __device__ __forceinline__ void add_open(T w, T v, int d, T &a0, T &a1, T &a2)
 // south are arrays of their own.
 template <typename T, bool PRE = false, typename Level = LevelDev<T>>
 __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDev &K,
-                                                    const T *__restrict__ b,
-                                                    const T *__restrict__ u, T *__restrict__ bc,
+                                                    const T *b, const T *u, T *__restrict__ bc,
                                                     int warp, int lane, int Jb, int k,
                                                     T om1 = T(0), int band = kRRBand)
 {
@@ -1124,9 +1131,9 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
     T a0 = 0, a1 = 0, a2 = 0;                              // rows Jlo, Jlo + 1, Jlo + 2
     P2 zero;
     zero.x = zero.y = T(0);
-    P2 Us = jfirst > 0 ? ld_pair(uk + (size_t)(jfirst - 1) * nf) : zero;
+    P2 Us = jfirst > 0 ? ld_pair_of(uk + (size_t)(jfirst - 1) * nf) : zero;
     P2 Tys = jfirst > 0 ? ld_pair(sk + (size_t)(jfirst - 1) * nf) : zero;
-    P2 Uc = ld_pair(uk + (size_t)jfirst * nf);
+    P2 Uc = ld_pair_of(uk + (size_t)jfirst * nf);
     // The PRE form has little arithmetic per row to cover its loads, so it
     // issues the next row's loads (u and t_y one row north, b and t_x on the
     // row) before combining this one: two rows in flight per thread (FP64, all
@@ -1136,8 +1143,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
     P2 nUn = zero, nB = zero, nTX = zero, nTYN = zero, nTW = zero, nTS = zero;
     if (kAhead) {
         const size_t o0 = (size_t)jfirst * nf;
-        nUn = jfirst + 1 < nlat ? ld_pair(uk + o0 + nf) : zero;
-        nB = ld_pair(bk + o0);
+        nUn = jfirst + 1 < nlat ? ld_pair_of(uk + o0 + nf) : zero;
+        nB = ld_pair_of(bk + o0);
         nTX = ld_pair(txk + o0);
         nTYN = jfirst + 1 < nlat ? ld_pair(tyk + o0) : zero;
         if (NS) {
@@ -1162,8 +1169,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
             if (j < jlast) {
                 const size_t o1 = oj + nf;
                 const bool n1 = j + 2 < nlat;
-                nUn = n1 ? ld_pair(uk + o1 + nf) : zero;
-                nB = ld_pair(bk + o1);
+                nUn = n1 ? ld_pair_of(uk + o1 + nf) : zero;
+                nB = ld_pair_of(bk + o1);
                 nTX = ld_pair(txk + o1);
                 nTYN = n1 ? ld_pair(tyk + o1) : zero;
                 if (NS) {
@@ -1172,8 +1179,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
                 }
             }
         } else {
-            Un = hasN ? ld_pair(uk + oj + nf) : zero;
-            B = ld_pair(bk + oj);
+            Un = hasN ? ld_pair_of(uk + oj + nf) : zero;
+            B = ld_pair_of(bk + oj);
             TX = ld_pair(txk + oj);
             TYN = hasN ? ld_pair(tyk + oj) : zero;
             if (NS) {
@@ -1203,8 +1210,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
         } else {
             const P2 Hh = ld_pair(hk + oj), TZ = ld_pair(tzk + oj);
             const P2 TZD = dn ? ld_pair(tzd + oj) : zero;
-            const P2 UU = up ? ld_pair(uu + oj) : zero;
-            const P2 UD = dn ? ld_pair(ud + oj) : zero;
+            const P2 UU = up ? ld_pair_of(uu + oj) : zero;
+            const P2 UD = dn ? ld_pair_of(ud + oj) : zero;
             T v0 = Hh.x * Uc.x;
             v0 = fma(TX.x, Uc.x - Uc.y, v0);
             v0 = fma(txw, Uc.x - uw, v0);

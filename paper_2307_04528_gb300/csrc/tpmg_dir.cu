@@ -48,7 +48,6 @@ k_dir_quad(LevelDev<float> L, const float *__restrict__ z, const float *__restri
            int kz, double *__restrict__ partial, const int *__restrict__ flag,
            const CgLoop *__restrict__ loop)
 {
-    after_previous();
     if (flag && !*flag) return;
     const bool odd = loop && (loop->its & 1);
     const float *__restrict__ dold = loop && loop->its == 0 ? z : odd ? d_to : d_even;
@@ -180,11 +179,11 @@ int launch_dir_quad(const LevelDev<float> &L, const float *z, const float *d_old
     if (blocks < 0) return -1;
     const Shape g = shape_of(L);
     if (d_old)
-        launch_after(k_dir_quad<false>, dim3(g.gx, g.gy), kBlock, 0, s, L, z, d_old, sc, d_new, q,
-                     g.kz, partial, flag, loop);
+        k_dir_quad<false><<<dim3(g.gx, g.gy), kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, g.kz,
+                                                              partial, flag, loop);
     else
-        launch_after(k_dir_quad<true>, dim3(g.gx, g.gy), kBlock, 0, s, L, z, d_old, sc, d_new, q,
-                     g.kz, partial, flag, loop);
+        k_dir_quad<true><<<dim3(g.gx, g.gy), kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, g.kz,
+                                                             partial, flag, loop);
     return blocks;
 }
 

@@ -49,7 +49,11 @@ struct CgScalars {
 // 1024 x 768 x 70 1.085 -> 1.014 ms, those of H and H^T at 512 x 384 x 70 and
 // two applies 1.62 -> 1.50).  Not under capture: in the body of the device-side
 // loop such edges cost more than plain ones (24 Chebyshev steps per coarse solve:
-// 39.9 -> 40.9 ms; 256 x 128 x 32 in FP64: 12.6 -> 13.2).
+// 39.9 -> 40.9 ms; 256 x 128 x 32 in FP64: 12.6 -> 13.2).  Such a kernel lives
+// while the one before it still writes, so it reads vectors by ordinary loads:
+// the read-only path (__ldg, or a const __restrict__ parameter) is for data that
+// nothing writes during the kernel's life, here the coefficients, factors and
+// links, which the setup leaves complete.
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_previous()
 {

@@ -54,7 +54,6 @@ k_dir_apply(LevelDev<T> L, const T *__restrict__ z, const T *__restrict__ d_even
             double *__restrict__ partial, const int *__restrict__ flag,
             const CgLoop *__restrict__ loop)
 {
-    after_previous();
     if (flag && !*flag) return;
     const bool odd = loop && (loop->its & 1);
     const T *__restrict__ dold = loop && loop->its == 0 ? z : odd ? d_to : d_even;
@@ -77,11 +76,11 @@ int launch_dir_apply(const LevelDev<T> &L, const T *z, const T *d_old, const CgS
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (d_old == nullptr)
-        launch_after(k_dir_apply<T, true>, grid, kBlock, 0, s, L, z, d_old, sc, d_new, q, partial,
-                     flag, loop);
+        k_dir_apply<T, true><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
+                                                     loop);
     else
-        launch_after(k_dir_apply<T, false>, grid, kBlock, 0, s, L, z, d_old, sc, d_new, q, partial,
-                     flag, loop);
+        k_dir_apply<T, false><<<grid, kBlock, 0, s>>>(L, z, d_old, sc, d_new, q, partial, flag,
+                                                      loop);
     return grid;
 }
 
@@ -212,7 +211,6 @@ __global__ void __launch_bounds__(kBlock)
 k_smooth(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
          T omega, const int *__restrict__ flag)
 {
-    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     smooth_column<T, false, 0, kYOut<T>>(L, b, uin, uout, omega,
@@ -224,7 +222,6 @@ __global__ void __launch_bounds__(kBlock)
 k_smooth0(LevelDev<T> L, const T *__restrict__ b, T *__restrict__ uout, T omega,
           const int *__restrict__ flag)
 {
-    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     smooth_staged<T, true>(L, b, nullptr, uout, omega, blockIdx.x * blockDim.x + threadIdx.x,
@@ -239,7 +236,6 @@ k_smooth_dot(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin,
              T *__restrict__ uout, T omega, double *__restrict__ partial,
              const int *__restrict__ flag)
 {
-    after_previous();
     if (flag && !*flag) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     T acc = 0;
@@ -257,8 +253,7 @@ int launch_smooth_dot(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out,
     const size_t smem = kYOut<T> ? 0 : (size_t)L.nz * kBlock * sizeof(T);
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
-    launch_after(k_smooth_dot<T>, grid, kBlock, smem, s, L, b, u_in, u_out, (T)omega, partial,
-                 flag);
+    k_smooth_dot<T><<<grid, kBlock, smem, s>>>(L, b, u_in, u_out, (T)omega, partial, flag);
     return grid;
 }
 
@@ -291,10 +286,10 @@ cudaError_t launch_smooth_walk(const LevelDev<T> &L, const T *b, const T *u_in, 
     const int grid = (ncol + kBlock - 1) / kBlock;
     if (u_in == nullptr) {
         const size_t smem = ring_smem_bytes<T, true>(L.nz, kBlock);
-        launch_after(k_smooth0<T>, grid, kBlock, smem, s, L, b, u_out, (T)omega, flag);
+        k_smooth0<T><<<grid, kBlock, smem, s>>>(L, b, u_out, (T)omega, flag);
     } else {
         const size_t smem = kYOut<T> ? 0 : (size_t)L.nz * kBlock * sizeof(T);
-        launch_after(k_smooth<T>, grid, kBlock, smem, s, L, b, u_in, u_out, (T)omega, flag);
+        k_smooth<T><<<grid, kBlock, smem, s>>>(L, b, u_in, u_out, (T)omega, flag);
     }
     return cudaGetLastError();
 }
@@ -373,8 +368,8 @@ k_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ r, T *__restrict__ bc
 // is latency-bound, and the extra resident warps outweigh a few spilled bytes.
 template <typename T, bool PRE>
 __global__ void __launch_bounds__(kBlock, (PRE && sizeof(T) == 4) ? 12 : 0)
-k_resid_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
-                 T *__restrict__ bc, T om1, int band0, int band, const int *__restrict__ flag)
+k_resid_restrict(LevelDev<T> F, LinkDev K, const T *b, const T *u, T *__restrict__ bc, T om1,
+                 int band0, int band, const int *flag)
 {
     after_previous();
     if (flag && !*flag) return;
@@ -390,8 +385,8 @@ k_resid_restrict(LevelDev<T> F, LinkDev K, const T *__restrict__ b, const T *__r
 // FP32: 74 -> 21 us on average.
 template <typename T>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 8 : 0)
-k_ns_presmooth_restrict(NsView<T> F, LinkDev K, const T *__restrict__ b, const T *__restrict__ u,
-                        T *__restrict__ bc, T om1, int band0, int band)
+k_ns_presmooth_restrict(NsView<T> F, LinkDev K, const T *b, const T *u, T *__restrict__ bc, T om1,
+                        int band0, int band)
 {
     after_previous();
     const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
@@ -492,8 +487,7 @@ cudaError_t launch_restrict(const LevelDev<T> &F, const LinkDev &K, const T *r, 
 // row serve both.
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_prolong_add(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict__ u, int kz,
-              const int *__restrict__ flag)
+k_prolong_add(LevelDev<T> F, LinkDev K, const T *ec, T *__restrict__ u, int kz, const int *flag)
 {
     after_previous();
     if (flag && !*flag) return;
@@ -510,8 +504,7 @@ k_prolong_add(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict_
 // in FP32 (1536 x 1152 x 70: 0.219 -> 0.184 ms).
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_prolong_quad(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict__ u, int kz,
-               const int *__restrict__ flag)
+k_prolong_quad(LevelDev<T> F, LinkDev K, const T *ec, T *__restrict__ u, int kz, const int *flag)
 {
     after_previous();
     if (flag && !*flag) return;
@@ -534,12 +527,12 @@ k_prolong_quad(LevelDev<T> F, LinkDev K, const T *__restrict__ ec, T *__restrict
     const T three = T(3);
 #pragma unroll 2
     for (int k = k0; k < k1; ++k, ea += plane_c, eb += plane_c, up += plane_f) {
-        const P2 a = ld_pair(ea), b = ld_pair(eb);
+        const P2 a = ld_pair_of(ea), b = ld_pair_of(eb);
         P2 u0 = reinterpret_cast<const P2 *>(up)[0], u1 = reinterpret_cast<const P2 *>(up)[1];
         const T g0 = fma(wb, b.x, wa * a.x), g1 = fma(wb, b.y, wa * a.y);
         T gl = __shfl_up_sync(kAll, g1, 1), gr = __shfl_down_sync(kAll, g0, 1);
-        if (left) gl = fma(wb, __ldg(eb + dl), wa * __ldg(ea + dl));
-        if (right) gr = fma(wb, __ldg(eb + dr), wa * __ldg(ea + dr));
+        if (left) gl = fma(wb, eb[dl], wa * ea[dl]);
+        if (right) gr = fma(wb, eb[dr], wa * ea[dr]);
         u0.x += fma(three, g0, gl);
         u0.y += fma(three, g0, g1);
         u1.x += fma(three, g1, g0);
@@ -601,7 +594,6 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock)
 k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, double *partial)
 {
-    after_previous();
     T acc = 0;
 #pragma unroll 4
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
@@ -624,7 +616,6 @@ static bool vec4_ok(size_t n, const void *a, const void *b = nullptr, const void
 __global__ void __launch_bounds__(kBlock)
 k_dot_f4(const float4 *__restrict__ a, const float4 *__restrict__ b, size_t n4, double *partial)
 {
-    after_previous();
     float acc = 0.f;
 #pragma unroll 2
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n4;
@@ -644,12 +635,12 @@ int launch_dot(const T *a, const T *b, size_t n, double *partial, cudaStream_t s
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
         if (vec4_ok(n, a, b)) {
-            launch_after(k_dot_f4, g, kBlock, 0, s, reinterpret_cast<const float4 *>(a),
-                         reinterpret_cast<const float4 *>(b), n / 4, partial);
+            k_dot_f4<<<g, kBlock, 0, s>>>(reinterpret_cast<const float4 *>(a),
+                                          reinterpret_cast<const float4 *>(b), n / 4, partial);
             return g;
         }
     }
-    launch_after(k_dot<T>, g, kBlock, 0, s, a, b, n, partial);
+    k_dot<T><<<g, kBlock, 0, s>>>(a, b, n, partial);
     return g;
 }
 
@@ -684,7 +675,6 @@ k_cg_update(T *__restrict__ xv, T *__restrict__ r, const T *__restrict__ d_even,
             const T *__restrict__ Ad, size_t n, const CgScalars *sc, double *partial,
             const CgLoop *__restrict__ loop, const T *__restrict__ d_odd)
 {
-    after_previous();
     T *__restrict__ x = loop ? static_cast<T *>(loop->x) : xv;
     const bool pairs = sizeof(T) == 4 && loop && d_odd != d_even, odd = loop && (loop->its & 1);
     const T *__restrict__ d = odd ? d_odd : d_even;
@@ -709,7 +699,6 @@ k_cg_update_f4(float4 *__restrict__ xv0, float4 *__restrict__ r, const float4 *_
                const float4 *__restrict__ Ad, size_t n4, const CgScalars *sc, double *partial,
                const CgLoop *__restrict__ loop, const float4 *__restrict__ d_odd)
 {
-    after_previous();
     float4 *__restrict__ x = loop ? static_cast<float4 *>(loop->x) : xv0;
     const bool odd = loop && (loop->its & 1);
     const float4 *__restrict__ d = odd ? d_odd : d_even;
@@ -754,7 +743,6 @@ __global__ void __launch_bounds__(kBlock)
 k_cg_flush(const float *__restrict__ d, size_t n, const CgScalars *sc,
            const CgLoop *__restrict__ loop)
 {
-    after_previous();
     if (!(loop->its & 1)) return;
     float *__restrict__ x = static_cast<float *>(loop->x);
     const float alpha = (float)sc->alpha;
@@ -767,7 +755,8 @@ k_cg_flush(const float *__restrict__ d, size_t n, const CgScalars *sc,
 cudaError_t launch_cg_flush(const float *d, size_t n, const CgScalars *sc, const CgLoop *loop,
                             cudaStream_t s)
 {
-    return launch_after(k_cg_flush, red_grid(n), kBlock, 0, s, d, n, sc, loop);
+    k_cg_flush<<<red_grid(n), kBlock, 0, s>>>(d, n, sc, loop);
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -777,14 +766,14 @@ int launch_cg_update(T *x, T *r, const T *d, const T *Ad, size_t n, const CgScal
     const int g = red_grid(n);
     if constexpr (sizeof(T) == 4) {
         if (vec4_ok(n, x, r, d, Ad) && vec4_ok(n, d_odd)) {
-            launch_after(k_cg_update_f4, g, kBlock, 0, s, reinterpret_cast<float4 *>(x),
-                         reinterpret_cast<float4 *>(r), reinterpret_cast<const float4 *>(d),
-                         reinterpret_cast<const float4 *>(Ad), n / 4, sc, partial, loop,
-                         reinterpret_cast<const float4 *>(d_odd));
+            k_cg_update_f4<<<g, kBlock, 0, s>>>(
+                reinterpret_cast<float4 *>(x), reinterpret_cast<float4 *>(r),
+                reinterpret_cast<const float4 *>(d), reinterpret_cast<const float4 *>(Ad), n / 4,
+                sc, partial, loop, reinterpret_cast<const float4 *>(d_odd));
             return g;
         }
     }
-    launch_after(k_cg_update<T>, g, kBlock, 0, s, x, r, d, Ad, n, sc, partial, loop, d_odd);
+    k_cg_update<T><<<g, kBlock, 0, s>>>(x, r, d, Ad, n, sc, partial, loop, d_odd);
     return g;
 }
 
@@ -793,7 +782,6 @@ __global__ void __launch_bounds__(kBlock)
 k_cg_direction(const T *__restrict__ z, const T *din, T *dout, size_t n, const CgScalars *sc,
                const CgLoop *__restrict__ loop)
 {
-    after_previous();
     if (loop && loop->its == 0) din = z;
     const T beta = BZ ? T(0) : (T)sc->beta;
 #pragma unroll 4
@@ -807,7 +795,6 @@ __global__ void __launch_bounds__(kBlock)
 k_cg_direction_f4(const float4 *__restrict__ z, const float4 *din, float4 *dout, size_t n4,
                   const CgScalars *sc, const CgLoop *__restrict__ loop)
 {
-    after_previous();
     if (loop && loop->its == 0) din = z;
     const float beta = BZ ? 0.f : (float)sc->beta;
 #pragma unroll 2
@@ -834,16 +821,15 @@ cudaError_t launch_cg_direction(const T *z, const T *d_in, T *d_out, size_t n, c
             const float4 *z4 = reinterpret_cast<const float4 *>(z);
             const float4 *di = reinterpret_cast<const float4 *>(d_in);
             float4 *dw = reinterpret_cast<float4 *>(d_out);
-            if (beta_zero) launch_after(k_cg_direction_f4<true>, g, kBlock, 0, s, z4, di, dw, n / 4,
-                                        sc, loop);
-            else launch_after(k_cg_direction_f4<false>, g, kBlock, 0, s, z4, di, dw, n / 4, sc,
-                              loop);
+            if (beta_zero)
+                k_cg_direction_f4<true><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
+            else
+                k_cg_direction_f4<false><<<g, kBlock, 0, s>>>(z4, di, dw, n / 4, sc, loop);
             return cudaGetLastError();
         }
     }
-    if (beta_zero) launch_after(k_cg_direction<T, true>, g, kBlock, 0, s, z, d_in, d_out, n, sc,
-                                loop);
-    else launch_after(k_cg_direction<T, false>, g, kBlock, 0, s, z, d_in, d_out, n, sc, loop);
+    if (beta_zero) k_cg_direction<T, true><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
+    else k_cg_direction<T, false><<<g, kBlock, 0, s>>>(z, d_in, d_out, n, sc, loop);
     return cudaGetLastError();
 }
 
@@ -978,7 +964,6 @@ __global__ void __launch_bounds__(1024)
 k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op, CgLoop *loop,
                 cudaGraphConditionalHandle cond)
 {
-    after_previous();
     __shared__ double ws[32];
     // the scalars of the last step, in flight while the partials are summed
     // (loaded after the sum: 64 x 32 x 16 in FP64 1.944 ms a solve instead of 1.925)
@@ -1014,7 +999,7 @@ k_loop_finalize(const double *__restrict__ partial, int n, CgScalars *sc, int op
 cudaError_t launch_loop_finalize(const double *partial, int n, CgScalars *sc, int op,
                                  CgLoop *loop, cudaGraphConditionalHandle cond, cudaStream_t s)
 {
-    launch_after(k_loop_finalize, 1, 1024, 0, s, partial, n, sc, op, loop, cond);
+    k_loop_finalize<<<1, 1024, 0, s>>>(partial, n, sc, op, loop, cond);
     return cudaGetLastError();
 }
 

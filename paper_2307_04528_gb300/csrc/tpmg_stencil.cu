@@ -41,6 +41,14 @@ __device__ __forceinline__ Two ld2(const double *p)
     return {{v.x, v.y}};
 }
 
+// The same of x or b, which the kernel before this one may have written
+// (after_previous).
+__device__ __forceinline__ Two ld2_of(const double *p)
+{
+    const double2 v = *reinterpret_cast<const double2 *>(p);
+    return {{v.x, v.y}};
+}
+
 // One layer of a thread's 2 x 2 columns: [row][column].
 template <bool SYM, bool RESID>
 struct Layer {
@@ -57,9 +65,8 @@ struct Layer {
 // form, as stencil_column.
 template <bool SYM, bool RESID, bool RED, bool CAST, bool NARROW, bool HSUM>
 __global__ void __launch_bounds__(kBlock, 3)
-k_stencil_quad(StencilView V, const double *__restrict__ b, const double *__restrict__ x,
-               void *__restrict__ yout, double scale, int kz, double *__restrict__ partial,
-               const int *__restrict__ flag)
+k_stencil_quad(StencilView V, const double *b, const double *x, void *__restrict__ yout,
+               double scale, int kz, double *__restrict__ partial, const int *flag)
 {
     after_previous();
     if (flag && !*flag) return;
@@ -80,9 +87,9 @@ k_stencil_quad(StencilView V, const double *__restrict__ b, const double *__rest
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const size_t c = o + (size_t)r * nlon;
-                l.x[r] = ld2(x + c);
-                l.xe[r] = __ldg(x + c + dE);
-                l.xw[r] = __ldg(x + c + dW);
+                l.x[r] = ld2_of(x + c);
+                l.xe[r] = x[c + dE];
+                l.xw[r] = x[c + dW];
                 l.e[r] = ld2(V.e + c);
                 l.ew[r] = __ldg(V.w + c + dW);
                 l.n[r] = ld2(V.n + c);
@@ -93,10 +100,10 @@ k_stencil_quad(StencilView V, const double *__restrict__ b, const double *__rest
                     l.sr[SYM ? 0 : r] = ld2(V.s + c);
                     l.d[SYM ? 0 : r] = ld2(V.d + c);
                 }
-                if (RESID) l.b[RESID ? r : 0] = ld2(b + c);
+                if (RESID) l.b[RESID ? r : 0] = ld2_of(b + c);
             }
-            l.xn = hasN ? ld2(x + o + 2 * (size_t)nlon) : zero;
-            l.xs = hasS ? ld2(x + o - nlon) : zero;
+            l.xn = hasN ? ld2_of(x + o + 2 * (size_t)nlon) : zero;
+            l.xs = hasS ? ld2_of(x + o - nlon) : zero;
             l.s0[0] = hasS ? ld2(V.s + o - nlon) : zero;
         };
         L cur, nxt;
@@ -111,7 +118,7 @@ k_stencil_quad(StencilView V, const double *__restrict__ b, const double *__rest
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const size_t c = (size_t)(k0 - 1) * plane + col + (size_t)r * nlon;
-                const Two xb = ld2(x + c);
+                const Two xb = ld2_of(x + c);
                 tdn[r] = ld2(V.d + c);
 #pragma unroll
                 for (int q = 0; q < 2; ++q) dn[r].a[q] = xb.a[q] - cur.x[r].a[q];

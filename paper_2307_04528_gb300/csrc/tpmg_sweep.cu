@@ -19,8 +19,8 @@ namespace {
 template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB,
           typename Level>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restrict__ uout,
-        T omega, double *__restrict__ partial, const int *__restrict__ flag)
+k_sweep(Level L, const T *b, const T *uin, T *__restrict__ uout, T omega,
+        double *__restrict__ partial, const int *flag)
 {
     after_previous();
     if (flag && !*flag) return;
@@ -38,8 +38,7 @@ k_sweep(Level L, const T *__restrict__ b, const T *__restrict__ uin, T *__restri
 // A Chebyshev step of the coarsest-level solve as one sweep (launch_cheb_sweep).
 template <typename T, int CV, int LZ, int QL, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_sweep_cheb(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ uin,
-             T *__restrict__ uout, ChebStep<T> ch)
+k_sweep_cheb(LevelDev<T> L, const T *b, const T *uin, T *__restrict__ uout, ChebStep<T> ch)
 {
     after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -192,8 +191,7 @@ constexpr int kClusterThreads = sizeof(T) == 4 && !kDirected<Level> ? 512
 
 template <typename T, int LZ, typename Level>
 __global__ void __launch_bounds__(kClusterThreads<T, LZ, Level>, 1)
-k_coarse_cluster(Level L, const T *__restrict__ b, T *__restrict__ out, T omega, int sweeps,
-                 int R)
+k_coarse_cluster(Level L, const T *b, T *__restrict__ out, T omega, int sweeps, int R)
 {
     after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];

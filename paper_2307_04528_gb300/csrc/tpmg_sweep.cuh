@@ -71,9 +71,10 @@ __device__ __forceinline__ Vals<T, CV> ldv(const T *__restrict__ p, unsigned byt
     return r;
 }
 
-// The same for values this kernel also writes (not through the read-only path).
+// The same of a vector that the kernel before this one may have written
+// (after_previous) or that this one writes: not through the read-only path.
 template <typename T, int CV>
-__device__ __forceinline__ Vals<T, CV> ldv_own(const T *p, unsigned byte)
+__device__ __forceinline__ Vals<T, CV> ldv_of(const T *p, unsigned byte)
 {
     Vals<T, CV> r;
     const char *q = reinterpret_cast<const char *>(p) + byte;
@@ -252,9 +253,9 @@ struct ChebStep {
 // level), and LZ blockDim CV more for DOT.
 template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, bool CHEB = false,
           typename Level>
-__device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
-                                        const T *__restrict__ uin, T *__restrict__ uout, T omega,
-                                        int tile, T *sh, const ChebStep<T> &ch = {})
+__device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin,
+                                        T *__restrict__ uout, T omega, int tile, T *sh,
+                                        const ChebStep<T> &ch = {})
 {
     using X = Vals<T, CV>;
     constexpr unsigned SZ = sizeof(T);
@@ -278,8 +279,8 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
     for (int c = 0; c < LZ; ++c) {
         m[c] = ldv<T, CV>(L.m, off);
         dq[c] = ldv<T, CV>(L.dq, off);
-        v[c] = ldv<T, CV>(b, off);
-        if (GUESS) uc[c] = ldv<T, CV>(uin, off);
+        v[c] = ldv_of<T, CV>(b, off);
+        if (GUESS) uc[c] = ldv_of<T, CV>(uin, off);
         if constexpr (NS) f[c] = ldv<T, CV>(down_of(L), off);
         off += k0 + c + 1 < nz ? plane : 0u;
     }
@@ -298,17 +299,17 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
         if constexpr (CHEB) {
             const unsigned dn = k0 > 0 && k0 < nz ? plane : 0u;
             tzd = ldv<T, CV>(up_of(L), first - dn);
-            ud = ldv<T, CV>(uin, first - dn);
-            ua = ldv<T, CV>(uin, first + (k0 + LZ < nz ? LZ * plane : 0u));
+            ud = ldv_of<T, CV>(uin, first - dn);
+            ua = ldv_of<T, CV>(uin, first + (k0 + LZ < nz ? LZ * plane : 0u));
         }
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
             const X t = ldv<T, CV>(east_of(L), off);
             X tb = t;  // the couplings of the cells to the west
             if constexpr (NS && CV > 1) tb = ldv<T, CV>(west_of(L), off);
-            const X N = ldv<T, CV>(un, off), S = ldv<T, CV>(us, off);
+            const X N = ldv_of<T, CV>(un, off), S = ldv_of<T, CV>(us, off);
             const X tn = ldv<T, CV>(north_of(L), off), tS = ldv<T, CV>(ts, off);
-            const T E = ldv<T, 1>(ue, off).a[0], W = ldv<T, 1>(uw, off).a[0];
+            const T E = ldv_of<T, 1>(ue, off).a[0], W = ldv_of<T, 1>(uw, off).a[0];
             const T tW = ldv<T, 1>(tw, off).a[0];
             if constexpr (CHEB) {
                 // r = b - H d in flux form
@@ -329,7 +330,6 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
                     v[c].a[e] -= s;
                 }
                 tzd = tz;
-                if (own < ncol && k0 + c < nz) stv<T, CV>(ch.r_out, off, v[c]);
                 off += k0 + c + 1 < nz ? plane : 0u;
                 continue;
             }
@@ -345,6 +345,12 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
             const X vs = vfma<T, CV>(tS, S, v[c]);
             v[c] = hasS ? vs : v[c];
             off += k0 + c + 1 < nz ? plane : 0u;
+        }
+        if constexpr (CHEB) {  // behind every load, which the compiler keeps in order with it
+            off = first;
+#pragma unroll
+            for (int c = 0; c < LZ; ++c, off += plane)
+                if (own < ncol && k0 + c < nz) stv<T, CV>(ch.r_out, off, v[c]);
         }
     }
     // layers past the top: 1/p = 0 makes their y and x zero; the sign of
@@ -391,7 +397,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
         off = first;
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
-            xv[c] = ch.first ? zero : ldv_own<T, CV>(ch.x, off);
+            xv[c] = ch.first ? zero : ldv_of<T, CV>(ch.x, off);
             off += k0 + c + 1 < nz ? plane : 0u;
         }
     }
@@ -443,7 +449,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *__restrict__ b,
 // The forward and backward maps of the segments are exchanged as in
 // sweep_tile, their factors once.  sh: 2 R nlon nz + 4 blockDim values.
 template <typename T, int LZ, typename Level>
-__device__ __forceinline__ void coarse_cluster(const Level &L, const T *__restrict__ b,
+__device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
                                                T *__restrict__ out, T omega, int sweeps, int R,
                                                T *sh)
 {
@@ -473,7 +479,7 @@ __device__ __forceinline__ void coarse_cluster(const Level &L, const T *__restri
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const int g = min(k0 + c, nz - 1) * plane + j * nlon + i;
-        bb[c] = __ldg(b + g);
+        bb[c] = b[g];
         te[c] = __ldg(east_of(L) + g);
         tw[c] = __ldg(west_of(L) + g + dw);
         tn[c] = hasN ? __ldg(north_of(L) + g) : T(0);
