@@ -245,7 +245,7 @@ static size_t carve(mg_handle *H, void *base)
         v.tz = cv.take<double>(n);
         v.h = cv.take<double>(n);
         v.m = cv.take<double>(n);
-        v.dq = cv.take<double>(n);
+        v.g = cv.take<double>(n);
         v.u = cv.take<double>(n);
         v.w = cv.take<double>(n);
         v.r = cv.take<double>(n);
@@ -267,7 +267,7 @@ static size_t carve(mg_handle *H, void *base)
             v.tz32 = cv.take<float>(n);
             v.h32 = cv.take<float>(n);
             v.m32 = cv.take<float>(n);
-            v.dq32 = cv.take<float>(n);
+            v.g32 = cv.take<float>(n);
             v.u32 = cv.take<float>(n);
             v.w32 = cv.take<float>(n);
             v.r32 = cv.take<float>(n);
@@ -465,7 +465,7 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
                 if (ratio - 1.0 <= H->p.iso_ratio) H->L = l + 2;  // level l+1 is the coarsest
             }
         }
-        KRUN(K_VEC, l, 0, launch_column_lu(dev<double>(v), v.m, v.dq, s));
+        KRUN(K_VEC, l, 0, launch_column_lu(dev<double>(v), v.m, v.g, s));
         // the uploads above read pageable host vectors: finish before they go away
         CU(cudaStreamSynchronize(s));
     }
@@ -504,7 +504,7 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
             KRUN(K_VEC, l, 1, launch_to_float(v.tz, v.tz32, H->scale32, v.n, s));
             KRUN(K_VEC, l, 1, launch_to_float(v.h, v.h32, H->scale32, v.n, s));
             KRUN(K_VEC, l, 1, launch_to_float(v.m, v.m32, 1.0 / H->scale32, v.n, s));
-            KRUN(K_VEC, l, 1, launch_to_float(v.dq, v.dq32, 1.0, v.n, s));
+            KRUN(K_VEC, l, 1, launch_to_float(v.g, v.g32, 1.0, v.n, s));
         }
     }
     CU(cudaStreamSynchronize(s));

@@ -367,12 +367,31 @@ __device__ __forceinline__ void stencil_cell(const LevelDev<T> &L, const T *__re
 }
 
 // ------------------------------------------------------------------ smoother
+// y + f x of a link factor stored as g (LevelDev): g's sign bit says that it is
+// f - 1, and x is added.  A product by f formed as 1 - q/p would keep the
+// absolute accuracy of q/p only: where t << p, as across a drop of the row sums
+// by 1e3, an FP32 column solve was off by 3e-5 instead of 2e-7.
+__device__ __forceinline__ int sign_word(float g) { return __float_as_int(g); }
+__device__ __forceinline__ int sign_word(double g) { return __double2hiint(g); }
+template <typename T>
+__device__ __forceinline__ T whole(T g, T x)
+{
+    return sign_word(g) < 0 ? x : T(0);
+}
+template <typename T>
+__device__ __forceinline__ T link(T g, T x, T y)
+{
+    return fma(g, x, y) + whole(g, x);
+}
+
 // One sweep of Eq. (1), u_out = (1 - omega) u_in + omega H_z^{-1}(b - dH u_in),
 // with the column tridiagonal H_z (diagonal s_k + t_{k-1} + t_k, couplings
 // -t_k, s_k = h + the four horizontal couplings) solved by elimination with
-// pivots p_k = q_k + t_k, on the setup factors m_k = 1/p_k and dq_k = q_k/p_k:
+// pivots p_k = q_k + t_k, on the setup factors m_k = 1/p_k and the link
+// factors f_k = t_k/p_k (stored as g, LevelDev):
 //   forward   y_k = (v_k + t_{k-1} y_{k-1}) m_k,  v_k = b_k + sum_h T u_in,nb
-//   backward  x_k = x_{k+1} + (y_k - dq_k x_{k+1})
+//   backward  x_k = y_k + f_k x_{k+1}, formed as x_{k+1} + (y_k - (q_k/p_k)
+//             x_{k+1}) where q_k is the smaller part of the pivot
 // This is the column walk on a non-zero guess; from a zero guess it is
 // smooth_staged.  Most levels sweep by segments instead (sweep_tile).
 // The forward values y wait in shared memory for the backward sweep
@@ -522,16 +541,16 @@ __device__ __forceinline__ void smooth_column(const LevelDev<T> &L, const T *__r
 
     const T om1 = T(1) - omega;
     T xk = yprev;
-    // backward sweep: prefetch u_in, q/p (and b) kBack layers ahead
+    // backward sweep: prefetch u_in, g (and b) kBack layers ahead
     constexpr int kBack = BACK > 0 ? BACK : SmoothDepth<T>::back;
-    T up[kBack], dqp[kBack], bp[kBack];
+    T up[kBack], gp[kBack], bp[kBack];
 #pragma unroll
     for (int d = 0; d < kBack; ++d) {
         const int k = nz - 1 - d;
         if (k >= 0) {
             const size_t o = (size_t)k * plane + col;
             up[d] = __ldg(uin + o);
-            dqp[d] = HINT ? ld_hint(L.dq + o, hp.stream) : __ldg(L.dq + o);
+            gp[d] = HINT ? ld_hint(L.g + o, hp.stream) : __ldg(L.g + o);
             bp[d] = DOT ? __ldg(b + o) : T(0);
         }
     }
@@ -542,7 +561,7 @@ __device__ __forceinline__ void smooth_column(const LevelDev<T> &L, const T *__r
             if (k >= 0) {
                 const size_t o = (size_t)k * plane + col;
                 if (k < nz - 1)
-                    xk = xk + fma(-dqp[d], xk, YOUT ? uout[o] : ys[(size_t)k * bd + tid]);
+                    xk = link(gp[d], xk, YOUT ? uout[o] : ys[(size_t)k * bd + tid]);
                 const T uo = fma(om1, up[d], omega * xk);
                 uout[o] = uo;
                 if (DOT) *dacc = fma(bp[d], uo, *dacc);
@@ -550,7 +569,7 @@ __device__ __forceinline__ void smooth_column(const LevelDev<T> &L, const T *__r
                 if (kn >= 0) {
                     const size_t on = (size_t)kn * plane + col;
                     up[d] = __ldg(uin + on);
-                    dqp[d] = HINT ? ld_hint(L.dq + on, hp.stream) : __ldg(L.dq + on);
+                    gp[d] = HINT ? ld_hint(L.g + on, hp.stream) : __ldg(L.g + on);
                     if (DOT) bp[d] = __ldg(b + on);
                 }
             }
@@ -565,7 +584,7 @@ __device__ __forceinline__ void smooth_column(const LevelDev<T> &L, const T *__r
 // [l C, l C + C), C = ceil(nz / 32).  Both recurrences are first-order and
 // linear, so they run as warp scans of affine maps:
 //   forward   y_k = (v_k + t_{k-1} y_{k-1}) / p_k  = (t_{k-1}/p_k) y_{k-1} + v_k/p_k
-//   backward  x_k = y_k + (1 - q_k/p_k) x_{k+1}      (x_nz = 0)
+//   backward  x_k = y_k + f_k x_{k+1}      (x_nz = 0)
 // Each lane composes the maps of its layers, a Kogge-Stone scan across the
 // lanes gives each lane the value entering its layers, and the lane then
 // re-runs its own layers with the serial formulas of smooth_column.  The
@@ -583,7 +602,7 @@ constexpr int kWarpLayers = (kMaxLayers + 31) / 32;  // layers per lane at most
 // H_z x = v on return; tprev = t_{k0-1} (0 for the first lane).
 template <typename T, int CM>
 __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], const T (&m)[CM],
-                                                 const T (&dq)[CM], T tprev, int C, int k0,
+                                                 const T (&g)[CM], T tprev, int C, int k0,
                                                  int nz, int lane)
 {
     // forward: this lane's map y_out = A y_in + Cy, then an inclusive scan
@@ -623,9 +642,8 @@ __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], 
 #pragma unroll
     for (int c = CM - 1; c >= 0; --c) {
         if (c < C && k0 + c < nz) {
-            const T e = T(1) - dq[c];
-            F = fma(e, F, v[c]);
-            E = e * E;
+            F = link(g[c], F, v[c]);
+            E = link(g[c], E, T(0));
         }
     }
 #pragma unroll
@@ -642,14 +660,14 @@ __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], 
 #pragma unroll
     for (int c = CM - 1; c >= 0; --c) {
         if (c < C && k0 + c < nz) {
-            x = x + fma(-dq[c], x, v[c]);
+            x = link(g[c], x, v[c]);
             v[c] = x;  // v now holds x
         }
     }
 }
 
 // The coarsest-level solve (sweeps of Eq. (1) from zero) by one block with
-// the whole level in shared memory: b, t_z, 1/p, q/p,
+// the whole level in shared memory: b, t_z, 1/p, g,
 // t_x, t_y and the two sweep vectors, each stored as [column][layer], so a
 // lane's own layers are consecutive words (bank-conflict free for an odd
 // layers-per-lane count).  The level is staged once from its [layer][column]
@@ -664,7 +682,7 @@ __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *_
 {
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat, n = ncol * nz;
-    T *sb = sh, *stz = sh + n, *sm = sh + 2 * n, *sdq = sh + 3 * n, *stx = sh + 4 * n,
+    T *sb = sh, *stz = sh + n, *sm = sh + 2 * n, *sg = sh + 3 * n, *stx = sh + 4 * n,
       *sty = sh + 5 * n;
     T *cur = sh + 6 * n, *oth = sh + 7 * n;
     for (int g = threadIdx.x; g < n; g += blockDim.x) {
@@ -672,7 +690,7 @@ __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *_
         sb[o] = __ldg(b + g);
         stz[o] = __ldg(L.tz + g);
         sm[o] = __ldg(L.m + g);
-        sdq[o] = __ldg(L.dq + g);
+        sg[o] = __ldg(L.g + g);
         stx[o] = __ldg(L.tx + g);
         sty[o] = __ldg(L.ty + g);
     }
@@ -688,11 +706,11 @@ __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *_
             const bool hasN = j + 1 < nlat, hasS = j > 0;
             const int oc = col * nz, oe = ie * nz, ow = iw * nz;
             const int on = (col + nlon) * nz, os = (col - nlon) * nz;
-            T v[CM], tz[CM], m[CM], dq[CM], u0[CM];
+            T v[CM], tz[CM], m[CM], g[CM], u0[CM];
 #pragma unroll
             for (int c = 0; c < CM; ++c) {
                 const int k = k0 + c;
-                v[c] = tz[c] = m[c] = dq[c] = u0[c] = T(0);
+                v[c] = tz[c] = m[c] = g[c] = u0[c] = T(0);
                 if (c < C && k < nz) {
                     T vv = sb[oc + k];
                     if (it > 0) {
@@ -705,11 +723,11 @@ __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *_
                     v[c] = vv;
                     tz[c] = stz[oc + k];
                     m[c] = sm[oc + k];
-                    dq[c] = sdq[oc + k];
+                    g[c] = sg[oc + k];
                 }
             }
             const T tprev = (k0 >= 1 && k0 - 1 < nz) ? stz[oc + k0 - 1] : T(0);
-            warp_column_scan<T, CM>(v, tz, m, dq, tprev, C, k0, nz, lane);
+            warp_column_scan<T, CM>(v, tz, m, g, tprev, C, k0, nz, lane);
 #pragma unroll
             for (int c = 0; c < CM; ++c) {
                 const int k = k0 + c;
@@ -759,7 +777,7 @@ __device__ __forceinline__ void stage_wait()
 
 // Layers in flight per thread in the staged sweep, and values staged per
 // layer: forward b, t_z, 1/p (+ t_x east/west, t_y north/south and the four
-// horizontal neighbours of u_in unless the guess is zero); backward q/p
+// horizontal neighbours of u_in unless the guess is zero); backward g
 // (+ u_in, + b for the fused inner product).
 constexpr int kRing = 8;
 
@@ -777,8 +795,8 @@ __host__ __device__ constexpr size_t ring_smem_bytes(int nz, int block)
     return ((size_t)kRing * RingSlot<ZERO>::NV + (size_t)nz) * (size_t)block * sizeof(T);
 }
 
-// One column of the sweep of Eq. (1) on precomputed factors (m = 1/p,
-// dq = q/p), the same arithmetic in the same order as smooth_column, with
+// One column of the sweep of Eq. (1) on precomputed factors (m = 1/p and
+// g), the same arithmetic in the same order as smooth_column, with
 // every load staged kRing layers ahead through shared memory by cp.async
 // (the copies hold no registers, so the depth of the pipeline is not left to
 // register allocation).  Horizontal neighbours missing at the poles read as 0
@@ -874,9 +892,9 @@ __device__ __forceinline__ void smooth_staged(const LevelDev<T> &L, const T *__r
     }
     stage_wait<0>();
 
-    // backward sweep: stage q/p (+ u_in, + b) of layers nz-1, nz-2, ...
+    // backward sweep: stage g (+ u_in, + b) of layers nz-1, nz-2, ...
     const size_t top = (size_t)(nz - 1) * plane + col;
-    const T *qq = L.dq + top, *qu = (ZERO ? b : uin) + top, *qb = b + top;
+    const T *qq = L.g + top, *qu = (ZERO ? b : uin) + top, *qb = b + top;
     auto issue_back = [&](int sl_) {
         T *sl = ring + (size_t)sl_ * NV * bd;
         stage(sl, qq);
@@ -901,7 +919,7 @@ __device__ __forceinline__ void smooth_staged(const LevelDev<T> &L, const T *__r
     for (int k = nz - 1; k >= 0; --k) {
         stage_wait<kRing - 1>();
         const T *sl = ring + (size_t)slot * NV * bd;
-        if (k < nz - 1) xk = xk + fma(-sl[0], xk, ys[(size_t)k * bd]);
+        if (k < nz - 1) xk = link(sl[0], xk, ys[(size_t)k * bd]);
         const T uo = ZERO ? omega * xk : fma(om1, sl[bd], omega * xk);
         *uo_p = uo;
         uo_p -= plane;

@@ -54,9 +54,9 @@ using tpmg::BicgScalars;
 struct LevelHost {
     int nlon = 0, nlat = 0, nz = 0;
     size_t n = 0;
-    double *tx = nullptr, *ty = nullptr, *tz = nullptr, *h = nullptr, *m = nullptr, *dq = nullptr;
+    double *tx = nullptr, *ty = nullptr, *tz = nullptr, *h = nullptr, *m = nullptr, *g = nullptr;
     float *tx32 = nullptr, *ty32 = nullptr, *tz32 = nullptr, *h32 = nullptr, *m32 = nullptr,
-          *dq32 = nullptr;
+          *g32 = nullptr;
     // V-cycle vectors: rhs, result, ping-pong scratch, residual
     double *b = nullptr, *u = nullptr, *w = nullptr, *r = nullptr;
     float *b32 = nullptr, *u32 = nullptr, *w32 = nullptr, *r32 = nullptr;
@@ -139,12 +139,12 @@ LevelDev<T> dev(const LevelHost &l);
 template <>
 inline LevelDev<double> dev<double>(const LevelHost &l)
 {
-    return {l.nlon, l.nlat, l.nz, l.tx, l.ty, l.tz, l.h, l.m, l.dq};
+    return {l.nlon, l.nlat, l.nz, l.tx, l.ty, l.tz, l.h, l.m, l.g};
 }
 template <>
 inline LevelDev<float> dev<float>(const LevelHost &l)
 {
-    return {l.nlon, l.nlat, l.nz, l.tx32, l.ty32, l.tz32, l.h32, l.m32, l.dq32};
+    return {l.nlon, l.nlat, l.nz, l.tx32, l.ty32, l.tz32, l.h32, l.m32, l.g32};
 }
 template <typename T>
 struct Vec;

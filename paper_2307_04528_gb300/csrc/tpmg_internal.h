@@ -15,7 +15,10 @@ struct LevelDev {
     int nlon, nlat, nz;
     const T *tx, *ty, *tz, *h;  // coefficients (FP32 copies are scaled by a power of two)
     const T *m;                 // 1 / p_k, pivot inverse of the column tridiagonal
-    const T *dq;                // q_k / p_k, p_k = q_k + tz_k (row-sum form of the pivot)
+    // the link factor f_k = t_k / p_k of p_k = q_k + t_k, less one where it is
+    // above a half, and on top (-q_k / p_k < 0): both f and 1 - f = q / p keep
+    // their full relative accuracy in one array (link, carry)
+    const T *g;
 };
 
 // Links from level l to level l+1 (device arrays, sizes in comments).
@@ -341,10 +344,10 @@ cudaError_t launch_validate(const LevelDev<double> &L, int *flag, cudaStream_t s
 // Coarse coefficients of level l+1 from level l (sums; lon faces x sx, lat faces x sy[J]).
 cudaError_t launch_coarsen(const LevelDev<double> &F, const LinkDev &K, double sx, double *txc,
                            double *tyc, double *tzc, double *hc, cudaStream_t s);
-// Column factors (m, dq) of every column of a level, in FP64.
-cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *dq, cudaStream_t s);
+// Column factors (m, g) of every column of a level, in FP64.
+cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, cudaStream_t s);
 // FP32 copies: out = (float)(scale * in) for coefficients; m32 = (float)(m / scale);
-// dq32 = (float)dq.
+// g32 = (float)g.
 cudaError_t launch_to_float(const double *in, float *out, double scale, size_t n, cudaStream_t s);
 
 // Coefficient gradient (see mg_coeff_grad); outputs may be null.
@@ -480,9 +483,14 @@ struct NsView {
     const T *m, *dq;
 };
 
-// The arrays of a level by the face they couple a cell across: a cell's own
-// coupling east / north, and its western / southern neighbour's row (the cell
-// one west, one south in the array), the same array in a symmetric level.
+// The arrays of a level (factor_of: g, or a directed level's q/p) by the face
+// they couple a cell across: a cell's own coupling east / north, and its western
+// / southern neighbour's row (the cell one west, one south in the array), the
+// same array in a symmetric level.
+template <typename T>
+__host__ __device__ inline const T *factor_of(const LevelDev<T> &L) { return L.g; }
+template <typename T>
+__host__ __device__ inline const T *factor_of(const NsView<T> &V) { return V.dq; }
 template <typename T>
 __host__ __device__ inline const T *mass_of(const LevelDev<T> &L) { return L.h; }
 template <typename T>

@@ -1080,9 +1080,10 @@ cudaError_t launch_coarsen(const LevelDev<double> &F, const LinkDev &K, double s
 }
 
 // Column factors: q_0 = s_0, q_k = s_k + t_{k-1} q_{k-1} / p_{k-1}, p_k = q_k + t_k;
-// store m = 1/p and dq = q/p.
+// store m = 1/p and g = t/p, or -q/p where that is the smaller (no closer to zero
+// than FP32's smallest normal value, so that its sign is never lost) and on top (-1).
 __global__ void __launch_bounds__(kBlock)
-k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ dq)
+k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g)
 {
     const int nlon = L.nlon, nlat = L.nlat;
     const int ncol = nlon * nlat;
@@ -1100,17 +1101,17 @@ k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ dq)
         const double tup = L.tz[o + col];
         const double p = q + tup;
         m[o + col] = 1.0 / p;
-        dq[o + col] = q / p;
+        g[o + col] = q < tup || k == L.nz - 1 ? -fmax(q / p, 0x1p-126) : tup / p;
         qp = q;
         pp = p;
         tdn = tup;
     }
 }
 
-cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *dq, cudaStream_t s)
+cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, cudaStream_t s)
 {
     const int ncol = L.nlon * L.nlat;
-    k_column_lu<<<(ncol + kBlock - 1) / kBlock, kBlock, 0, s>>>(L, m, dq);
+    k_column_lu<<<(ncol + kBlock - 1) / kBlock, kBlock, 0, s>>>(L, m, g);
     return cudaGetLastError();
 }
 

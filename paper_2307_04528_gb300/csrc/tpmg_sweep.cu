@@ -241,7 +241,7 @@ int pick(const Level &L, const Sweep<T> &a)
     const uintptr_t ptrs = (uintptr_t)a.b | (uintptr_t)a.uin | (uintptr_t)a.uout |
                            (uintptr_t)east_of(L) | (uintptr_t)north_of(L) |
                            (uintptr_t)west_of(L) | (uintptr_t)south_of(L) |
-                           (uintptr_t)down_of(L) | (uintptr_t)L.m | (uintptr_t)L.dq |
+                           (uintptr_t)down_of(L) | (uintptr_t)L.m | (uintptr_t)factor_of(L) |
                            (uintptr_t)mass_of(L) | (uintptr_t)up_of(L) |
                            (a.ch ? (uintptr_t)a.ch->r_out | (uintptr_t)a.ch->x : 0);
     if constexpr (sizeof(T) == 8) {

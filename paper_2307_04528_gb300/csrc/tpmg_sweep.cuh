@@ -3,14 +3,15 @@
 //
 // Both recurrences of the column solve are first-order and linear, so a
 // segment of layers acts on the value entering it as an affine map.  With
-// the setup factors m = 1/p and dq = q/p, p = q + t, the forward elimination
+// the setup factors m = 1/p and f = t/p, p = q + t, the forward elimination
 //   y_k = (v_k + t_{k-1} y_{k-1}) m_k
-// is carried as h_k = t_k y_k = t_k m_k w_k = (1 - dq_k) w_k, w_k = v_k +
-// h_{k-1}, y_k = m_k w_k: t_z is not read at all (20 -> 16 bytes per cell
-// from a zero guess in FP32, 32 -> 28 on a guess), and w - dq w keeps the row
-// sums that the rounded factor t m would lose.  The backward substitution x_k
-// = x_{k+1} + (y_k - dq_k x_{k+1}) is as in the serial sweep (smooth_column);
-// the maps of both directions share the factor A = prod (1 - dq).
+// is carried as h_k = t_k y_k = f_k w_k, w_k = v_k + h_{k-1}, y_k = m_k w_k:
+// t_z is not read at all (20 -> 16 bytes per cell from a zero guess in FP32, 32
+// -> 28 on a guess).  f is kept as g (LevelDev): where q is the smaller part of
+// the pivot, w - (q/p) w keeps the row sums that a rounded f would lose, where t
+// is, f w keeps the coupling that 1 - q/p would lose.  The backward substitution
+// x_k = y_k + f_k x_{k+1} is as in the serial sweep (smooth_column); the maps of
+// both directions share the factor A = prod f.
 //
 // A thread owns CV adjacent columns and LZ consecutive layers; QL lanes sit
 // side by side along longitude, so a warp covers QL CV columns of 32 / QL
@@ -24,6 +25,8 @@
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "tpmg_device.cuh"
 #include "tpmg_internal.h"
@@ -227,14 +230,105 @@ __device__ __forceinline__ Vals<T, CV> lds_v(const T *p)
     return r;
 }
 
-// w of the layer's map h_out = F w: (1 - q/p) w, or in a directed level f w
-// with f = d m (the coupling down of the row above times 1/p).
-template <bool NS, typename T, int CV>
-__device__ __forceinline__ Vals<T, CV> carry(const Vals<T, CV> &ndq, const Vals<T, CV> &f,
+// How the link factors f, kept as g (LevelDev), are taken:
+//   LINK_EITHER    w counts where g is f - 1: in FP64 by a select, in FP32 by a factor
+//                  of one or zero
+//   LINK_LESS_ONE  every g of the warp is f - 1 (a vote): f w = g w + w.  The coarsest-
+//                  level solve in FP64, whose sweeps share one vote
+//   LINK_DIRECTED  g = -q/p, with f = d m (the coupling down of the row above times
+//                  1/p) beside it
+// A vote in the sweeps of sweep_tile lets all warps but the 1 to 4 % at the poles of a
+// lat-lon grid take the short form, but its branches undid the order of the loads
+// (with <b, u_out> at 512 x 384 x 70 in FP32: 84 -> 150 us).
+enum { LINK_LESS_ONE, LINK_EITHER, LINK_DIRECTED };
+
+// One where g is f - 1, else zero: a saturated product, which issues on the FMA pipe
+// (selects by g's sign go to the integer pipe at half its rate; the FP32 V-cycle at
+// 1024 x 768 x 70: 1.11 -> 1.03 ms); no negative g lies above -2^-126
+// (launch_column_lu).  volatile: formed anew at each use instead of held in registers.
+__device__ __forceinline__ float one_of(float g)
+{
+    float z;
+    asm volatile("mul.rn.sat.f32 %0, %1, %2;" : "=f"(z) : "f"(g), "f"(-0x1p127f));
+    return z;
+}
+template <int CV>
+__device__ __forceinline__ Vals<float, CV> vone(const Vals<float, CV> &g)
+{
+    Vals<float, CV> r;
+#pragma unroll
+    for (int i = 0; i < CV; ++i) r.a[i] = one_of(g.a[i]);
+    return r;
+}
+
+// f w, w = v + h.  In FP32 the w that counts is formed beside w, as z h + z v, so
+// that the chain from h to f w stays two operations long.
+template <int LINK, typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> carry(const Vals<T, CV> &g, const Vals<T, CV> &f,
+                                             const Vals<T, CV> &v, const Vals<T, CV> &h,
                                              const Vals<T, CV> &w)
 {
-    if constexpr (NS) return vmul<T, CV>(f, w);
-    else return vfma<T, CV>(ndq, w, w);
+    if constexpr (LINK == LINK_DIRECTED) {
+        return vmul<T, CV>(f, w);
+    } else if constexpr (LINK == LINK_LESS_ONE) {
+        return vfma<T, CV>(g, w, w);
+    } else if constexpr (sizeof(T) == 4) {
+        const Vals<T, CV> z = vone(g);
+        return vfma<T, CV>(g, w, vfma<T, CV>(z, h, vmul<T, CV>(z, v)));
+    } else {
+        Vals<T, CV> r;
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = fma(g.a[i], w.a[i], whole(g.a[i], w.a[i]));
+        return r;
+    }
+}
+
+// y + f x; in a directed level x + (y - (q/p) x).
+template <int LINK, typename T, int CV>
+__device__ __forceinline__ Vals<T, CV> back(const Vals<T, CV> &g, const Vals<T, CV> &x,
+                                            const Vals<T, CV> &y)
+{
+    const Vals<T, CV> t = vfma<T, CV>(g, x, y);
+    if constexpr (LINK != LINK_EITHER) {
+        return vadd<T, CV>(x, t);
+    } else if constexpr (sizeof(T) == 4) {
+        return vfma<T, CV>(vone(g), x, t);
+    } else {
+        Vals<T, CV> r;
+#pragma unroll
+        for (int i = 0; i < CV; ++i) r.a[i] = whole(g.a[i], x.a[i]) + t.a[i];
+        return r;
+    }
+}
+
+// Whether some lane of the warp holds a g that is not f - 1 (FP64).
+template <bool NS, typename T, int CV, int LZ>
+__device__ __forceinline__ bool any_either(const Vals<T, CV> (&g)[LZ])
+{
+    if constexpr (NS || sizeof(T) == 4) {
+        return true;
+    } else {
+        int sign = -1;
+#pragma unroll
+        for (int c = 0; c < LZ; ++c)
+#pragma unroll
+            for (int i = 0; i < CV; ++i) sign &= sign_word(g[c].a[i]);
+        return __any_sync(0xffffffffu, sign >= 0);
+    }
+}
+
+// run(the warp's LINK_*).
+template <typename T, bool NS, typename F>
+__device__ __forceinline__ void with_links(bool either, F &&run)
+{
+    if constexpr (NS) {
+        run(std::integral_constant<int, LINK_DIRECTED>{});
+    } else if constexpr (sizeof(T) == 4) {
+        run(std::integral_constant<int, LINK_EITHER>{});
+    } else {
+        if (either) run(std::integral_constant<int, LINK_EITHER>{});
+        else run(std::integral_constant<int, LINK_LESS_ONE>{});
+    }
 }
 
 // A Chebyshev step instead of a sweep: with b the residual and u_in the step d,
@@ -260,6 +354,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
     using X = Vals<T, CV>;
     constexpr unsigned SZ = sizeof(T);
     constexpr bool NS = kDirected<Level>;
+    constexpr int LINK = NS ? LINK_DIRECTED : LINK_EITHER;
     static_assert(!(NS && DOT), "no <b, u_out> of a directed level");
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat;
@@ -272,13 +367,13 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
     const int row = blockDim.x * CV;  // values per slot row of shared memory
     T *sb = sh + 3 * row + threadIdx.x * CV;
 
-    X v[LZ], m[LZ], dq[LZ], uc[GUESS ? LZ : 1], f[NS ? LZ : 1];
+    X v[LZ], m[LZ], g[LZ], uc[GUESS ? LZ : 1], f[NS ? LZ : 1];
     // No load sits behind a branch: layers past the top re-read the last one.
     unsigned off = first;
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         m[c] = ldv<T, CV>(L.m, off);
-        dq[c] = ldv<T, CV>(L.dq, off);
+        g[c] = ldv<T, CV>(factor_of(L), off);
         v[c] = ldv_of<T, CV>(b, off);
         if (GUESS) uc[c] = ldv_of<T, CV>(uin, off);
         if constexpr (NS) f[c] = ldv<T, CV>(down_of(L), off);
@@ -353,14 +448,16 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
                 if (own < ncol && k0 + c < nz) stv<T, CV>(ch.r_out, off, v[c]);
         }
     }
-    // layers past the top: 1/p = 0 makes their y and x zero; the sign of
-    // every use of q/p is taken here
+    // layers past the top: 1/p = 0 makes their y and x zero; a directed level's
+    // q/p takes the sign of its uses
     const X zero = splat<T, CV>(T(0));
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         m[c] = k0 + c < nz ? m[c] : zero;
-        dq[c] = vneg<T, CV>(dq[c]);
-        if constexpr (NS) f[c] = vmul<T, CV>(f[c], m[c]);
+        if constexpr (NS) {
+            g[c] = vneg<T, CV>(g[c]);
+            f[c] = vmul<T, CV>(f[c], m[c]);
+        }
     }
 
     // forward: the segment's map h_out = A h_in + C; backward factor B (= A in
@@ -369,9 +466,9 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const X t = vadd<T, CV>(v[c], C);
-        C = carry<NS, T, CV>(dq[c], f[NS ? c : 0], t);
-        A = carry<NS, T, CV>(dq[c], f[NS ? c : 0], A);
-        if constexpr (NS) B = vfma<T, CV>(dq[c], B, B);
+        C = carry<LINK, T, CV>(g[c], f[NS ? c : 0], v[c], C, t);
+        A = carry<LINK, T, CV>(g[c], f[NS ? c : 0], zero, A, A);
+        if (NS) B = vfma<T, CV>(g[c], B, B);
     }
     T *sA = sh + q * CV, *sC = sA + row, *sF = sC + row, *sB = sA;
     if constexpr (NS) {
@@ -389,7 +486,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
         const X w = vadd<T, CV>(v[c], h);
-        h = carry<NS, T, CV>(dq[c], f[NS ? c : 0], w);
+        h = carry<LINK, T, CV>(g[c], f[NS ? c : 0], v[c], h, w);
         v[c] = vmul<T, CV>(w, m[c]);
     }
     X xv[CHEB ? LZ : 1];
@@ -403,7 +500,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
     }
     X F = zero;
 #pragma unroll
-    for (int c = LZ - 1; c >= 0; --c) F = vadd<T, CV>(F, vfma<T, CV>(dq[c], F, v[c]));
+    for (int c = LZ - 1; c >= 0; --c) F = back<LINK, T, CV>(g[c], F, v[c]);
     stv<T, CV>(sF + seg * QL * CV, 0u, F);
     __syncthreads();
     X x = zero;
@@ -414,7 +511,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
     off = first + (unsigned)(min(LZ, nz - k0) - 1) * plane;
 #pragma unroll
     for (int c = LZ - 1; c >= 0; --c) {
-        x = vadd<T, CV>(x, vfma<T, CV>(dq[c], x, v[c]));
+        x = back<LINK, T, CV>(g[c], x, v[c]);
         X uo;
         if constexpr (CHEB) {
             uo = vfma<T, CV>(splat<T, CV>(ch.c2), x, vmul<T, CV>(splat<T, CV>(ch.c1), uc[c]));
@@ -475,29 +572,40 @@ __device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
         n0 = r + 1 < rows ? u0 + lc + nlon : cl.map_shared_rank(u0, rank + 1) + i;
     if (hasS)
         s0 = r > 0 ? u0 + lc - nlon : cl.map_shared_rank(u0, rank - 1) + (R - 1) * nlon + i;
-    T m[LZ], dq[LZ], bb[LZ], te[LZ], tw[LZ], tn[LZ], ts[LZ], uc[LZ], f[NS ? LZ : 1], A = 1, B = 1;
+    using X = Vals<T, 1>;
+    T m[LZ], bb[LZ], te[LZ], tw[LZ], tn[LZ], ts[LZ], uc[LZ];
+    X g[LZ], f[NS ? LZ : 1];
 #pragma unroll
     for (int c = 0; c < LZ; ++c) {
-        const int g = min(k0 + c, nz - 1) * plane + j * nlon + i;
-        bb[c] = b[g];
-        te[c] = __ldg(east_of(L) + g);
-        tw[c] = __ldg(west_of(L) + g + dw);
-        tn[c] = hasN ? __ldg(north_of(L) + g) : T(0);
-        ts[c] = hasS ? __ldg(south_of(L) + g - nlon) : T(0);
-        m[c] = k0 + c < nz ? __ldg(L.m + g) : T(0);
-        dq[c] = -__ldg(L.dq + g);
+        const int o = min(k0 + c, nz - 1) * plane + j * nlon + i;
+        bb[c] = b[o];
+        te[c] = __ldg(east_of(L) + o);
+        tw[c] = __ldg(west_of(L) + o + dw);
+        tn[c] = hasN ? __ldg(north_of(L) + o) : T(0);
+        ts[c] = hasS ? __ldg(south_of(L) + o - nlon) : T(0);
+        m[c] = k0 + c < nz ? __ldg(L.m + o) : T(0);
+        g[c].a[0] = NS ? -__ldg(factor_of(L) + o) : __ldg(factor_of(L) + o);
         uc[c] = 0;
-        if constexpr (NS) f[c] = __ldg(down_of(L) + g) * m[c];
-        A = NS ? f[NS ? c : 0] * A : fma(dq[c], A, A);
-        B = fma(dq[c], B, B);
+        if constexpr (NS) f[c].a[0] = __ldg(down_of(L) + o) * m[c];
     }
-    sA[threadIdx.x] = A;
-    if (NS) sB[threadIdx.x] = B;
+    const X zero = {{T(0)}};
+    const bool either = any_either<NS>(g);
+    X A = {{T(1)}}, B = A;
+    with_links<T, NS>(either, [&](auto link) {
+        constexpr int LINK = decltype(link)::value;
+#pragma unroll
+        for (int c = 0; c < LZ; ++c) {
+            A = carry<LINK, T, 1>(g[c], f[NS ? c : 0], zero, A, A);
+            if (NS) B = vfma<T, 1>(g[c], B, B);
+        }
+    });
+    sA[threadIdx.x] = A.a[0];
+    if (NS) sB[threadIdx.x] = B.a[0];
     const T om1 = T(1) - omega;
     for (int it = 0; it < sweeps; ++it) {
         const int cur = (it & 1) * part * nz;  // the copy read; the other is written
         T *nxt = (it & 1) ? u0 : u1;
-        T v[LZ], C = 0;
+        X v[LZ], C = zero;
 #pragma unroll
         for (int c = 0; c < LZ; ++c) {
             T x = bb[c];
@@ -508,33 +616,45 @@ __device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
                 x = fma(tn[c], n0[o], x);
                 x = fma(ts[c], s0[o], x);
             }
-            v[c] = x;
-            const T t = x + C;
-            C = NS ? f[NS ? c : 0] * t : fma(dq[c], t, t);
+            v[c].a[0] = x;
         }
-        sC[threadIdx.x] = C;
-        __syncthreads();
-        T h = 0;
-#pragma unroll 4
-        for (int s = 0; s < seg; ++s) h = fma(sA[s * cols + lc], h, sC[s * cols + lc]);
+        with_links<T, NS>(either, [&](auto link) {
+            constexpr int LINK = decltype(link)::value;
 #pragma unroll
-        for (int c = 0; c < LZ; ++c) {
-            const T w = v[c] + h;
-            h = NS ? f[NS ? c : 0] * w : fma(dq[c], w, w);
-            v[c] = w * m[c];
-        }
-        T F = 0;
-#pragma unroll
-        for (int c = LZ - 1; c >= 0; --c) F = F + fma(dq[c], F, v[c]);
-        sF[threadIdx.x] = F;
+            for (int c = 0; c < LZ; ++c)
+                C = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], C, vadd<T, 1>(v[c], C));
+        });
+        sC[threadIdx.x] = C.a[0];
         __syncthreads();
-        T x = 0;
+        X h = zero;
 #pragma unroll 4
-        for (int s = nseg - 1; s > seg; --s) x = fma(sB[s * cols + lc], x, sF[s * cols + lc]);
+        for (int s = 0; s < seg; ++s) h.a[0] = fma(sA[s * cols + lc], h.a[0], sC[s * cols + lc]);
+        X F = zero;
+        with_links<T, NS>(either, [&](auto link) {
+            constexpr int LINK = decltype(link)::value;
+#pragma unroll
+            for (int c = 0; c < LZ; ++c) {
+                const X w = vadd<T, 1>(v[c], h);
+                h = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], h, w);
+                v[c].a[0] = w.a[0] * m[c];
+            }
+#pragma unroll
+            for (int c = LZ - 1; c >= 0; --c) F = back<LINK, T, 1>(g[c], F, v[c]);
+        });
+        sF[threadIdx.x] = F.a[0];
+        __syncthreads();
+        X x = zero;
+#pragma unroll 4
+        for (int s = nseg - 1; s > seg; --s)
+            x.a[0] = fma(sB[s * cols + lc], x.a[0], sF[s * cols + lc]);
+        with_links<T, NS>(either, [&](auto link) {
+            constexpr int LINK = decltype(link)::value;
+#pragma unroll
+            for (int c = LZ - 1; c >= 0; --c) v[c] = x = back<LINK, T, 1>(g[c], x, v[c]);
+        });
 #pragma unroll
         for (int c = LZ - 1; c >= 0; --c) {
-            x = x + fma(dq[c], x, v[c]);
-            uc[c] = fma(om1, uc[c], omega * x);
+            uc[c] = fma(om1, uc[c], omega * v[c].a[0]);
             if (mine && k0 + c < nz) {
                 if (it + 1 < sweeps)
                     nxt[(k0 + c) * part + lc] = uc[c];
