@@ -307,8 +307,9 @@ int mg_update_fp64(double *x, const float *e, double scale, size_t n, void *stre
  * systems is one persistent-kernel launch over a precomputed work list of
  * (system level, column tile), the batched V-cycle is replayed from one CUDA
  * graph, and converged systems are switched off by device-side flags.  In the
- * mixed solve, systems large enough to fill the GPU by themselves are solved
- * one after the other instead, as by mg_solve_mixed.
+ * mixed solve, systems that fill the GPU by themselves, and middling ones that
+ * are too few to share the lock step, are solved one after the other instead,
+ * as by mg_solve_mixed.
  * mg_batch_setup autotunes the smoother's column-tile width and persistent
  * grid on the batch itself (mg_batch_tuning reports them); the other steps
  * run on persistent grids of as many blocks as the GPU holds at once. */

@@ -108,6 +108,7 @@ struct mg_batch {
     int n = 0;
     mg_params p{};
     std::vector<mg_grid> grids;
+    std::vector<char> own;  // solved on its own in the mixed solve (on_their_own)
     std::vector<mg_handle *> h;
     std::vector<size_t> ws_off;
     int nzmax = 1;
@@ -164,15 +165,39 @@ struct SysOp {
 constexpr long long kBigColumns = 1LL << 18;
 
 // Systems whose mixed solve runs on its own, one after the other, instead of
-// in lock step with the rest: from 2^21 cells a single-system V-cycle fills
-// the GPU on the levels that matter, with kernels of its own (launch bounds,
-// tiles and register budgets per level) where the work lists have one kernel
-// for all sizes, and its iterations need no host.  Mixed solves to 1e-10 in lock
-// step and alone: two of 256 x 192 x 70 (3.4 M cells) 18.4 and 9.5 ms, eight
-// 34.9 and 37.5; eight of 192 x 128 x 70 (1.7 M) 20.1 and 25.6.
-constexpr long long kOwnCells = 1LL << 21;
+// in lock step with the rest: a single-system V-cycle has kernels of its own
+// (launch bounds, tiles and register budgets per level) where the work lists have
+// one kernel for all sizes, and its iterations need no host; the lock step shares
+// the launches of the small levels and costs some 8 ms however few take part.
+// Below kOwnFrom cells a system always takes part, from kOwnAlways it never gains
+// by it.  One between gains about 2.4 ms (1 - cells / kOwnAlways), so they take
+// part together where their missing cells sum up to kLockAlone of kOwnAlways, or to
+// kLockBeside where smaller systems run the lock step in any case.  Mixed solves
+// to 1e-10 in ms, alone and in lock step (70 layers):
+//   256 x 192, 3.4 M cells  2 of them 9.7, 15.1; 6: 28.8, 29.5; 8: 38.5, 36.8; 24: 114, 92.6
+//   320 x 240, 5.4 M        4: 25.3, 30.7; 8: 50.9, 53.1; 16: 101.8, 98.7
+//   384 x 288, 7.7 M        4: 29.4, 38.8; 16: 114.7, 125.3
+//   256 x 192 beside smaller ones  1 of them beside three of 128 x 96 19.6, 23.7; 2
+//     beside one 16.8, 17.1; 3 beside one 20.7, 19.8; 4 beside four of 192 x 128 33.2, 30.7
+constexpr long long kOwnFrom = 1LL << 21, kOwnAlways = 7LL << 20;
+constexpr double kLockAlone = 3.3, kLockBeside = 1.5;
 
-bool on_its_own(const mg_grid &g) { return (long long)g.nlon * g.nlat * g.nz >= kOwnCells; }
+long long cells(const mg_grid &g) { return (long long)g.nlon * g.nlat * g.nz; }
+
+std::vector<char> on_their_own(const std::vector<mg_grid> &grids)
+{
+    double missing = 0;
+    bool beside = false;
+    for (const mg_grid &g : grids) {
+        const long long c = cells(g);
+        if (c < kOwnFrom) beside = true;
+        else if (c < kOwnAlways) missing += 1.0 - (double)c / kOwnAlways;
+    }
+    const bool together = missing >= (beside ? kLockBeside : kLockAlone);
+    std::vector<char> own;
+    for (const mg_grid &g : grids) own.push_back(cells(g) >= (together ? kOwnAlways : kOwnFrom));
+    return own;
+}
 
 // Layers per work item of the cell-type steps: the residual walks whole
 // columns where a level has enough of them (as the single-system path), and
@@ -347,7 +372,7 @@ void build_program(mg_batch *B)
         mg_handle *H = B->h[s];
         LevelHost &f = H->lev[0];
         CgVecs<T> &cg = Vec<T>::cg(H);
-        if (sizeof(T) == 4 && on_its_own(B->grids[s])) continue;
+        if (sizeof(T) == 4 && B->own[s]) continue;
         gen_level<T>(H, s, 0, Lmax, cg.r, cg.z, Vec<T>::w(f), Vec<T>::r(f), phases, B->n);
     }
     P.vsteps.clear();
@@ -690,6 +715,7 @@ static mg_batch *batch_new(int n, const mg_grid *grids, const mg_params *params)
     B->n = n;
     B->p = *params;
     B->grids.assign(grids, grids + n);
+    B->own = on_their_own(B->grids);
     B->h.assign(n, nullptr);
     B->ws_off.assign(n, 0);
     for (int s = 0; s < n; ++s) B->nzmax = std::max(B->nzmax, grids[s].nz);
@@ -1267,11 +1293,11 @@ extern "C" int mg_batch_solve(mg_batch *B, const double *const *b, double *const
         CHK(up(R.ops, R.ops_dev, s));
         CHK(up(R.items, R.items_dev, s));
         CHK(up(R.off, R.off_dev, s));
-        std::vector<mg_stats> own(n, mg_stats{});
+        std::vector<mg_stats> alone(n, mg_stats{});
         for (int i = 0; i < n; ++i) {
-            if (!on_its_own(B->grids[i])) continue;
+            if (!B->own[i]) continue;
             act[i] = 0;
-            st[i] = solve_mixed(B->h[i], b[i], x[i], tol, MG_METHOD_CG, &own[i], s);
+            st[i] = solve_mixed(B->h[i], b[i], x[i], tol, MG_METHOD_CG, &alone[i], s);
             if (st[i] == MG_ERR_CUDA) return st[i];
         }
         const std::vector<int> listed = act;
@@ -1394,7 +1420,7 @@ extern "C" int mg_batch_solve(mg_batch *B, const double *const *b, double *const
             if (listed[i])
                 batch_stats(stats, i, outer[i], its_in[i], relv[i]);
             else
-                batch_stats(stats, i, own[i].iterations, own[i].inner_iterations, own[i].rel_res);
+                batch_stats(stats, i, alone[i].iterations, alone[i].inner_iterations, alone[i].rel_res);
         }
     }
     int first = MG_OK;
