@@ -1211,7 +1211,8 @@ extern "C" int mg_batch_setup(int n, const mg_grid *grids, const mg_coeffs *coef
     build_vector_plans<double>(B);
     if ((st = upload_plan<double>(B->p64, s)) != MG_OK) return bail(st);
     if (B->p.mixed && (st = upload_plan<float>(B->p32, s)) != MG_OK) return bail(st);
-    if (B->p.mixed) st = autotune<float>(B, s);
+    // on the FP32 sweeps, or the FP64 ones where no FP32 solve takes the work lists
+    if (B->p.mixed && std::count(B->own.begin(), B->own.end(), 0)) st = autotune<float>(B, s);
     else st = autotune<double>(B, s);
     if (st != MG_OK) return bail(st);
     if ((st = rebuild_items<double>(B, s)) != MG_OK) return bail(st);

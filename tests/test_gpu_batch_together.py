@@ -5,7 +5,7 @@ these systems times that)."""
 import pytest
 import torch
 
-from gpu_common import dev, problem, rel_2, host
+from gpu_common import dev, host, problem, rel_2
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +31,20 @@ def test_many_of_middle_size():
     for i, (x, info) in enumerate(zip(xs, infos)):
         assert info["status"] == 0 and info["rel_res"] <= 1e-9
         assert rel_2(host(x), host(alone[i % 2])) <= 1e-7
+
+
+def test_work_lists_tuned_without_fp32_members():
+    """A batch whose FP32 solves all run on their own still times its work lists
+    (the FP64 ones) at setup: at least eight widths and grids, four launches each."""
+    from paper_2307_04528_gb300.solver import MGBatch, MGHandle
+    p = problem(256, 128, 65, sigma=0.1, seed=70)
+    fields = tuple(dev(p[k]) for k in ("tx", "ty", "tz", "h"))
+    n0 = launches()
+    MGHandle(*fields, mixed=1)
+    handle = launches() - n0
+    n0 = launches()
+    B = MGBatch([fields], mixed=1)
+    assert launches() - n0 >= handle + 32
+    b = dev(p["b"])
+    x, info = B.solve([b], tol=1e-9, mixed=0)
+    assert info[0]["status"] == 0 and info[0]["rel_res"] <= 1e-9
