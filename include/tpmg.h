@@ -285,6 +285,12 @@ int mg_level_prolong_add(mg_handle *h, int level, int prec, const void *ec, void
  * scaled (FP32 level l holds c * coefficients); 0 when not built. */
 double mg_fp32_scale(const mg_handle *h);
 
+/* 1 when the conjugate-gradient iterations of that precision have run as a loop
+ * on the device (built by the first solve that takes it), 0 when every solve so
+ * far was driven by the host: while profiling, from an FP32 x off its 16-byte
+ * boundary, or where the driver refuses the graph. */
+int mg_device_loop(const mg_handle *h, int prec);
+
 /* The precision changes of the mixed-precision refinement (Section 1:
  * single-precision multigrid; the outer residual and the update in double
  * precision), on n device values, stream-ordered, no handle needed.

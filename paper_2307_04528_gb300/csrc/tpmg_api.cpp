@@ -1487,6 +1487,11 @@ extern "C" int mg_level_shape(const mg_handle *H, int level, int *nlon, int *nla
 
 extern "C" double mg_fp32_scale(const mg_handle *H) { return H ? H->scale32 : 0.0; }
 
+extern "C" int mg_device_loop(const mg_handle *H, int prec)
+{
+    return H && (prec == MG_PREC_FP64 || prec == MG_PREC_FP32) && H->loop[prec].exec ? 1 : 0;
+}
+
 // ------------------------------------------------------------------ C ABI: precision changes
 static int conv_check(const void *a, const void *b, double scale, size_t n)
 {

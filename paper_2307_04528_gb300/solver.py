@@ -103,6 +103,11 @@ class MGHandle:
     def fp32_scale(self) -> float:
         return float(self.lib.mg_fp32_scale(self._hh))
 
+    def device_loop(self, prec=L.MG_PREC_FP64) -> bool:
+        """Whether a solve's conjugate-gradient iterations have run as a loop on the
+        device in that precision."""
+        return bool(self.lib.mg_device_loop(self._hh, prec))
+
     # ------------------------------------------------------------- fine level
     def apply(self, x, y=None):
         _field(x, torch.float64, self.shape, "x")
