@@ -132,31 +132,27 @@ k_dir_quad(LevelDev<float> L, const float *__restrict__ z, const float *__restri
     block_store_at<0>((double)acc, partial, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-int g_dir_sms = 152;
-
 struct Shape {
     int gx, gy, kz;
 };
 
-// Blocks along the columns, and the layers split until there are two waves
-// of four blocks per SM.
+// Blocks along the columns, and the layers split until there are two waves of
+// four blocks per SM: of a fixed number of SMs, since a batch lays out its
+// partial sums (dir_quad_blocks) before it asks for a device.
+constexpr long long kFillBlocks = 8 * 152;
+
 Shape shape_of(const LevelDev<float> &L)
 {
     Shape s;
     s.gx = (int)(((long long)(L.nlon / 4) * L.nlat + kBlock - 1) / kBlock);
     s.kz = L.nz;
-    while (s.kz > 8 && (long long)s.gx * ((L.nz + s.kz - 1) / s.kz) < 8LL * g_dir_sms)
+    while (s.kz > 8 && (long long)s.gx * ((L.nz + s.kz - 1) / s.kz) < kFillBlocks)
         s.kz = (s.kz + 1) / 2;
     s.gy = (L.nz + s.kz - 1) / s.kz;
     return s;
 }
 
 }  // namespace
-
-void dir_prepare(int sms)
-{
-    if (sms > 0) g_dir_sms = sms;
-}
 
 int dir_quad_blocks(const LevelDev<float> &L, const float *z, const float *d_old,
                     const float *d_new, const float *q)

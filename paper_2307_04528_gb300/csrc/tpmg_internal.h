@@ -153,8 +153,6 @@ int dir_quad_blocks(const LevelDev<float> &L, const float *z, const float *d_old
 int launch_dir_quad(const LevelDev<float> &L, const float *z, const float *d_old,
                     const CgScalars *sc, float *d_new, float *q, double *partial, cudaStream_t s,
                     const int *flag, const CgLoop *loop);
-// Records the SM count.
-void dir_prepare(int sms);
 
 // The FP64 stencil with a thread per 2 x 2 columns (tpmg_stencil.cu; the
 // values of launch_stencil): the number of blocks (and partial sums), or -1

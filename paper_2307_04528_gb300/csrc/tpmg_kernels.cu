@@ -319,7 +319,6 @@ cudaError_t smooth_prepare()
         return e;
     if (sms > 0) g_sms = sms;
     stencil_prepare(sms);
-    dir_prepare(sms);
     if (lim > 0) g_smem_optin = lim;
     const void *kernels[] = {(const void *)k_smooth<double>,     (const void *)k_smooth<float>,
                              (const void *)k_smooth0<double>,    (const void *)k_smooth0<float>,
