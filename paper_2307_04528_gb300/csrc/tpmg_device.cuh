@@ -381,7 +381,10 @@ __device__ __forceinline__ T whole(T g, T x)
 template <typename T>
 __device__ __forceinline__ T link(T g, T x, T y)
 {
-    return fma(g, x, y) + whole(g, x);
+    // FP32: one where g is f - 1, else zero, as a saturated product (a select sits in the
+    // serial chain of the walk; 129 x 66 x 70 on a guess: 15.3 -> 13.6 us)
+    if constexpr (sizeof(T) == 4) return fma(__saturatef(g * -0x1p127f), x, fma(g, x, y));
+    else return fma(g, x, y) + whole(g, x);
 }
 
 // One sweep of Eq. (1), u_out = (1 - omega) u_in + omega H_z^{-1}(b - dH u_in),
