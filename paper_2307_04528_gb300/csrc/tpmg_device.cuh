@@ -1067,11 +1067,12 @@ __device__ __forceinline__ typename Pair<T>::type ld_pair(const T *p)
 }
 
 // The same of a vector that the kernel before this one may have written
-// (after_previous).
-template <typename T>
+// (after_previous; OWN false: that is complete).
+template <bool OWN = true, typename T>
 __device__ __forceinline__ typename Pair<T>::type ld_pair_of(const T *p)
 {
-    return *reinterpret_cast<const typename Pair<T>::type *>(p);
+    if constexpr (OWN) return *reinterpret_cast<const typename Pair<T>::type *>(p);
+    else return ld_pair(p);
 }
 
 // a_d += w v of three open sums, d warp-uniform.  FP64: one operation on the
@@ -1118,6 +1119,9 @@ __device__ __forceinline__ void add_open(T w, T v, int d, T &a0, T &a1, T &a2)
 // omega b cancels everything else; om1 = 1 - omega): the same walk without
 // h, t_z and the layers above and below, terms added east, west, north,
 // south.
+// The full form, ten arrays to a row, wants the freedom that read-only loads of b
+// and u leave the compiler (512 x 384 x 76 in FP32: 84 us, 124 with ordinary ones);
+// its kernel waits for the one before it in the ordinary way.
 // Level: LevelDev, or (PRE) NsView, whose couplings from the west and the
 // south are arrays of their own.
 template <typename T, bool PRE = false, typename Level = LevelDev<T>>
@@ -1152,9 +1156,9 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
     T a0 = 0, a1 = 0, a2 = 0;                              // rows Jlo, Jlo + 1, Jlo + 2
     P2 zero;
     zero.x = zero.y = T(0);
-    P2 Us = jfirst > 0 ? ld_pair_of(uk + (size_t)(jfirst - 1) * nf) : zero;
+    P2 Us = jfirst > 0 ? ld_pair_of<PRE>(uk + (size_t)(jfirst - 1) * nf) : zero;
     P2 Tys = jfirst > 0 ? ld_pair(sk + (size_t)(jfirst - 1) * nf) : zero;
-    P2 Uc = ld_pair_of(uk + (size_t)jfirst * nf);
+    P2 Uc = ld_pair_of<PRE>(uk + (size_t)jfirst * nf);
     // The PRE form has little arithmetic per row to cover its loads, so it
     // issues the next row's loads (u and t_y one row north, b and t_x on the
     // row) before combining this one: two rows in flight per thread (FP64, all
@@ -1164,8 +1168,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
     P2 nUn = zero, nB = zero, nTX = zero, nTYN = zero, nTW = zero, nTS = zero;
     if (kAhead) {
         const size_t o0 = (size_t)jfirst * nf;
-        nUn = jfirst + 1 < nlat ? ld_pair_of(uk + o0 + nf) : zero;
-        nB = ld_pair_of(bk + o0);
+        nUn = jfirst + 1 < nlat ? ld_pair_of<PRE>(uk + o0 + nf) : zero;
+        nB = ld_pair_of<PRE>(bk + o0);
         nTX = ld_pair(txk + o0);
         nTYN = jfirst + 1 < nlat ? ld_pair(tyk + o0) : zero;
         if (NS) {
@@ -1190,8 +1194,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
             if (j < jlast) {
                 const size_t o1 = oj + nf;
                 const bool n1 = j + 2 < nlat;
-                nUn = n1 ? ld_pair_of(uk + o1 + nf) : zero;
-                nB = ld_pair_of(bk + o1);
+                nUn = n1 ? ld_pair_of<PRE>(uk + o1 + nf) : zero;
+                nB = ld_pair_of<PRE>(bk + o1);
                 nTX = ld_pair(txk + o1);
                 nTYN = n1 ? ld_pair(tyk + o1) : zero;
                 if (NS) {
@@ -1200,8 +1204,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
                 }
             }
         } else {
-            Un = hasN ? ld_pair_of(uk + oj + nf) : zero;
-            B = ld_pair_of(bk + oj);
+            Un = hasN ? ld_pair_of<PRE>(uk + oj + nf) : zero;
+            B = ld_pair_of<PRE>(bk + oj);
             TX = ld_pair(txk + oj);
             TYN = hasN ? ld_pair(tyk + oj) : zero;
             if (NS) {
@@ -1231,8 +1235,8 @@ __device__ __forceinline__ void resid_restrict_band(const Level &F, const LinkDe
         } else {
             const P2 Hh = ld_pair(hk + oj), TZ = ld_pair(tzk + oj);
             const P2 TZD = dn ? ld_pair(tzd + oj) : zero;
-            const P2 UU = up ? ld_pair_of(uu + oj) : zero;
-            const P2 UD = dn ? ld_pair_of(ud + oj) : zero;
+            const P2 UU = up ? ld_pair_of<PRE>(uu + oj) : zero;
+            const P2 UD = dn ? ld_pair_of<PRE>(ud + oj) : zero;
             T v0 = Hh.x * Uc.x;
             v0 = fma(TX.x, Uc.x - Uc.y, v0);
             v0 = fma(txw, Uc.x - uw, v0);

@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kBlock, (PRE && sizeof(T) == 4) ? 12 : 0)
 k_resid_restrict(LevelDev<T> F, LinkDev K, const T *b, const T *u, T *__restrict__ bc, T om1,
                  int band0, int band, const int *flag)
 {
-    after_previous();
+    if (PRE) after_previous();
     if (flag && !*flag) return;
     const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     if (warp * kRROwned >= F.nlon / 2) return;  // whole warps
@@ -450,8 +450,8 @@ cudaError_t launch_resid_restrict(const LevelDev<T> &F, const LinkDev &K, const 
             launch_after(k_resid_restrict<T, true>, grid, kBlock, 0, s, F, K, b, u, bc, om1, band0,
                          band, flag);
         else
-            launch_after(k_resid_restrict<T, false>, grid, kBlock, 0, s, F, K, b, u, bc, om1, band0,
-                         band, flag);
+            k_resid_restrict<T, false><<<grid, kBlock, 0, s>>>(F, K, b, u, bc, om1, band0, band,
+                                                               flag);
     }
     return cudaGetLastError();
 }
