@@ -156,18 +156,25 @@ k_stencil_cells(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ x,
 
 // below this many columns the column loops cannot fill the GPU
 constexpr int kCellParallelColumns = 32768;
+// Below this many cells the threads of 2 x 2 columns leave FP64 pipes idle: without an
+// inner product a thread takes a cell.  FP64 apply by cells and by quads: 64 x 32 x 16
+// 2.5 and 9.1 us, 48 x 82 x 70 8.5 and 11.6, 96 x 80 x 33 7.9 and 11.4, 256 x 192 x 3
+// 5.3 and 6.9; from 128 x 64 x 70 (15.2 and 16.1; launched directly 17.4 and 16.7) to
+// 256 x 126 x 20 (17.0 and 16.2; 19.1 and 16.7) the quads' early launch decides.
+constexpr long long kQuadCells = 1LL << 19;
 
 template <typename T>
 int launch_stencil(const LevelDev<T> &L, int mode, const T *b, const T *x, T *y, double *partial,
                    cudaStream_t s, const int *flag)
 {
-    if constexpr (sizeof(T) == 8) {
-        const int blocks = launch_stencil_quad(L, mode, b, x, y, partial, s, flag);
-        if (blocks >= 0) return partial ? blocks : 0;
-    }
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
-    if (!partial && ncol < kCellParallelColumns) {
+    const bool few = sizeof(T) == 8 && !partial && (long long)ncol * L.nz < kQuadCells;
+    if constexpr (sizeof(T) == 8) {
+        const int blocks = few ? -1 : launch_stencil_quad(L, mode, b, x, y, partial, s, flag);
+        if (blocks >= 0) return partial ? blocks : 0;
+    }
+    if (!partial && (few || ncol < kCellParallelColumns)) {
         const dim3 g2(grid, L.nz);
         if (mode) k_stencil_cells<T, 1><<<g2, kBlock, 0, s>>>(L, b, x, y, flag);
         else k_stencil_cells<T, 0><<<g2, kBlock, 0, s>>>(L, b, x, y, flag);
