@@ -228,10 +228,36 @@ ClusterShape cluster_shape(int nlon, int nlat, int nz)
     return c;
 }
 
+// Layers a block of shape S holds for nz, its empty slots and segments included.
+template <typename S>
+int slots_of(int nz)
+{
+    return threads_of<S>(nz) / S::QL * S::LZ;
+}
+
+// Whether an FP64 level of at most 8192 columns sweeps by segments (slots: of the long
+// segments, 0: of the short ones) rather than by the column walk.  The walk takes its
+// serial chain, some 1.8 + 0.25 nz us from zero and 1.7 + 0.61 nz on a guess whatever
+// the columns; the segments their FP64 operations, empty slots included, about 3.5 +
+// 2.1e-5 us a slot from zero (3e-5 beyond 800,000) and 5 + 4.4e-5 on a guess.  In us,
+// segments and walk: 128 x 64 x 16 from zero 8.1 and 5.8, on a guess 11.4 and 9.7;
+// x 70 15.0 and 19.3, 25.0 and 43.0; x 76 26.4 and 20.7, 39 and 47; 64 x 98 x 50 12.9
+// and 14.3, 20.9 and 31.2.  A Chebyshev step is weighed against the walk, the residual
+// by cells and the vector update (7 of them, 96 x 80 x 50: 292 and 236 us; x 70: 294
+// and 306).
+bool fp64_segments(long long ncol, int nz, int slots, bool guess, bool cheb)
+{
+    if (slots == 0) return cheb || nz > 4;  // 32 x 32 x 4: 3.1 and 2.7 us, x 6 3.1 and 3.4
+    const double s = (double)ncol * slots;
+    if (cheb) return 6.0 * s < 2.5e5 + 2.5e4 * nz + 2.7 * (double)ncol * nz;
+    if (guess) return s < 13900.0 * nz - 75000.0;
+    return s < std::min(12000.0 * nz - 80000.0, 8200.0 * nz + 52000.0);
+}
+
 // The shape for a level and its buffers, or -1 where the column walk is the
 // faster form: FP64 levels beyond 8192 columns (the maps cost 16 FP64
-// operations per cell against 10, and the walk is bound by the FP64 pipe),
-// FP32 levels that fill the GPU with rows of no whole quad, and layer counts
+// operations per cell against 10, and the walk is bound by the FP64 pipe) or of
+// few layers (fp64_segments), FP32 levels that fill the GPU with rows of no whole quad, and layer counts
 // beyond the shapes' registers.
 template <typename T, typename Level>
 int pick(const Level &L, const Sweep<T> &a)
@@ -246,7 +272,12 @@ int pick(const Level &L, const Sweep<T> &a)
                            (a.ch ? (uintptr_t)a.ch->r_out | (uintptr_t)a.ch->x : 0);
     if constexpr (sizeof(T) == 8) {
         if (ncol > kMidColumns) return -1;
-        if (ncol * L.nz >= 1 << 16 && suits<T, Mid64>(L, ptrs)) return go<T, Mid64>(L, a);
+        const bool mid = ncol * L.nz >= 1 << 16 && suits<T, Mid64>(L, ptrs);
+        if constexpr (!kDirected<Level>)
+            if (!fp64_segments(ncol, L.nz, mid ? slots_of<Mid64>(L.nz) : 0, a.uin != nullptr,
+                               a.ch != nullptr))
+                return -1;
+        if (mid) return go<T, Mid64>(L, a);
     } else if (ncol < kMidColumns) {
         if (ncol >= kSmallColumns && suits<T, Mid>(L, ptrs)) return go<T, Mid>(L, a);
     } else if constexpr (kDirected<Level>) {

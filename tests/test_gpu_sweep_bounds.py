@@ -41,6 +41,14 @@ def test_walks(shape):
         assert abs(dot - O.dot(b, guess)) <= tol * O.norm2(b) * O.norm2(guess)
 
 
+# FP64 on either side of the line between segments and walk, by layers and by columns
+@pytest.mark.parametrize("shape", [(32, 32, 4), (32, 32, 5), (64, 64, 16), (96, 80, 10),
+                                   (64, 98, 50), (96, 80, 50), (128, 64, 70)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_fp64_segments_and_walk(shape):
+    test_walks(shape)
+
+
 # rows of eight blocks that just fit and just do not: 70 layers in 9 segments (FP32) and
 # 18 (FP64), 100 layers in 9 and 17, one and two layers
 @pytest.mark.parametrize("shape", [(8, 56, 70), (8, 58, 70), (14, 32, 70), (10, 16, 70),
