@@ -409,22 +409,21 @@ bool resid_restrict_fits(const void *b, const void *u, size_t value_bytes)
 // Coarse rows per band of the fused residual + restriction: the widest band
 // (of kRRBand, 4, 2, 1) whose warps still make two waves of 48 per SM.  FP64,
 // bound by the operations spent on band-edge rows that are formed twice,
-// starts from 2 kRRBand and narrows only below 16 warps per SM (256 x 128 x
-// 32: bands of one row would form every fine row 2.4 times).
+// narrows only below 16 warps per SM (256 x 128 x 32: bands of one row would
+// form every fine row 2.4 times), and takes 2 kRRBand where the last of so long
+// bands do not leave SMs idle: from 24 warps per SM after one sweep (256 x 192 x
+// 70, 18 warps: 100 -> 80 us with kRRBand; 384 x 256 x 50, 25: 98 and 101; 1024 x
+// 768 x 70 922 and 954), from 96 in full (512 x 384 x 70, 66 warps: 536 and 530 us;
+// 384 x 256 x 50 237 and 208; 1024 x 768 x 70, 250: 1980 and 2047).
 template <typename T>
-static int rr_band(int nlon, int nz, const LinkDev &K)
+static int rr_band(int nlon, int nz, const LinkDev &K, bool presmooth)
 {
-    const long long warps = (nlon / 2 + kRROwned - 1) / kRROwned;
-    const long long enough = (sizeof(T) == 8 ? 16LL : 2LL * 48) * g_sms;
-    int band = sizeof(T) == 8 ? 2 * kRRBand : kRRBand;
-    while (band > 1 && warps * nz * ((K.nlat_c + band - 1) / band) < enough) band /= 2;
+    const long long warps = (nlon / 2 + kRROwned - 1) / kRROwned * (long long)nz;
+    auto per_sm = [&](int band) { return warps * ((K.nlat_c + band - 1) / band) / g_sms; };
+    if (sizeof(T) == 8 && per_sm(2 * kRRBand) >= (presmooth ? 24 : 96)) return 2 * kRRBand;
+    int band = kRRBand;
+    while (band > 1 && per_sm(band) < (sizeof(T) == 8 ? 16 : 2 * 48)) band /= 2;
     return band;
-}
-
-template <typename T>
-int rr_band(const LevelDev<T> &F, const LinkDev &K)
-{
-    return rr_band<T>(F.nlon, F.nz, K);
 }
 
 template <typename T>
@@ -432,7 +431,7 @@ cudaError_t launch_ns_presmooth_restrict(const NsView<T> &F, const LinkDev &K, c
                                          const T *u, T *bc, double omega, cudaStream_t s)
 {
     const int warps = (F.nlon / 2 + kRROwned - 1) / kRROwned;
-    const int band = rr_band<T>(F.nlon, F.nz, K), bands = (K.nlat_c + band - 1) / band;
+    const int band = rr_band<T>(F.nlon, F.nz, K, true), bands = (K.nlat_c + band - 1) / band;
     for (int band0 = 0; band0 < bands; band0 += 65535) {  // grid z limit
         const dim3 grid((warps * 32 + kBlock - 1) / kBlock, F.nz, std::min(65535, bands - band0));
         launch_after(k_ns_presmooth_restrict<T>, grid, kBlock, 0, s, F, K, b, u, bc,
@@ -448,7 +447,7 @@ cudaError_t launch_resid_restrict(const LevelDev<T> &F, const LinkDev &K, const 
 {
     const int nc = F.nlon / 2;
     const int warps = (nc + kRROwned - 1) / kRROwned;
-    const int band = rr_band(F, K);
+    const int band = rr_band<T>(F.nlon, F.nz, K, presmooth);
     const int bands = (K.nlat_c + band - 1) / band;
     const T om1 = T(1) - (T)omega;
     for (int band0 = 0; band0 < bands; band0 += 65535) {  // grid z limit
@@ -1182,7 +1181,6 @@ cudaError_t launch_coeff_grad(int nlon, int nlat, int nz, const double *lam, con
     template cudaError_t launch_resid_restrict<T>(const LevelDev<T> &, const LinkDev &, const T *, \
                                                   const T *, T *, cudaStream_t, const int *, bool, \
                                                   double);                                        \
-    template int rr_band<T>(const LevelDev<T> &, const LinkDev &);                                 \
     template cudaError_t launch_ns_presmooth_restrict<T>(const NsView<T> &, const LinkDev &,       \
                                                          const T *, const T *, T *, double,        \
                                                          cudaStream_t);                            \
