@@ -711,7 +711,7 @@ static int coarse_chebyshev(mg_handle *H, int l, const LevelDev<T> &D, const T *
     const int m = H->p.coarse_iters;
     // One launch per step where the segmented sweeps take the level: the
     // residual r - H d, the column solve and the updates of d and x in one pass
-    // over two copies of d and of r (64 x 98 x 70 in FP32: 4.7 us a step, against
+    // over two copies of d and of r (64 x 86 x 70 in FP32: 4.6 us a step, against
     // 10.1 as three kernels).  The terms and their order are the separate
     // kernels'.  (Carrying x instead of r, z = H_z^{-1}(b + the horizontal
     // couplings of x) - x, took 4.4 us, but the difference lost a factor of 4
@@ -904,9 +904,10 @@ static int bicg_precond(mg_handle *H, int slot, const T *in, T *out, cudaStream_
     if (H->p.method == MG_METHOD_BICGSTAB) return vcycle_graph<T>(H, slot, in, out, s, nullptr);
     LevelHost &f = H->lev[0];
     if constexpr (sizeof(T) == 8) {
-        // FP64 runs to the rounding floor of a line-relaxed Krylov method, whose
-        // attainable accuracy hangs on the preconditioner's roundings: the
-        // column walk, with the same roundings at every size
+        // The column walk at every size: at a residual of 5e-12 the solution of a
+        // line-relaxed Krylov solve is good to 1e-11 to 4e-10 (eight systems of 64 x
+        // 32 x 16 and 96 x 46 x 9; with the walk and with the segments alike), by the
+        // roundings of the preconditioner, which so stay the same at every size
         const LevelDev<T> D = dev<T>(f);
         const int sweeps = H->p.line_sweeps;
         T *cur = (sweeps % 2 == 1) ? out : Vec<T>::w(f), *oth = (cur == out) ? Vec<T>::w(f) : out;

@@ -580,34 +580,31 @@ __device__ __forceinline__ void smooth_column(const LevelDev<T> &L, const T *__r
     }
 }
 
-// ------------------------------------------------------------------ warp sweep
-// One column of the sweep of Eq. (1) solved by a whole warp, for the small
-// coarse levels, where one thread per column leaves the GPU waiting on the
-// 2 nz dependent steps of the column recurrences.  Lane l owns layers
-// [l C, l C + C), C = ceil(nz / 32).  Both recurrences are first-order and
-// linear, so they run as warp scans of affine maps:
+// ------------------------------------------------------------------ warp scan
+// One column solved by a whole warp, for the coarsest levels of a batch
+// (coarse_solve_sh), where one thread per column would wait on the 2 nz
+// dependent steps of the column recurrences.  Lane l owns layers [l C, l C + C),
+// C = ceil(nz / 32).  Both recurrences are first-order and linear, so they run
+// as warp scans of affine maps:
 //   forward   y_k = (v_k + t_{k-1} y_{k-1}) / p_k  = (t_{k-1}/p_k) y_{k-1} + v_k/p_k
 //   backward  x_k = y_k + f_k x_{k+1}      (x_nz = 0)
 // Each lane composes the maps of its layers, a Kogge-Stone scan across the
 // lanes gives each lane the value entering its layers, and the lane then
 // re-runs its own layers with the serial formulas of smooth_column.  The
-// values differ from the serial sweep only by rounding.  u_in is read with
-// ordinary (coherent) loads, so a block may read what its own earlier sweep
-// wrote after a block barrier.  All 32 lanes must call it with the same
-// col < ncol.
+// values differ from the serial sweep only by rounding.  All 32 lanes must call
+// it for the same column.
 constexpr int kWarpLayers = (kMaxLayers + 31) / 32;  // layers per lane at most
-// CM: the layers per lane the code is unrolled for (ceil(nz / 32) <= CM <=
-// kWarpLayers; the launchers take the smallest of 2, 3, kWarpLayers that
-// holds the level, so no predicated-off layer slots are issued).
 
-// The two scans of the warp sweep over one lane's layers k0 .. k0 + C - 1:
+// The two scans over one lane's layers k0 .. k0 + C - 1:
 // v holds the right-hand sides v_k on entry and the column solution x_k of
 // H_z x = v on return; tprev = t_{k0-1} (0 for the first lane).
-template <typename T, int CM>
-__device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], const T (&m)[CM],
-                                                 const T (&g)[CM], T tprev, int C, int k0,
+template <typename T>
+__device__ __forceinline__ void warp_column_scan(T (&v)[kWarpLayers], const T (&tz)[kWarpLayers],
+                                                 const T (&m)[kWarpLayers],
+                                                 const T (&g)[kWarpLayers], T tprev, int C, int k0,
                                                  int nz, int lane)
 {
+    constexpr int CM = kWarpLayers;
     // forward: this lane's map y_out = A y_in + Cy, then an inclusive scan
     T A = 1, Cy = 0, tp = tprev;
 #pragma unroll
@@ -679,10 +676,11 @@ __device__ __forceinline__ void warp_column_scan(T (&v)[CM], const T (&tz)[CM], 
 // kCoarseShArrays * ncol * nz values of dynamic shared memory.
 constexpr int kCoarseShArrays = 8;
 
-template <typename T, int CM = kWarpLayers>
+template <typename T>
 __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *__restrict__ b,
                                                 T *__restrict__ out, T omega, int sweeps, T *sh)
 {
+    constexpr int CM = kWarpLayers;
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat, n = ncol * nz;
     T *sb = sh, *stz = sh + n, *sm = sh + 2 * n, *sg = sh + 3 * n, *stx = sh + 4 * n,
@@ -730,7 +728,7 @@ __device__ __forceinline__ void coarse_solve_sh(const LevelDev<T> &L, const T *_
                 }
             }
             const T tprev = (k0 >= 1 && k0 - 1 < nz) ? stz[oc + k0 - 1] : T(0);
-            warp_column_scan<T, CM>(v, tz, m, g, tprev, C, k0, nz, lane);
+            warp_column_scan<T>(v, tz, m, g, tprev, C, k0, nz, lane);
 #pragma unroll
             for (int c = 0; c < CM; ++c) {
                 const int k = k0 + c;

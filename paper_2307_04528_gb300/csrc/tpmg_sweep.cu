@@ -1,5 +1,5 @@
-// Launchers of the segmented sweeps (tpmg_sweep.cuh) and of the one-block
-// coarsest-level solve, and the rules that pick a shape for a level.
+// Launchers of the segmented sweeps (tpmg_sweep.cuh) and of the coarsest-level
+// solve on a thread-block cluster, and the rules that pick a shape for a level.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -15,7 +15,7 @@ namespace {
 // A block takes the tiles blockIdx, + gridDim, ...: one, unless a level has
 // more tiles than there are slots for partial sums.  (The loop also has the
 // compiler issue a tile's loads in one run: 0.534 ms against 0.698 without it
-// at 1536 x 1152 x 70, the same instructions otherwise.)
+// at 1536 x 1152 x 70, the same instructions otherwise, on q/p alone.)
 template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB,
           typename Level>
 __global__ void __launch_bounds__(MAXT, MINB)
@@ -58,30 +58,31 @@ struct Shape {
     static constexpr bool GUESS = GUESS_;  // false: sweeps from zero only
 };
 
-// FP32 levels that fill the GPU.  From zero the sweep reads b, 1/p and q/p and
-// is bound by HBM: pairs of columns in 256-byte rows (1536 x 1152 x 70: 0.480
-// -> 0.274 ms, 7.2 TB/s; quads 0.290, single columns 0.316).  On a guess a
-// thread also reads five arrays around it, and instructions bind beside HBM:
-// quads of columns (16-byte loads), 64 columns to a block of 128 threads so
-// that two blocks share an SM (0.777 -> 0.534 ms, 6.5 TB/s; with <b, u_out>
-// 0.817 -> 0.627; one block of 256 threads 0.584 / 0.659, pairs 0.77 / 1.04).
+// FP32 levels that fill the GPU.  From zero the sweep reads b, 1/p and g and is
+// bound by HBM: pairs of columns in 256-byte rows (1536 x 1152 x 70: 0.480 ->
+// 0.278 ms, 7.1 TB/s; quads and single columns, on q/p alone, 0.290 and 0.316
+// against 0.274).  On a guess a thread also reads five arrays around it, and
+// instructions bind beside HBM: quads of columns (16-byte loads), 64 columns to
+// a block of 128 threads so that two blocks share an SM (0.777 -> 0.560 ms, 6.2
+// TB/s; with <b, u_out> 0.817 -> 0.653; on q/p alone 0.534 and 0.627, one block
+// of 256 threads 0.584 and 0.659, pairs 0.77 and 1.04).
 using Large0 = Shape<2, 9, 32, 256, 3, false>;
 using Large = Shape<4, 9, 16, 128, 2>;
 // the same with segments of 5 layers, for layer counts that leave fewer of
-// their slots empty (256 x 192 x 50: 10.7 -> 9.3 us; 352 x 226 x 37: 17.1 -> 12.2)
+// their slots empty (256 x 192 x 50: 10.7 -> 9.2 us; 352 x 226 x 37: 17.1 -> 11.7)
 using Large5 = Shape<4, 5, 16, 256, 2>;
 // rows that are no multiple of 2 columns (only from zero: 0.316 ms as above)
 using Odd0 = Shape<1, 9, 32, 256, 4, false>;
 // Levels of 2048 to 8192 columns in FP32: latency; 32 columns to a block
-// (48 x 82 x 70 on a guess: 13.5 -> 3.3 us, Large 3.6)
+// (48 x 82 x 70 on a guess: 13.5 -> 3.2 us, Large 3.6)
 using Mid = Shape<2, 5, 16, 256, 2>;
 // Small levels: 8 columns to a block, short segments (24 x 46 x 70 on a guess:
-// FP32 4.7 -> 3.0 us, Mid 3.2; 8 x 18 x 70 in FP64: 43 -> 6.2 us)
+// FP32 4.7 -> 2.8 us, Mid 3.2; 8 x 18 x 70 in FP64: 43 -> 6.2 us)
 using Small = Shape<1, 3, 8, 192, 1>;
 using SmallTall = Shape<1, 3, 8, 512, 1>;  // more than 72 layers
 // FP64 levels from 2^16 cells to 8192 columns, where the extra FP64 operations
 // of the exchanged maps begin to count: long segments (64 x 98 x 70 on a guess:
-// 43.8 -> 20.3 us, Small 26.2; 64 x 32 x 16: 9.6 -> 7.6, Small 4.1)
+// 43.8 -> 21.2 us, Small 26.2; 64 x 32 x 16: 9.6 -> 7.6, Small 4.4)
 using Mid64 = Shape<1, 9, 8, 192, 1>;
 
 // Directed FP32 levels that fill the GPU: one more array per layer in
@@ -257,8 +258,9 @@ bool fp64_segments(long long ncol, int nz, int slots, bool guess, bool cheb)
 // The shape for a level and its buffers, or -1 where the column walk is the
 // faster form: FP64 levels beyond 8192 columns (the maps cost 16 FP64
 // operations per cell against 10, and the walk is bound by the FP64 pipe) or of
-// few layers (fp64_segments), FP32 levels that fill the GPU with rows of no whole quad, and layer counts
-// beyond the shapes' registers.
+// few layers (fp64_segments), FP32 levels that fill the GPU with rows of no
+// whole quad, and layer counts beyond the shapes' threads (FP32 levels that fill
+// the GPU: 72, or 75 by segments of 5).
 template <typename T, typename Level>
 int pick(const Level &L, const Sweep<T> &a)
 {
@@ -327,7 +329,7 @@ int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *uin, T *uout)
 
 // Levels whose rows fit eight blocks' threads take the cluster (up to 448
 // columns of 70 layers in FP32, 168 in FP64).  Per sweep, FP32: 1.35 us at 11
-// x 18 x 37 and 1.7 us at 6 x 14 x 70, against 4.5 and 4.1 us for one block
+// x 18 x 37 and 1.8 us at 6 x 14 x 70, against 4.5 and 4.1 us for one block
 // with the level's factors in registers and ~3 us for a launch per sweep.
 template <typename T>
 bool coarse_solve_fits(int nlon, int nlat, int nz)
