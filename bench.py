@@ -221,13 +221,13 @@ def run_reference(args):
 # (reads + writes of distinct arrays; horizontal neighbours counted once)
 KERNEL_WORDS = {
     # (kind, prec): (name, words per cell)
-    (0, 1): ("smooth fp32 (+ <r, z>)", 7),            # u b tx ty m dq -> u
-    (1, 1): ("smooth fp32 zero guess", 4),            # b m dq -> u
+    (0, 1): ("smooth fp32 (+ <r, z>)", 7),            # u b tx ty m g -> u
+    (1, 1): ("smooth fp32 zero guess", 4),            # b m g -> u
     (2, 1): ("residual + restriction fp32", 6),       # u b tx ty tz h -> b_c (+ coarse write;
                                                       # u b tx ty after a sweep from zero)
     (3, 1): ("direction update + apply fp32", 8),     # z d tx ty tz h -> d q
     (5, 1): ("prolongation + correction fp32", 2),    # u e_c -> u (+ coarse read)
-    (0, 0): ("smooth fp64", 8),                       # u b tx ty tz m dq -> u
+    (0, 0): ("smooth fp64", 8),                       # u b tx ty tz m g -> u
     (1, 0): ("smooth fp64 zero guess", 5),
     (2, 0): ("residual fp64 -> scaled fp32", 6.5),    # x b tx ty tz h -> r32
     (3, 0): ("apply fp64", 6),
@@ -235,12 +235,12 @@ KERNEL_WORDS = {
 
 
 # DRAM bytes per fine cell of one launch of the FP32 sweep with <r, z> (ncu
-# capture at 512x384x70: 330.3 MB read + 40.7 MB written for 13,762,560 cells)
-SMOOTH_DOT_DRAM_BYTES_PER_CELL = (330.349056e6 + 40.736e6) / (512 * 384 * 70)
+# capture at 512x384x70: 330.4 MB read + 43.4 MB written for 13,762,560 cells)
+SMOOTH_DOT_DRAM_BYTES_PER_CELL = (330.384128e6 + 43.357952e6) / (512 * 384 * 70)
 # DRAM bytes per fine cell of one k_resid_restrict<float> launch in its
 # presmoothing form on the finest level (ncu capture at 512x384x70: 232.5 MB
-# read + 13.0 MB written for 13,762,560 fine cells)
-RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.47872e6 + 13.043456e6) / (512 * 384 * 70)
+# read + 15.9 MB written for 13,762,560 fine cells)
+RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.475392e6 + 15.930112e6) / (512 * 384 * 70)
 
 
 def kernel_table(H, L, N):
@@ -428,7 +428,7 @@ def run_ours(args):
 
     peak, peak_kind = load_peaks()
     # the kernel with the largest share of the mixed solve: the V-cycle's last
-    # fine-level sweep with <r, z> fused (reads u, b, tx, ty, m, dq; writes u:
+    # fine-level sweep with <r, z> fused (reads u, b, tx, ty, m, g; writes u:
     # 7 x 4 B per cell)
     sm_bytes = 28 * N
     sm_avg_ms = sm_ms / max(sm_calls, 1)
@@ -622,9 +622,9 @@ def ensemble_measure(steps, warmup):
 # ----------------------------------------------------------------- one kernel
 # --kernel name -> (precision, what runs, algorithmic words per fine cell or None)
 PROBE_KERNELS = {
-    "smooth32": (1, "smooth", 8),
-    "smooth32_dot": (1, "smooth_dot", 8),
-    "smooth32_zero": (1, "smooth0", 5),
+    "smooth32": (1, "smooth", 7),
+    "smooth32_dot": (1, "smooth_dot", 7),
+    "smooth32_zero": (1, "smooth0", 4),
     "resid32": (1, "residual", 7),
     "apply32": (1, "apply", 6),
     "restrict32": (1, "restrict", None),
