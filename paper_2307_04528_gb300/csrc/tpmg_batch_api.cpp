@@ -115,6 +115,7 @@ struct mg_batch {
     // tuned launch shapes
     int smooth_block = kBlock, smooth_grid = 0, cell_grid = 0, vec_grid = 0;
     int sm_count = 0;
+    bool tune64 = false;  // the FP64 sweeps are still to be timed
     // device extras
     CgScalars *sc = nullptr;          // [n]
     int *active = nullptr;            // [n]
@@ -1211,8 +1212,10 @@ extern "C" int mg_batch_setup(int n, const mg_grid *grids, const mg_coeffs *coef
     build_vector_plans<double>(B);
     if ((st = upload_plan<double>(B->p64, s)) != MG_OK) return bail(st);
     if (B->p.mixed && (st = upload_plan<float>(B->p32, s)) != MG_OK) return bail(st);
-    // on the FP32 sweeps, or the FP64 ones where no FP32 solve takes the work lists
-    if (B->p.mixed && std::count(B->own.begin(), B->own.end(), 0)) st = autotune<float>(B, s);
+    // on the FP32 sweeps; where no FP32 solve takes the work lists, on the FP64
+    // ones in the first FP64 solve (the timed sweeps would double such a setup)
+    B->tune64 = B->p.mixed && !std::count(B->own.begin(), B->own.end(), 0);
+    if (B->p.mixed) st = autotune<float>(B, s);
     else st = autotune<double>(B, s);
     if (st != MG_OK) return bail(st);
     if ((st = rebuild_items<double>(B, s)) != MG_OK) return bail(st);
@@ -1269,6 +1272,12 @@ extern "C" int mg_batch_solve(mg_batch *B, const double *const *b, double *const
     std::vector<int> st(n, MG_OK), its, its_in(n, 0);
     std::vector<double> rel;
     if (!mixed) {
+        if (B->tune64) {
+            CHK(autotune<double>(B, s));
+            CHK(rebuild_items<double>(B, s));
+            CU(cudaStreamSynchronize(s));  // the uploads read the work lists' host vectors
+            B->tune64 = false;
+        }
         std::vector<int> want(n, 1);
         CHK(batch_cg<double>(B, want, std::vector<double>(n, tol), B->p.maxit, st, its, rel, s));
         for (int i = 0; i < n; ++i) batch_stats(stats, i, its[i], 0, rel[i]);
