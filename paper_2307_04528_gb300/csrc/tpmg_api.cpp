@@ -326,7 +326,7 @@ static size_t carve(mg_handle *H, void *base)
     H->sc_coarse = cv.take<CgScalars>(1);
     H->bsc = cv.take<BicgScalars>(1);
     H->cg_loop = cv.take<CgLoop>(1);
-    H->flag = cv.take<int>(4);
+    H->flag = cv.take<int>(4 + kMaxLevels);  // validation, then LevelDev::either of each level
     return cv.off + 256;
 }
 
@@ -427,7 +427,7 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
     CU(cudaMemcpyAsync(f.ty, co->ty, bytes0, cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(f.tz, co->tz, bytes0, cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(f.h, co->h, bytes0, cudaMemcpyDeviceToDevice, s));
-    CU(cudaMemsetAsync(H->flag, 0, 4 * sizeof(int), s));
+    CU(cudaMemsetAsync(H->flag, 0, (4 + kMaxLevels) * sizeof(int), s));
     KRUN(K_VEC, 0, 0, launch_validate(dev<double>(f), H->flag, s));
     int flag = 0;
     CU(cudaMemcpyAsync(&flag, H->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -465,10 +465,14 @@ static int setup_impl(mg_handle *H, const mg_coeffs *co, void *ws, size_t ws_byt
                 if (ratio - 1.0 <= H->p.iso_ratio) H->L = l + 2;  // level l+1 is the coarsest
             }
         }
-        KRUN(K_VEC, l, 0, launch_column_lu(dev<double>(v), v.m, v.g, s));
+        KRUN(K_VEC, l, 0, launch_column_lu(dev<double>(v), v.m, v.g, H->flag + 4 + l, s));
         // the uploads above read pageable host vectors: finish before they go away
         CU(cudaStreamSynchronize(s));
     }
+    int either[kMaxLevels];
+    CU(cudaMemcpyAsync(either, H->flag + 4, sizeof either, cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+    for (int l = 0; l < H->L; ++l) H->lev[l].either = either[l] != 0;
     if (H->p.coarse_method == MG_COARSE_CHEBYSHEV) {
         // spectrum of H_z^{-1} H on the coarsest level in [mu, 2]:
         // mu = 1 / max over cells of (h + horizontal couplings) / h

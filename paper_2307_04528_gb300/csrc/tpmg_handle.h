@@ -51,9 +51,11 @@ using tpmg::CgScalars;
 using tpmg::BicgScalars;
 
 // ------------------------------------------------------------------ handle
+constexpr int kMaxLevels = 32;  // nlon halves at most 30 times
 struct LevelHost {
     int nlon = 0, nlat = 0, nz = 0;
     size_t n = 0;
+    bool either = true;  // LevelDev; known after setup
     double *tx = nullptr, *ty = nullptr, *tz = nullptr, *h = nullptr, *m = nullptr, *g = nullptr;
     float *tx32 = nullptr, *ty32 = nullptr, *tz32 = nullptr, *h32 = nullptr, *m32 = nullptr,
           *g32 = nullptr;
@@ -139,12 +141,12 @@ LevelDev<T> dev(const LevelHost &l);
 template <>
 inline LevelDev<double> dev<double>(const LevelHost &l)
 {
-    return {l.nlon, l.nlat, l.nz, l.tx, l.ty, l.tz, l.h, l.m, l.g};
+    return {l.nlon, l.nlat, l.nz, l.tx, l.ty, l.tz, l.h, l.m, l.g, l.either};
 }
 template <>
 inline LevelDev<float> dev<float>(const LevelHost &l)
 {
-    return {l.nlon, l.nlat, l.nz, l.tx32, l.ty32, l.tz32, l.h32, l.m32, l.g32};
+    return {l.nlon, l.nlat, l.nz, l.tx32, l.ty32, l.tz32, l.h32, l.m32, l.g32, l.either};
 }
 template <typename T>
 struct Vec;

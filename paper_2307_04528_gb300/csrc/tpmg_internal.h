@@ -19,6 +19,7 @@ struct LevelDev {
     // above a half, and on top (-q_k / p_k < 0): both f and 1 - f = q / p keep
     // their full relative accuracy in one array (link, carry)
     const T *g;
+    bool either;  // some g below the top may be f itself, not f - 1
 };
 
 // Links from level l to level l+1 (device arrays, sizes in comments).
@@ -184,7 +185,7 @@ int launch_sweep(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out, doub
 // Partial sums launch_smooth_dot writes for these arguments.
 template <typename T>
 int smooth_dot_partials(const LevelDev<T> &L, const T *b, const T *u_in, T *u_out);
-// Shared-memory limits of the segmented sweeps (before any stream capture).
+// Shared-memory limits of the coarsest-level solve (before any stream capture).
 cudaError_t sweep_prepare();
 
 // The coarsest-level solve: `sweeps` sweeps from a zero guess in one launch of
@@ -338,8 +339,10 @@ cudaError_t launch_validate(const LevelDev<double> &L, int *flag, cudaStream_t s
 // Coarse coefficients of level l+1 from level l (sums; lon faces x sx, lat faces x sy[J]).
 cudaError_t launch_coarsen(const LevelDev<double> &F, const LinkDev &K, double sx, double *txc,
                            double *tyc, double *tzc, double *hc, cudaStream_t s);
-// Column factors (m, g) of every column of a level, in FP64.
-cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, cudaStream_t s);
+// Column factors (m, g) of every column of a level, in FP64; *either (device, 0
+// before) becomes 1 where some g below the top is f itself.
+cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, int *either,
+                             cudaStream_t s);
 // FP32 copies: out = (float)(scale * in) for coefficients; m32 = (float)(m / scale);
 // g32 = (float)g.
 cudaError_t launch_to_float(const double *in, float *out, double scale, size_t n, cudaStream_t s);

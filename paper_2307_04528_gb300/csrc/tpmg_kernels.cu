@@ -1088,7 +1088,7 @@ cudaError_t launch_coarsen(const LevelDev<double> &F, const LinkDev &K, double s
 // store m = 1/p and g = t/p, or -q/p where that is the smaller (no closer to zero
 // than FP32's smallest normal value, so that its sign is never lost) and on top (-1).
 __global__ void __launch_bounds__(kBlock)
-k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g)
+k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g, int *either)
 {
     const int nlon = L.nlon, nlat = L.nlat;
     const int ncol = nlon * nlat;
@@ -1098,6 +1098,7 @@ k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g)
     const int iw = (i == 0) ? col + nlon - 1 : col - 1;
     const size_t plane = (size_t)ncol;
     double qp = 0, pp = 1, tdn = 0;
+    bool whole_f = false;
     for (int k = 0; k < L.nz; ++k) {
         const size_t o = (size_t)k * plane;
         double s = L.h[o + col] + L.tx[o + col] + L.tx[o + iw] + L.ty[o + col];
@@ -1106,17 +1107,21 @@ k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g)
         const double tup = L.tz[o + col];
         const double p = q + tup;
         m[o + col] = 1.0 / p;
-        g[o + col] = q < tup || k == L.nz - 1 ? -fmax(q / p, 0x1p-126) : tup / p;
+        const bool less_one = q < tup || k == L.nz - 1;
+        g[o + col] = less_one ? -fmax(q / p, 0x1p-126) : tup / p;
+        whole_f |= !less_one;
         qp = q;
         pp = p;
         tdn = tup;
     }
+    if (whole_f) *either = 1;
 }
 
-cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, cudaStream_t s)
+cudaError_t launch_column_lu(const LevelDev<double> &L, double *m, double *g, int *either,
+                             cudaStream_t s)
 {
     const int ncol = L.nlon * L.nlat;
-    k_column_lu<<<(ncol + kBlock - 1) / kBlock, kBlock, 0, s>>>(L, m, g);
+    k_column_lu<<<(ncol + kBlock - 1) / kBlock, kBlock, 0, s>>>(L, m, g, either);
     return cudaGetLastError();
 }
 

@@ -16,7 +16,7 @@ namespace {
 // more tiles than there are slots for partial sums.  (The loop also has the
 // compiler issue a tile's loads in one run: 0.534 ms against 0.698 without it
 // at 1536 x 1152 x 70, the same instructions otherwise, on q/p alone.)
-template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int MAXT, int MINB,
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int LINK, int MAXT, int MINB,
           typename Level>
 __global__ void __launch_bounds__(MAXT, MINB)
 k_sweep(Level L, const T *b, const T *uin, T *__restrict__ uout, T omega,
@@ -29,14 +29,14 @@ k_sweep(Level L, const T *b, const T *uin, T *__restrict__ uout, T omega,
     T acc = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         if (tile != (int)blockIdx.x) __syncthreads();  // the last tile's maps have been read
-        acc += sweep_tile<T, CV, LZ, QL, GUESS, DOT>(L, b, uin, uout, omega, tile,
-                                                     reinterpret_cast<T *>(smraw));
+        acc += sweep_tile<T, CV, LZ, QL, GUESS, DOT, LINK>(L, b, uin, uout, omega, tile,
+                                                           reinterpret_cast<T *>(smraw));
     }
     if (DOT) block_store<0>((double)acc, partial);
 }
 
 // A Chebyshev step of the coarsest-level solve as one sweep (launch_cheb_sweep).
-template <typename T, int CV, int LZ, int QL, int MAXT, int MINB>
+template <typename T, int CV, int LZ, int QL, int LINK, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
 k_sweep_cheb(LevelDev<T> L, const T *b, const T *uin, T *__restrict__ uout, ChebStep<T> ch)
 {
@@ -45,8 +45,8 @@ k_sweep_cheb(LevelDev<T> L, const T *b, const T *uin, T *__restrict__ uout, Cheb
     const int tiles = (L.nlon * L.nlat + QL * CV - 1) / (QL * CV);
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         if (tile != (int)blockIdx.x) __syncthreads();  // the last tile's maps have been read
-        sweep_tile<T, CV, LZ, QL, true, false, true>(L, b, uin, uout, T(1), tile,
-                                                     reinterpret_cast<T *>(smraw), ch);
+        sweep_tile<T, CV, LZ, QL, true, false, LINK, true>(L, b, uin, uout, T(1), tile,
+                                                           reinterpret_cast<T *>(smraw), ch);
     }
 }
 
@@ -93,10 +93,22 @@ using Mid64 = Shape<1, 9, 8, 192, 1>;
 using NsLarge0 = Shape<2, 9, 32, 256, 2, false>;
 using NsLarge = Shape<4, 5, 16, 256, 2>;
 
-template <typename T, typename S, bool GUESS, bool DOT, typename Level = LevelDev<T>>
+// f(LINK_*) for the form of a level's link factors.
+template <typename Level, typename F>
+auto with_link(const Level &L, F &&f)
+{
+    if constexpr (kDirected<Level>) {
+        return f(std::integral_constant<int, LINK_DIRECTED>{});
+    } else {
+        return L.either ? f(std::integral_constant<int, LINK_EITHER>{})
+                        : f(std::integral_constant<int, LINK_LESS_ONE>{});
+    }
+}
+
+template <typename T, typename S, bool GUESS, bool DOT, int LINK, typename Level = LevelDev<T>>
 constexpr auto kernel_of()
 {
-    return k_sweep<T, S::CV, S::LZ, S::QL, GUESS, DOT, S::MAXT, S::MINB, Level>;
+    return k_sweep<T, S::CV, S::LZ, S::QL, GUESS, DOT, LINK, S::MAXT, S::MINB, Level>;
 }
 
 template <typename S>
@@ -106,7 +118,7 @@ int threads_of(int nz)  // whole warps: a segment past the last owns no layer
 }
 
 template <typename T, typename S, bool DOT, typename Level = LevelDev<T>>
-size_t smem_of(int threads)
+constexpr size_t smem_of(int threads)
 {
     return (size_t)(3 + kDirected<Level> + (DOT ? S::LZ : 0)) * threads * S::CV * sizeof(T);
 }
@@ -136,6 +148,7 @@ int go(const Level &L, const Sweep<T> &a)
     const long long per = S::QL * S::CV;
     const long long tiles = ((long long)L.nlon * L.nlat + per - 1) / per;
     const int grid = (int)std::min<long long>(tiles, kReduceSlots), threads = threads_of<S>(L.nz);
+    static_assert(smem_of<T, S, S::GUESS, Level>(S::MAXT) <= 48 * 1024, "no opt-in is asked for");
     if (a.count) return grid;
     const T *b = a.b, *uin = a.uin;
     T *uout = a.uout;
@@ -143,28 +156,31 @@ int go(const Level &L, const Sweep<T> &a)
     const double omega = a.omega;
     const cudaStream_t s = a.s;
     const int *flag = a.flag;
-    if (!uin)
-        launch_after(kernel_of<T, S, false, false, Level>(), grid, threads,
-                     smem_of<T, S, false, Level>(threads), s, L, b, uin, uout, (T)omega, partial,
-                     flag);
-    if constexpr (S::GUESS && !kDirected<Level>) {
-        if (a.ch) {
-            launch_after(k_sweep_cheb<T, S::CV, S::LZ, S::QL, S::MAXT, S::MINB>, grid, threads,
-                         smem_of<T, S, false>(threads), s, L, b, uin, uout, *a.ch);
-            return grid;
-        }
-    }
-    if constexpr (S::GUESS) {
-        if constexpr (!kDirected<Level>)
-            if (uin && partial)
-                launch_after(kernel_of<T, S, true, true>(), grid, threads,
-                             smem_of<T, S, true>(threads), s, L, b, uin, uout, (T)omega, partial,
-                             flag);
-        if (uin && !partial)
-            launch_after(kernel_of<T, S, true, false, Level>(), grid, threads,
+    with_link(L, [&](auto link) {
+        constexpr int LINK = decltype(link)::value;
+        if (!uin)
+            launch_after(kernel_of<T, S, false, false, LINK, Level>(), grid, threads,
                          smem_of<T, S, false, Level>(threads), s, L, b, uin, uout, (T)omega,
                          partial, flag);
-    }
+        if constexpr (S::GUESS && !kDirected<Level>) {
+            if (a.ch) {
+                launch_after(k_sweep_cheb<T, S::CV, S::LZ, S::QL, LINK, S::MAXT, S::MINB>, grid,
+                             threads, smem_of<T, S, false>(threads), s, L, b, uin, uout, *a.ch);
+                return;
+            }
+        }
+        if constexpr (S::GUESS) {
+            if constexpr (!kDirected<Level>)
+                if (uin && partial)
+                    launch_after(kernel_of<T, S, true, true, LINK>(), grid, threads,
+                                 smem_of<T, S, true>(threads), s, L, b, uin, uout, (T)omega,
+                                 partial, flag);
+            if (uin && !partial)
+                launch_after(kernel_of<T, S, true, false, LINK, Level>(), grid, threads,
+                             smem_of<T, S, false, Level>(threads), s, L, b, uin, uout, (T)omega,
+                             partial, flag);
+        }
+    });
     return grid;
 }
 
@@ -172,15 +188,6 @@ int go(const Level &L, const Sweep<T> &a)
 int waste(int nz, int lz) { return ((nz + lz - 1) / lz * lz - nz) * 100 / nz; }
 
 constexpr int kSmallColumns = 2048, kMidColumns = 8192;
-
-template <typename T, typename S, bool DOT, typename Level = LevelDev<T>>
-cudaError_t allow_smem()
-{
-    const int need = (int)smem_of<T, S, DOT, Level>(S::MAXT);
-    if (need <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute((const void *)kernel_of<T, S, true, DOT, Level>(),
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, need);
-}
 
 constexpr int kClusterBlocks = 8;  // the portable cluster size
 
@@ -190,13 +197,13 @@ constexpr int kClusterThreads = sizeof(T) == 4 && !kDirected<Level> ? 512
                                 : sizeof(T) == 4 || LZ <= 4         ? 384
                                                                     : 256;
 
-template <typename T, int LZ, typename Level>
+template <typename T, int LZ, int LINK, typename Level>
 __global__ void __launch_bounds__(kClusterThreads<T, LZ, Level>, 1)
 k_coarse_cluster(Level L, const T *b, T *__restrict__ out, T omega, int sweeps, int R)
 {
     after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
-    coarse_cluster<T, LZ, Level>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
+    coarse_cluster<T, LZ, LINK, Level>(L, b, out, omega, sweeps, R, reinterpret_cast<T *>(smraw));
 }
 
 // Layers per segment, balancing the dependent steps: about ten operations a
@@ -370,8 +377,11 @@ static cudaError_t coarse_solve(const Level &L, const T *b, T *out, double omega
     cfg.numAttrs = capturing(s) ? 1 : 2;
     const T om = (T)omega;
     auto run = [&](auto lz) {
-        return cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, decltype(lz)::value, Level>, L, b, out,
-                                  om, sweeps, c.R);
+        return with_link(L, [&](auto link) {
+            return cudaLaunchKernelEx(
+                &cfg, k_coarse_cluster<T, decltype(lz)::value, decltype(link)::value, Level>, L, b,
+                out, om, sweeps, c.R);
+        });
     };
     if constexpr (sizeof(T) == 8) {
         if (c.lz == 2) return run(std::integral_constant<int, 2>{});
@@ -407,14 +417,14 @@ int launch_ns_sweep(const NsView<T> &V, const T *b, const T *u_in, T *u_out, dou
     return pick<T>(V, {b, u_in, u_out, omega, nullptr, s, nullptr, false, false});
 }
 
-template <typename T, typename Level>
+template <typename T, typename Level, int... LINK>
 static cudaError_t allow_coarse_smem()
 {
-    const void *k4[] = {(const void *)k_coarse_cluster<T, 4, Level>,
-                        (const void *)k_coarse_cluster<T, 6, Level>,
-                        (const void *)k_coarse_cluster<T, sizeof(T) == 4 ? 8 : 2, Level>,
-                        (const void *)k_coarse_cluster<T, sizeof(T) == 4 ? 12 : 3, Level>};
-    for (const void *k : k4) {
+    constexpr int A = sizeof(T) == 4 ? 8 : 2, B = sizeof(T) == 4 ? 12 : 3;
+    for (const void *k : {(const void *)k_coarse_cluster<T, 4, LINK, Level>...,
+                          (const void *)k_coarse_cluster<T, 6, LINK, Level>...,
+                          (const void *)k_coarse_cluster<T, A, LINK, Level>...,
+                          (const void *)k_coarse_cluster<T, B, LINK, Level>...}) {
         const cudaError_t e =
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
         if (e != cudaSuccess) return e;
@@ -424,13 +434,11 @@ static cudaError_t allow_coarse_smem()
 
 cudaError_t sweep_prepare()
 {
-    for (cudaError_t q : {allow_smem<float, Large, true>(), allow_smem<float, Large5, true>(),
-                          allow_smem<float, Mid, true>(), allow_smem<float, SmallTall, true>(),
-                          allow_smem<double, Mid64, true>(), allow_smem<double, SmallTall, true>(),
-                          allow_coarse_smem<float, LevelDev<float>>(),
-                          allow_coarse_smem<double, LevelDev<double>>(),
-                          allow_coarse_smem<float, NsView<float>>(),
-                          allow_coarse_smem<double, NsView<double>>()})
+    for (cudaError_t q :
+         {allow_coarse_smem<float, LevelDev<float>, LINK_EITHER, LINK_LESS_ONE>(),
+          allow_coarse_smem<double, LevelDev<double>, LINK_EITHER, LINK_LESS_ONE>(),
+          allow_coarse_smem<float, NsView<float>, LINK_DIRECTED>(),
+          allow_coarse_smem<double, NsView<double>, LINK_DIRECTED>()})
         if (q != cudaSuccess) return q;
     return cudaSuccess;
 }

@@ -26,8 +26,6 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
-#include <type_traits>
-
 #include "tpmg_device.cuh"
 #include "tpmg_internal.h"
 
@@ -231,15 +229,16 @@ __device__ __forceinline__ Vals<T, CV> lds_v(const T *p)
 }
 
 // How the link factors f, kept as g (LevelDev), are taken:
+//   LINK_LESS_ONE  every g of the level is f - 1: f w = g w + w.  The coarse levels of a
+//                  lat-lon grid, bound by latency: a cluster solve of 8 x 6 x 70 19.6 us
+//                  instead of 21.7, the FP32 V-cycle of 88 x 60 x 70 58.8 instead of 60.3
 //   LINK_EITHER    w counts where g is f - 1: in FP64 by a select, in FP32 by a factor
-//                  of one or zero
-//   LINK_LESS_ONE  every g of the warp is f - 1 (a vote): f w = g w + w.  The coarsest-
-//                  level solve in FP64, whose sweeps share one vote
+//                  of one or zero.  The finest levels, at whose poles the horizontal
+//                  couplings outweigh the vertical ones (1 to 4 % of the warps; a vote
+//                  of the warp for the short form undid the order of the loads: with
+//                  <b, u_out> at 512 x 384 x 70 in FP32 84 -> 150 us)
 //   LINK_DIRECTED  g = -q/p, with f = d m (the coupling down of the row above times
 //                  1/p) beside it
-// A vote in the sweeps of sweep_tile lets all warps but the 1 to 4 % at the poles of a
-// lat-lon grid take the short form, but its branches undid the order of the loads
-// (with <b, u_out> at 512 x 384 x 70 in FP32: 84 -> 150 us).
 enum { LINK_LESS_ONE, LINK_EITHER, LINK_DIRECTED };
 
 // One where g is f - 1, else zero: a saturated product, which issues on the FMA pipe
@@ -301,36 +300,6 @@ __device__ __forceinline__ Vals<T, CV> back(const Vals<T, CV> &g, const Vals<T, 
     }
 }
 
-// Whether some lane of the warp holds a g that is not f - 1 (FP64).
-template <bool NS, typename T, int CV, int LZ>
-__device__ __forceinline__ bool any_either(const Vals<T, CV> (&g)[LZ])
-{
-    if constexpr (NS || sizeof(T) == 4) {
-        return true;
-    } else {
-        int sign = -1;
-#pragma unroll
-        for (int c = 0; c < LZ; ++c)
-#pragma unroll
-            for (int i = 0; i < CV; ++i) sign &= sign_word(g[c].a[i]);
-        return __any_sync(0xffffffffu, sign >= 0);
-    }
-}
-
-// run(the warp's LINK_*).
-template <typename T, bool NS, typename F>
-__device__ __forceinline__ void with_links(bool either, F &&run)
-{
-    if constexpr (NS) {
-        run(std::integral_constant<int, LINK_DIRECTED>{});
-    } else if constexpr (sizeof(T) == 4) {
-        run(std::integral_constant<int, LINK_EITHER>{});
-    } else {
-        if (either) run(std::integral_constant<int, LINK_EITHER>{});
-        else run(std::integral_constant<int, LINK_LESS_ONE>{});
-    }
-}
-
 // A Chebyshev step instead of a sweep: with b the residual and u_in the step d,
 // r_out = b - H d, x += d (first: x = d) and u_out = c1 d + c2 H_z^{-1} r_out;
 // last: x takes the new step too.  Each cell of x is its own thread's.
@@ -345,7 +314,7 @@ struct ChebStep {
 // b waiting for the last pass in the thread's own slots of shared memory.
 // Byte offsets are 32-bit (pick).  sh: 3 blockDim CV values (4 in a directed
 // level), and LZ blockDim CV more for DOT.
-template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, bool CHEB = false,
+template <typename T, int CV, int LZ, int QL, bool GUESS, bool DOT, int LINK, bool CHEB = false,
           typename Level>
 __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin,
                                         T *__restrict__ uout, T omega, int tile, T *sh,
@@ -354,7 +323,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
     using X = Vals<T, CV>;
     constexpr unsigned SZ = sizeof(T);
     constexpr bool NS = kDirected<Level>;
-    constexpr int LINK = NS ? LINK_DIRECTED : LINK_EITHER;
+    static_assert(NS == (LINK == LINK_DIRECTED), "a level's own link form");
     static_assert(!(NS && DOT), "no <b, u_out> of a directed level");
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat;
@@ -545,7 +514,7 @@ __device__ __forceinline__ T sweep_tile(const Level &L, const T *b, const T *uin
 // neighbours' shared memory, and one cluster barrier separates the sweeps.
 // The forward and backward maps of the segments are exchanged as in
 // sweep_tile, their factors once.  sh: 2 R nlon nz + 4 blockDim values.
-template <typename T, int LZ, typename Level>
+template <typename T, int LZ, int LINK, typename Level>
 __device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
                                                T *__restrict__ out, T omega, int sweeps, int R,
                                                T *sh)
@@ -589,16 +558,12 @@ __device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
         if constexpr (NS) f[c].a[0] = __ldg(down_of(L) + o) * m[c];
     }
     const X zero = {{T(0)}};
-    const bool either = any_either<NS>(g);
     X A = {{T(1)}}, B = A;
-    with_links<T, NS>(either, [&](auto link) {
-        constexpr int LINK = decltype(link)::value;
 #pragma unroll
-        for (int c = 0; c < LZ; ++c) {
-            A = carry<LINK, T, 1>(g[c], f[NS ? c : 0], zero, A, A);
-            if (NS) B = vfma<T, 1>(g[c], B, B);
-        }
-    });
+    for (int c = 0; c < LZ; ++c) {
+        A = carry<LINK, T, 1>(g[c], f[NS ? c : 0], zero, A, A);
+        if (NS) B = vfma<T, 1>(g[c], B, B);
+    }
     sA[threadIdx.x] = A.a[0];
     if (NS) sB[threadIdx.x] = B.a[0];
     const T om1 = T(1) - omega;
@@ -618,40 +583,31 @@ __device__ __forceinline__ void coarse_cluster(const Level &L, const T *b,
             }
             v[c].a[0] = x;
         }
-        with_links<T, NS>(either, [&](auto link) {
-            constexpr int LINK = decltype(link)::value;
 #pragma unroll
-            for (int c = 0; c < LZ; ++c)
-                C = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], C, vadd<T, 1>(v[c], C));
-        });
+        for (int c = 0; c < LZ; ++c)
+            C = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], C, vadd<T, 1>(v[c], C));
         sC[threadIdx.x] = C.a[0];
         __syncthreads();
         X h = zero;
 #pragma unroll 4
         for (int s = 0; s < seg; ++s) h.a[0] = fma(sA[s * cols + lc], h.a[0], sC[s * cols + lc]);
         X F = zero;
-        with_links<T, NS>(either, [&](auto link) {
-            constexpr int LINK = decltype(link)::value;
 #pragma unroll
-            for (int c = 0; c < LZ; ++c) {
-                const X w = vadd<T, 1>(v[c], h);
-                h = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], h, w);
-                v[c].a[0] = w.a[0] * m[c];
-            }
+        for (int c = 0; c < LZ; ++c) {
+            const X w = vadd<T, 1>(v[c], h);
+            h = carry<LINK, T, 1>(g[c], f[NS ? c : 0], v[c], h, w);
+            v[c].a[0] = w.a[0] * m[c];
+        }
 #pragma unroll
-            for (int c = LZ - 1; c >= 0; --c) F = back<LINK, T, 1>(g[c], F, v[c]);
-        });
+        for (int c = LZ - 1; c >= 0; --c) F = back<LINK, T, 1>(g[c], F, v[c]);
         sF[threadIdx.x] = F.a[0];
         __syncthreads();
         X x = zero;
 #pragma unroll 4
         for (int s = nseg - 1; s > seg; --s)
             x.a[0] = fma(sB[s * cols + lc], x.a[0], sF[s * cols + lc]);
-        with_links<T, NS>(either, [&](auto link) {
-            constexpr int LINK = decltype(link)::value;
 #pragma unroll
-            for (int c = LZ - 1; c >= 0; --c) v[c] = x = back<LINK, T, 1>(g[c], x, v[c]);
-        });
+        for (int c = LZ - 1; c >= 0; --c) v[c] = x = back<LINK, T, 1>(g[c], x, v[c]);
 #pragma unroll
         for (int c = LZ - 1; c >= 0; --c) {
             uc[c] = fma(om1, uc[c], omega * v[c].a[0]);

@@ -30,7 +30,8 @@ def contrast(nlon, nlat, nz, factor, coupling):
 
 SHAPES = [(30, 10, 16), (6, 4, 100), (64, 34, 70), (132, 64, 70), (128, 66, 37), (130, 64, 70),
           (129, 66, 12)]
-SYSTEMS = [(1e4, 0.1), (1e4, 10.0), (1e-4, 0.1)]
+# the last: the vertical coupling is the larger part of every pivot below the top
+SYSTEMS = [(1e4, 0.1), (1e4, 10.0), (1e-4, 0.1), (1.0, 10.0)]
 
 
 @pytest.mark.parametrize("factor,coupling", SYSTEMS)
