@@ -184,6 +184,8 @@ static int check_grid(const mg_grid *g, const mg_params *p, int *L_out)
         return fail(MG_ERR_ARG, "nlat=%d must be even and >= 2", g->nlat);
     if (g->nlon < 4) return fail(MG_ERR_ARG, "nlon=%d must be >= 4", g->nlon);
     const int L = p->levels > 0 ? p->levels : auto_levels(g->nlon);
+    if (L > 30)  // an int halves at most 30 times
+        return fail(MG_ERR_ARG, "%d levels are more than any nlon has", L);
     if (L > 1 && (g->nlon % (1 << (L - 1)) || (g->nlon >> (L - 1)) < 2))
         return fail(MG_ERR_ARG, "nlon=%d not divisible by 2^(levels-1) = %d", g->nlon,
                     1 << (L - 1));
