@@ -1108,7 +1108,8 @@ k_column_lu(LevelDev<double> L, double *__restrict__ m, double *__restrict__ g, 
         const double p = q + tup;
         m[o + col] = 1.0 / p;
         const bool less_one = q < tup || k == L.nz - 1;
-        g[o + col] = less_one ? -fmax(q / p, 0x1p-126) : tup / p;
+        const double d = q / p;
+        g[o + col] = less_one ? -(d < 0x1p-126 ? 0x1p-126 : d) : tup / p;  // a NaN stays one
         whole_f |= !less_one;
         qp = q;
         pp = p;
