@@ -341,11 +341,13 @@ __device__ __forceinline__ T dir_apply_column(const LevelDev<T> &L, const T *__r
     return acc;
 }
 
-// One cell of the stencil (cell-parallel form).
+// One cell of the stencil (cell-parallel form).  FP64, launched early, reads b and x
+// by ordinary loads (after_previous); FP32 keeps the read-only path, which lets the
+// compiler issue all loads ahead of the branches at the poles (176 x 148 x 30: 4.8 us
+// against 6.7), and an ordinary launch.
 template <typename T, int MODE>
-__device__ __forceinline__ void stencil_cell(const LevelDev<T> &L, const T *__restrict__ b,
-                                             const T *__restrict__ x, T *__restrict__ y, int col,
-                                             int k)
+__device__ __forceinline__ void stencil_cell(const LevelDev<T> &L, const T *b, const T *x,
+                                             T *__restrict__ y, int col, int k)
 {
     const int nlon = L.nlon, nlat = L.nlat, nz = L.nz;
     const int ncol = nlon * nlat;
@@ -355,15 +357,16 @@ __device__ __forceinline__ void stencil_cell(const LevelDev<T> &L, const T *__re
     const int iw = (i == 0) ? col + nlon - 1 : col - 1;
     const size_t plane = (size_t)ncol;
     const size_t o = (size_t)k * plane;
-    const T xc = __ldg(x + o + col);
+    auto of = [](const T *p) { return sizeof(T) == 8 ? *p : __ldg(p); };
+    const T xc = of(x + o + col);
     T v = __ldg(L.h + o + col) * xc;
-    v = fma(__ldg(L.tx + o + col), xc - __ldg(x + o + ie), v);
-    v = fma(__ldg(L.tx + o + iw), xc - __ldg(x + o + iw), v);
-    if (j + 1 < nlat) v = fma(__ldg(L.ty + o + col), xc - __ldg(x + o + col + nlon), v);
-    if (j > 0) v = fma(__ldg(L.ty + o + col - nlon), xc - __ldg(x + o + col - nlon), v);
-    if (k + 1 < nz) v = fma(__ldg(L.tz + o + col), xc - __ldg(x + o + plane + col), v);
-    if (k > 0) v = fma(__ldg(L.tz + o - plane + col), xc - __ldg(x + o - plane + col), v);
-    y[o + col] = MODE ? __ldg(b + o + col) - v : v;
+    v = fma(__ldg(L.tx + o + col), xc - of(x + o + ie), v);
+    v = fma(__ldg(L.tx + o + iw), xc - of(x + o + iw), v);
+    if (j + 1 < nlat) v = fma(__ldg(L.ty + o + col), xc - of(x + o + col + nlon), v);
+    if (j > 0) v = fma(__ldg(L.ty + o + col - nlon), xc - of(x + o + col - nlon), v);
+    if (k + 1 < nz) v = fma(__ldg(L.tz + o + col), xc - of(x + o + plane + col), v);
+    if (k > 0) v = fma(__ldg(L.tz + o - plane + col), xc - of(x + o - plane + col), v);
+    y[o + col] = MODE ? of(b + o + col) - v : v;
 }
 
 // ------------------------------------------------------------------ smoother

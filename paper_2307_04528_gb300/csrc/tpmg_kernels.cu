@@ -147,9 +147,9 @@ int launch_residual_cast(const LevelDev<double> &L, const double *b, const doubl
 // for levels with too few columns to fill the GPU with column loops.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kBlock)
-k_stencil_cells(LevelDev<T> L, const T *__restrict__ b, const T *__restrict__ x, T *__restrict__ y,
-                const int *__restrict__ flag)
+k_stencil_cells(LevelDev<T> L, const T *b, const T *x, T *__restrict__ y, const int *flag)
 {
+    if (sizeof(T) == 8) after_previous();
     if (flag && !*flag) return;
     stencil_cell<T, MODE>(L, b, x, y, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
 }
@@ -159,9 +159,11 @@ constexpr int kCellParallelColumns = 32768;
 // Below this many cells the threads of 2 x 2 columns leave FP64 pipes idle: without an
 // inner product a thread takes a cell.  FP64 apply by cells and by quads: 64 x 32 x 16
 // 2.5 and 9.1 us, 48 x 82 x 70 8.5 and 11.6, 96 x 80 x 33 7.9 and 11.4, 256 x 192 x 3
-// 5.3 and 6.9; from 128 x 64 x 70 (15.2 and 16.1; launched directly 17.4 and 16.7) to
-// 256 x 126 x 20 (17.0 and 16.2; 19.1 and 16.7) the quads' early launch decides.
+// 5.3 and 6.9, 256 x 126 x 20 17.0 and 16.2.  Below kQuadColumns, whose blocks the
+// layers' split only multiplies, the line is twice as high (128 x 64 x 70 15.2 and
+// 16.1, 64 x 98 x 100 16.5 and 20.4, 90 x 88 x 150 29.6 and 30.6).
 constexpr long long kQuadCells = 1LL << 19;
+constexpr int kQuadColumns = 16384;
 
 template <typename T>
 int launch_stencil(const LevelDev<T> &L, int mode, const T *b, const T *x, T *y, double *partial,
@@ -169,15 +171,17 @@ int launch_stencil(const LevelDev<T> &L, int mode, const T *b, const T *x, T *y,
 {
     const int ncol = L.nlon * L.nlat;
     const int grid = (ncol + kBlock - 1) / kBlock;
-    const bool few = sizeof(T) == 8 && !partial && (long long)ncol * L.nz < kQuadCells;
+    const bool few = sizeof(T) == 8 && !partial &&
+                     (long long)ncol * L.nz < (ncol < kQuadColumns ? 2 : 1) * kQuadCells;
     if constexpr (sizeof(T) == 8) {
         const int blocks = few ? -1 : launch_stencil_quad(L, mode, b, x, y, partial, s, flag);
         if (blocks >= 0) return partial ? blocks : 0;
     }
     if (!partial && (few || ncol < kCellParallelColumns)) {
         const dim3 g2(grid, L.nz);
-        if (mode) k_stencil_cells<T, 1><<<g2, kBlock, 0, s>>>(L, b, x, y, flag);
-        else k_stencil_cells<T, 0><<<g2, kBlock, 0, s>>>(L, b, x, y, flag);
+        const auto kernel = mode ? k_stencil_cells<T, 1> : k_stencil_cells<T, 0>;
+        if constexpr (sizeof(T) == 8) launch_after(kernel, g2, kBlock, 0, s, L, b, x, y, flag);
+        else kernel<<<g2, kBlock, 0, s>>>(L, b, x, y, flag);
         return 0;
     }
     if (partial) {
