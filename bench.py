@@ -235,12 +235,12 @@ KERNEL_WORDS = {
 
 
 # DRAM bytes per fine cell of one launch of the FP32 sweep with <r, z> (ncu
-# capture at 512x384x70: 330.4 MB read + 43.4 MB written for 13,762,560 cells)
-SMOOTH_DOT_DRAM_BYTES_PER_CELL = (330.384128e6 + 43.357952e6) / (512 * 384 * 70)
+# capture at 512x384x70: 330.3 MB read + 43.4 MB written for 13,762,560 cells)
+SMOOTH_DOT_DRAM_BYTES_PER_CELL = (330.345984e6 + 43.403008e6) / (512 * 384 * 70)
 # DRAM bytes per fine cell of one k_resid_restrict<float> launch in its
-# presmoothing form on the finest level (ncu capture at 512x384x70: 232.5 MB
-# read + 15.9 MB written for 13,762,560 fine cells)
-RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.475392e6 + 15.930112e6) / (512 * 384 * 70)
+# presmoothing form on the finest level (ncu capture at 512x384x70: 232.6 MB
+# read + 15.6 MB written for 13,762,560 fine cells)
+RESID_RESTRICT_PRE_DRAM_BYTES_PER_CELL = (232.555264e6 + 15.615744e6) / (512 * 384 * 70)
 
 
 def kernel_table(H, L, N):
